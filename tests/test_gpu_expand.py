@@ -199,3 +199,33 @@ def test_expand_capacity_insert_and_edge_cases(torch_cuda):
     out6, _, k6 = _run_expand(torch, rgb, one, cam, pose, u1, u_angle, 0.5, 0, max_scale=0.07)
     assert k6 == 1
     np.testing.assert_allclose(to_np(out6.scale[:1]), 0.07)   # no neighbour in P_s
+
+
+@pytest.mark.parametrize("w,h,ratio,f,cx,outliers", [
+    (61, 47, 1.0, 60.0, 30.5, 0.0),          # every pixel a point
+    (333, 251, 0.3, 300.0, 166.5, 0.01),     # depth outliers: neighbours far from the pixel
+    (333, 251, 0.003, 300.0, 400.0, 0.05),   # sparse points, principal point off the image
+    (333, 251, 0.04, 90.0, 166.5, 0.0),      # wide field of view
+    (2100, 2003, 0.01, 1500.0, 1050.0, 0.0)  # more pixel blocks than sum their counts themselves
+])
+def test_expand_nearest_is_the_minimum(torch_cuda, w, h, ratio, f, cx, outliers):
+    """The windowed neighbour search against the k-d tree over all of P_s;
+    the bound is the rounding of two FP32 points (8 operations each, at the
+    scale of the camera-space point plus the translation)."""
+    torch = torch_cuda
+    cam = scenes.Camera(f, f, cx, h / 2, w, h)
+    rgb, depth = scenes.rgbd_frame(w + h, cam)
+    rng = np.random.default_rng(w)
+    depth = np.where(rng.uniform(size=depth.shape) < outliers, 6.0 * depth, depth).astype(np.float32)
+    u_keep = rng.uniform(size=(h, w)).astype(np.float32)
+    u_angle = rng.uniform(size=(h, w)).astype(np.float32)
+    pose = scenes.perturb_pose(scenes.identity_pose(), 0.3, 20.0, seed=w)
+    R = pose.R.astype(np.float32).astype(np.float64)
+    t = pose.t.astype(np.float32).astype(np.float64)
+    o = ex.expand(rgb, depth, cam, R, t, u_keep, u_angle, ratio, 0)
+    out, _, k = _run_expand(torch, rgb, depth, cam, pose, u_keep, u_angle, ratio, 0)
+    assert k == len(o["pixel"])
+    size = np.linalg.norm(o["mu"] @ R.T + t, axis=1) + np.abs(t).sum()
+    tol = 32 * 2.0 ** -24 * size + 1e-6 * o["scale"][:, 0]
+    err = np.abs(to_np(out.scale[:k])[:, 0] - o["scale"][:, 0])
+    assert np.all(err <= tol), (err / tol).max()
