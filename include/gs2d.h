@@ -231,13 +231,15 @@ int gs2d_render_count(const float* proj, const gs2d_bins* bins, const gs2d_camer
 /* Scheduling of the one-pixel-per-thread tile kernels of gs2d_render_fwd and
  * gs2d_track_step (no counterpart in the paper; results do not depend on
  * it): a tile grid of at most max_tiles tiles runs the grouped form of the
- * compositing loops, which keeps four (pixel, surfel) evaluations in flight
- * per thread at two blocks per SM -- for images too small to fill the GPU
- * (160x120 has 80 tiles of 16x16), where each pixel's serial walk over its
- * tile's list is the bound.  -1 (the default) = twice the device's SM count;
- * 0 = never.  Process-wide; read at each launch (so a captured graph keeps
- * the form it was captured with).  Not thread-safe against concurrent
- * launches from other host threads. */
+ * compositing, in which four blocks share a tile (one per 8 x 8 quadrant of
+ * it) and four lanes a pixel -- for images too small to fill the GPU (160x120
+ * has 80 tiles of 16x16) and for tiles whose lists are long against the
+ * rest, where each pixel's serial walk over its tile's list is the bound.
+ * -1 (the default): gs2d_render_fwd takes that form for at most twice the
+ * device's SM count of tiles, gs2d_track_step decides tile by tile from the
+ * list lengths; 0 = never.  Process-wide; read at each launch (so a captured
+ * graph keeps the form it was captured with).  Not thread-safe against
+ * concurrent launches from other host threads. */
 void gs2d_set_grouped_tiles(int max_tiles);
 
 /* Backward of gs2d_render_fwd (Sec. III-B): replays compositing back to

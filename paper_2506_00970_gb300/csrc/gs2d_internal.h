@@ -104,6 +104,10 @@ struct TrackStep {
   unsigned long long* seg_keys;
   unsigned long long* seg_tmp;
   int n;  // surfels (ids are clamped below it)
+  // tiles run on quadrants: partials [n_tiles * 8 * 7] of their 8 x 4 pixel
+  // blocks, and quadrants finished [n_tiles] (zero between iterations)
+  float* quad_part;
+  uint32_t* quad_done;
 };
 
 // Fused tracking iteration per tile (forward, tracking loss, pose backward)

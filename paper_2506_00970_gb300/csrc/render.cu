@@ -42,25 +42,21 @@
 #include "gs2d_common.cuh"
 #include "gs2d_internal.h"
 #include "loss_pixel.cuh"
+#include "quad.cuh"
 #include "tile_loops.cuh"
 #include "tile_sort.cuh"
 #include "track_update.cuh"
 
 namespace gs2d {
 
-// Blocks per SM of the tile kernels: with P pixels per thread, and for the
-// grouped one-pixel loops (kG > 1: kG evaluations in flight per thread,
-// meant for grids too small to fill the GPU, where registers are plentiful
-// and the per-pixel walk's latency is the bound).
-constexpr int kGroup = 4;  // evaluations in flight of the grouped loops
-
-template <int P, int kG>
+// Blocks per SM of the tile kernels with P pixels per thread.
+template <int P>
 constexpr int tile_blocks_per_sm() {
-  return kG > 1 ? 2 : (P == 1 ? 4 : (P == 2 ? 3 : 2));
+  return P == 1 ? 4 : (P == 2 ? 3 : 2);
 }
 
-template <bool kCount, int P, int kG = 1>
-__global__ void __launch_bounds__(kTileThreads, tile_blocks_per_sm<P, kG>()) render_fwd_kernel(
+template <bool kCount, int P>
+__global__ void __launch_bounds__(kTileThreads, tile_blocks_per_sm<P>()) render_fwd_kernel(
     const float4* __restrict__ proj, const uint32_t* __restrict__ vals,
     const int32_t* __restrict__ ranges, gs2d_camera cam, gs2d_config cfg, int tiles_x,
     float* __restrict__ out_rgb, float* __restrict__ out_depth, float* __restrict__ out_normal,
@@ -79,7 +75,7 @@ __global__ void __launch_bounds__(kTileThreads, tile_blocks_per_sm<P, kG>()) ren
   const float yt = (float)tile_y0 + 0.5f - cam.cy;
   uint32_t cnt[5] = {0u, 0u, 0u, 0u, 0u};
   FwdState st[P];
-  fwd_tile<kFwdVec4, kCount, P, kG>(proj, vals + ranges[2 * tile], ranges[2 * tile], ranges[2 * tile + 1], xt, yt,
+  fwd_tile<kFwdVec4, kCount, P>(proj, vals + ranges[2 * tile], ranges[2 * tile], ranges[2 * tile + 1], xt, yt,
                                     tile_x0, tile_y0, tp, inside, cam, cfg, s_rec, hl, cnt, st);
   if (kCount) {
 #pragma unroll
@@ -105,6 +101,84 @@ __global__ void __launch_bounds__(kTileThreads, tile_blocks_per_sm<P, kG>()) ren
     out_opac[p] = 1.f - st[k].T;
     out_T[p] = st[k].T;
     out_nlast[p] = st[k].last;
+  }
+}
+
+// The forward pass on 8 x 8 quadrants (quad.cuh), four blocks per tile: the
+// tile's sorted list in batches of 256 positions, the entries that touch the
+// quadrant staged in order.
+__global__ void __launch_bounds__(kTileThreads, 4) render_fwd_quad_kernel(
+    const float4* __restrict__ proj, const uint32_t* __restrict__ vals,
+    const int32_t* __restrict__ ranges, gs2d_camera cam, gs2d_config cfg, int tiles_x,
+    float* __restrict__ out_rgb, float* __restrict__ out_depth, float* __restrict__ out_normal,
+    float* __restrict__ out_opac, float* __restrict__ out_T, uint32_t* __restrict__ out_nlast,
+    const int32_t* __restrict__ gate) {
+  __shared__ QuadStage<kFwdVec4> s;
+  __shared__ uint8_t s_pos[kQuadBatch];       // list position within the batch of a staged entry
+  __shared__ int s_cnt[2][kTileThreads / 32];
+  if (gate && *gate) return;
+  const int tile = blockIdx.x / kQuads, q = blockIdx.x % kQuads;
+  const int tile_x0 = (tile % tiles_x) * cfg.tile_w, tile_y0 = (tile / tiles_x) * cfg.tile_h;
+  const QuadPix tp = quad_pixel(q, tile_x0, tile_y0, cfg.tile_w);
+  const bool inside = tp.px < cam.width && tp.py < cam.height;
+  const float xt = (float)tile_x0 + 0.5f - cam.cx;
+  const float yt = (float)tile_y0 + 0.5f - cam.cy;
+  const int start = ranges[2 * tile], end = ranges[2 * tile + 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  QuadFwd st = quad_fwd_init(inside);
+  // the next batch's ids are in flight while this one is blended
+  int idx = start + (int)threadIdx.x;
+  uint32_t id = idx < end ? vals[idx] : 0u;
+  for (int b = start, turn = 0; b < end; b += kQuadBatch, turn ^= 1) {
+    uint32_t m = 0u;
+    if (idx < end) {
+      const float4 r7 = proj[(size_t)id * (kProjFloats / 4) + 7];
+      m = quad_mask(r7.z, r7.w, tp.x0, tp.y0);
+    }
+    const uint32_t bal = __ballot_sync(0xffffffffu, m != 0u);
+    if (lane == 0) s_cnt[turn][warp] = __popc(bal);
+    // also: the previous batch is no longer read
+    if (__syncthreads_count(!st.done) == 0) break;
+    int at = __popc(bal & ((1u << lane) - 1u)), n = 0;
+#pragma unroll
+    for (int w = 0; w < kTileThreads / 32; ++w) {
+      const int c = s_cnt[turn][w];
+      if (w < warp) at += c;
+      n += c;
+    }
+    if (m) {
+      stage_record_to<kFwdVec4>(proj, id, xt, yt, s.rec[at]);
+      s.mask[at] = (uint8_t)m;
+      s_pos[at] = (uint8_t)threadIdx.x;
+    }
+    idx += kQuadBatch;
+    id = idx < end ? vals[idx] : 0u;
+    __syncthreads();
+    const int nh = quad_hits(s, n);
+    quad_blend(s, nh, tp, cam, cfg, st,
+               [&](int j) { return (uint32_t)(b - start + s_pos[j] + 1); });
+  }
+  if (!inside) return;
+  const size_t p = (size_t)tp.py * cam.width + tp.px;
+  switch (lane & 3) {   // each lane its components of the pixel
+    case 0:
+      out_rgb[3 * p] = st.a0;
+      out_rgb[3 * p + 1] = st.a1;
+      out_opac[p] = 1.f - st.T;
+      break;
+    case 1:
+      out_rgb[3 * p + 2] = st.a0;
+      out_depth[p] = st.a1;
+      out_T[p] = st.T;
+      break;
+    case 2:
+      out_normal[3 * p] = st.a0;
+      out_normal[3 * p + 1] = st.a1;
+      out_nlast[p] = st.last;
+      break;
+    default:
+      out_normal[3 * p + 2] = st.a0;
+      break;
   }
 }
 
@@ -192,6 +266,51 @@ __global__ void __launch_bounds__(kBwdWarps * 32, kBwdWarpBlocks) render_bwd_war
                          sm[warp]);
 }
 
+// Shared memory of a fused tracking block that runs a whole tile.
+struct TrackSmem {
+  BwdSmem b;
+  HitLists hl;
+  float pose[kTileThreads / 32][6];
+  float loss[kTileThreads / 32];
+  uint32_t ids[kSegSmem];
+};
+
+// Ranks of n (distinct) keys of shared memory by counting, several keys per
+// thread (at most kRankPer): two barriers instead of a bitonic network's
+// stages; ids[rank] = the key's id, clamped below n_ids.  a has room for one
+// key more.
+constexpr int kRankPer = 3;
+__device__ __forceinline__ void rank_ids(unsigned long long* a, int n, uint32_t* ids, int n_ids) {
+  unsigned long long k[kRankPer];
+  int r[kRankPer];
+#pragma unroll
+  for (int c = 0; c < kRankPer; ++c) {
+    const int i = (int)threadIdx.x + c * kTileThreads;
+    k[c] = i < n ? a[i] : 0ull;
+    r[c] = 0;
+  }
+  if (threadIdx.x == 0) a[n] = ~0ull;   // pairs of keys are read
+  __syncthreads();
+  if (n <= kTileThreads) {
+    if ((int)threadIdx.x < n)
+      for (int j = 0; j < n; j += 2) {
+        const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(a + j);
+        r[0] += (int)(kk.x < k[0]) + (int)(kk.y < k[0]);
+      }
+  } else {
+    for (int j = 0; j < n; j += 2) {
+      const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(a + j);
+#pragma unroll
+      for (int c = 0; c < kRankPer; ++c) r[c] += (int)(kk.x < k[c]) + (int)(kk.y < k[c]);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < kRankPer; ++c)
+    if ((int)threadIdx.x + c * kTileThreads < n)
+      ids[r[c]] = min((uint32_t)(k[c] & 0xFFFFFFFFull), (uint32_t)(n_ids - 1));
+  __syncthreads();
+}
+
 // Fused tracking iteration on one tile: the depth sort of the tile's
 // segment, forward compositing, the tracking loss and its image gradient per
 // pixel (in registers), and the pose-only backward replay -- the images never
@@ -200,30 +319,17 @@ __global__ void __launch_bounds__(kBwdWarps * 32, kBwdWarpBlocks) render_bwd_war
 // sorted in shared memory and its ids stay there; a longer one is sorted in
 // chunks merged in global memory and its ids written to vals, which this
 // block then reads back (coherent loads: vals is written in this launch).
-template <int P, int kG = 1>
-__global__ void __launch_bounds__(kTileThreads, tile_blocks_per_sm<P, kG>()) track_tile_kernel(
-    const float4* __restrict__ proj, uint32_t* vals,
-    const int32_t* __restrict__ ranges, gs2d_camera cam, gs2d_config cfg, int tiles_x,
-    const float* __restrict__ obs_rgb, const float* __restrict__ obs_depth, gs2d_track_params prm,
-    float* __restrict__ loss_part, float* __restrict__ pose_part, TrackStep ts,
-    int32_t* __restrict__ status) {
-  __shared__ BwdSmem sm;
-  __shared__ HitLists hl;
-  __shared__ float s_pose[kTileThreads / 32][6];
-  __shared__ float s_loss[kTileThreads / 32];
-  __shared__ bool s_last;
-  __shared__ uint32_t s_ids[kSegSmem];
-  {
-    const int32_t g = *status;
-    if (g != 0) {
-      if (g == kConverged && blockIdx.x == 0 && threadIdx.x == 0)
-        record_converged(ts.pose, ts.loss_hist, ts.pose_hist, ts.grad_hist, ts.iter);
-      return;
-    }
-  }
-  // longest lists first: the blocks of the heaviest tiles start in the first
-  // wave instead of trailing the grid (partials stay indexed by tile)
-  const int tile = ts.order ? ts.order[blockIdx.x] : (int)blockIdx.x;
+// The block's per-warp sums end up in s.pose and s.loss (not yet visible to
+// the other warps).
+template <int P>
+__device__ __forceinline__ void track_tile(
+    int tile, const float4* __restrict__ proj, uint32_t* vals, const int32_t* __restrict__ ranges,
+    const gs2d_camera& cam, const gs2d_config& cfg, int tiles_x,
+    const float* __restrict__ obs_rgb, const float* __restrict__ obs_depth,
+    const gs2d_track_params& prm, const TrackStep& ts, TrackSmem& s) {
+  BwdSmem& sm = s.b;
+  HitLists& hl = s.hl;
+  uint32_t* s_ids = s.ids;
   const TilePix<P> tp = tile_pixel<P>(tile, tiles_x, cfg.tile_w, cfg.tile_h);
   bool inside[P];
 #pragma unroll
@@ -241,21 +347,8 @@ __global__ void __launch_bounds__(kTileThreads, tile_blocks_per_sm<P, kG>()) tra
     unsigned long long* keys = reinterpret_cast<unsigned long long*>(&sm.rec[0][0]);
     static_assert(sizeof(sm.rec) >= kSegSmem * sizeof(unsigned long long), "sort area");
     if (len <= kTileThreads) {
-      // one key per thread: its rank among the segment's (distinct) keys is
-      // its position -- two barriers instead of a bitonic network's stages
-      unsigned long long ki = 0ull;
-      if ((int)threadIdx.x < len) ki = keys[threadIdx.x] = ts.seg_keys[start + threadIdx.x];
-      __syncthreads();
-      if ((int)threadIdx.x < len) {
-        int rank = 0, j = 0;
-        for (; j + 1 < len; j += 2) {
-          const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(keys + j);
-          rank += (int)(kk.x < ki) + (int)(kk.y < ki);
-        }
-        if (j < len) rank += (int)(keys[j] < ki);
-        s_ids[rank] = min((uint32_t)(ki & 0xFFFFFFFFull), (uint32_t)(ts.n - 1));
-      }
-      __syncthreads();
+      if ((int)threadIdx.x < len) keys[threadIdx.x] = ts.seg_keys[start + threadIdx.x];
+      rank_ids(keys, len, s_ids, ts.n);
       ids = s_ids;
     } else if (len <= kSegSmem) {
       for (int i = threadIdx.x; i < len; i += kTileThreads) keys[i] = ts.seg_keys[start + i];
@@ -273,7 +366,7 @@ __global__ void __launch_bounds__(kTileThreads, tile_blocks_per_sm<P, kG>()) tra
     }
   }
   FwdState st[P];
-  fwd_tile<kBwdVec4, false, P, kG>(proj, ids, start, end, xt, yt, tile_x0, tile_y0, tp, inside,
+  fwd_tile<kBwdVec4, false, P>(proj, ids, start, end, xt, yt, tile_x0, tile_y0, tp, inside,
                                    cam, cfg, sm.rec, hl, nullptr, st);
   float pr[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   const float inv = 1.f / (float)(cam.width * cam.height);
@@ -299,37 +392,290 @@ __global__ void __launch_bounds__(kTileThreads, tile_blocks_per_sm<P, kG>()) tra
     pg[k].gD = L.g_depth;
     pg[k].gO = L.g_opac;
   }
-  {
-    float v = loss;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if ((threadIdx.x & 31) == 0) s_loss[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float t = 0.f;
-      for (int w = 0; w < kTileThreads / 32; ++w) t += s_loss[w];
-      loss_part[tile] = t;
-    }
-  }
+  for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, off);
+  if ((threadIdx.x & 31) == 0) s.loss[threadIdx.x >> 5] = loss;
   // a list of at most one batch is still staged with its hit lists
-  bwd_tile_pose<false, P, kG>(proj, ids, start, end, xt, yt, tile_x0, tile_y0, tp, inside, rx, ry,
+  bwd_tile_pose<false, P>(proj, ids, start, end, xt, yt, tile_x0, tile_y0, tp, inside, rx, ry,
                               cam, cfg, pg, sm, hl, pr, end - start <= kTileThreads);
-  block_sum6(pr, s_pose, pose_part + (size_t)tile * 6);
-  // the last block to finish reduces every tile's partials and updates the pose
+  warp_sum6(pr, s.pose);
+}
+
+// The last block of a fused tracking launch to finish reduces the tiles'
+// partials and updates the pose.
+__device__ __forceinline__ void track_finish(const float* pose_part, const float* loss_part,
+                                             int n_tiles, const TrackStep& ts,
+                                             const gs2d_track_params& prm, int32_t* status,
+                                             bool* s_last, float (*s_red)[256]) {
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(ts.counter, 1u) == gridDim.x - 1;
+  if (threadIdx.x == 0) *s_last = atomicAdd(ts.counter, 1u) == gridDim.x - 1;
   __syncthreads();
-  if (!s_last) return;
+  if (!*s_last) return;
   __threadfence();
-  float(*s_red)[256] = reinterpret_cast<float(*)[256]>(&sm.rec[0][0]);  // 7 x 256 floats fit
-  reduce_and_step(pose_part, loss_part, gridDim.x, ts.pose, ts.adam, prm, ts.loss_hist,
+  reduce_and_step(pose_part, loss_part, n_tiles, ts.pose, ts.adam, prm, ts.loss_hist,
                   ts.pose_hist, ts.grad_hist, ts.iter, status, s_red);
   if (threadIdx.x == 0) *ts.counter = 0u;
   // the next iteration's binning starts from zeroed counters (its kernels
   // run after this one; this iteration's binning finished before it)
   if (ts.sort_zero)
     for (size_t i = threadIdx.x; i < ts.sort_zero_words; i += blockDim.x) ts.sort_zero[i] = 0u;
+}
+
+// The tile's partial from its warps' sums, added in warp order.
+__device__ __forceinline__ void write_tile_partial(const TrackSmem& s, int tile, float* pose_part,
+                                                   float* loss_part) {
+  __syncthreads();
+  if (threadIdx.x < 7) {
+    float v = 0.f;
+    for (int w = 0; w < kTileThreads / 32; ++w)
+      v += threadIdx.x < 6 ? s.pose[w][threadIdx.x] : s.loss[w];
+    if (threadIdx.x < 6)
+      pose_part[(size_t)tile * 6 + threadIdx.x] = v;
+    else
+      loss_part[tile] = v;
+  }
+}
+
+// Whether the launch's status lets the block run; records the history of an
+// iteration skipped after convergence.
+__device__ __forceinline__ bool track_runs(const TrackStep& ts, const int32_t* status) {
+  const int32_t g = *status;
+  if (g == kConverged && blockIdx.x == 0 && threadIdx.x == 0)
+    record_converged(ts.pose, ts.loss_hist, ts.pose_hist, ts.grad_hist, ts.iter);
+  return g == 0;
+}
+
+template <int P>
+__global__ void __launch_bounds__(kTileThreads, tile_blocks_per_sm<P>()) track_tile_kernel(
+    const float4* __restrict__ proj, uint32_t* vals,
+    const int32_t* __restrict__ ranges, gs2d_camera cam, gs2d_config cfg, int tiles_x,
+    const float* __restrict__ obs_rgb, const float* __restrict__ obs_depth, gs2d_track_params prm,
+    float* __restrict__ loss_part, float* __restrict__ pose_part, TrackStep ts,
+    int32_t* __restrict__ status) {
+  __shared__ TrackSmem s;
+  __shared__ bool s_last;
+  if (!track_runs(ts, status)) return;
+  // longest lists first: the blocks of the heaviest tiles start in the first
+  // wave instead of trailing the grid (partials stay indexed by tile)
+  const int tile = ts.order ? ts.order[blockIdx.x] : (int)blockIdx.x;
+  track_tile<P>(tile, proj, vals, ranges, cam, cfg, tiles_x, obs_rgb, obs_depth, prm, ts, s);
+  write_tile_partial(s, tile, pose_part, loss_part);
+  // 7 x 256 floats fit
+  track_finish(pose_part, loss_part, gridDim.x, ts, prm, status, &s_last,
+               reinterpret_cast<float(*)[256]>(&s.b.rec[0][0]));
+}
+
+// The fused iteration with one pixel per thread, tile by tile or on 8 x 8
+// quadrants (quad.cuh): a quadrant's block takes the keys of its tile's
+// segment whose footprint touches the quadrant, sorts them, blends, evaluates
+// the loss and replays.  The first `split` tiles of the launch order have four
+// blocks each (three of them leave at once when their tile runs whole), the
+// others one; SplitRule says where the line lies.  Segments of more than
+// kQuadKeys keys run whole.
+// A quadrant writes one partial per 8 x 4 pixel block and the last of the
+// tile's four blocks adds the eight up in the whole-tile form's order, so the
+// results do not depend on the choice.
+constexpr int kQuadKeys = 3072;
+struct QuadTrackSmem {
+  union {
+    QuadStage<kBwdVec4> st;
+    unsigned long long keys[kQuadKeys + 2];
+  };
+  uint32_t ids[kQuadKeys];
+  float out[7][64];     // per pixel: the pose 6-vector and the loss
+  int cnt;
+};
+constexpr int kTileParts = kTileThreads / 32;   // 8 x 4 blocks (partials) per tile
+
+// Which tiles run on quadrants.  Four blocks finish a tile in a third of the
+// time one takes, with about twice the instructions in all, so they pay where
+// a tile would outlast the rest of the launch: where its list is longer than
+// per_slot x K, the mean share of the K entries per resident block slot times
+// a constant, and than min_len (below it the fixed cost of a block, ~15 us,
+// is most of a tile's time).  Measured over 10 iterations, whole tiles alone
+// -> this rule (three poses each, us):
+//   160x120 (80 tiles), 200k surfels   2088-2649 -> 734-1219
+//   320x240 (300 tiles), 200k surfels  1086-1742 -> 938-1075
+//   480x360 (690 tiles), 200k surfels   973-1464 -> 964-1015
+//   640x480 (1200 tiles), 200k surfels 1087-1366 -> 1099-1254
+//   320x240 (300 tiles), 50k surfels    423-620  -> 417-523
+// Up to two tiles per SM every tile may split and the other three blocks of
+// each follow the tiles (their early exits then cost nothing where no tile
+// splits); in larger grids only the half of the SM count longest tiles may,
+// and their blocks lead the launch, so that they overlap the whole of it.
+struct SplitRule {
+  int split;         // tiles (in launch order) that may run on quadrants
+  int extras_first;  // their four blocks each lead the grid
+  int min_len;
+  float per_slot;
+};
+
+__global__ void __launch_bounds__(kTileThreads, 4) track_quad_kernel(
+    const float4* __restrict__ proj, uint32_t* vals,
+    const int32_t* __restrict__ ranges, const int32_t* __restrict__ n_isect, gs2d_camera cam,
+    gs2d_config cfg, int tiles_x, int n_tiles,
+    const float* __restrict__ obs_rgb, const float* __restrict__ obs_depth, gs2d_track_params prm,
+    float* __restrict__ loss_part, float* __restrict__ pose_part, SplitRule rule, TrackStep ts,
+    int32_t* __restrict__ status) {
+  __shared__ union Smem {
+    QuadTrackSmem q;
+    TrackSmem t;
+    float red[7][256];
+    __device__ Smem() {}
+  } sh;
+  __shared__ bool s_last;
+  if (!track_runs(ts, status)) return;
+  const int b0 = (int)blockIdx.x;
+  int rank, quad;
+  if (rule.extras_first) {
+    const int rest = b0 - kQuads * rule.split;
+    rank = rest < 0 ? b0 / kQuads : rule.split + rest;
+    quad = rest < 0 ? b0 % kQuads : 0;
+  } else {
+    const int extra = b0 - n_tiles;
+    rank = extra < 0 ? b0 : extra / (kQuads - 1);
+    quad = extra < 0 ? 0 : 1 + extra % (kQuads - 1);
+  }
+  const int tile = ts.order[rank];
+  const int start = ranges[2 * tile], end = ranges[2 * tile + 1], len = end - start;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool on_quads = rank < rule.split && len > rule.min_len && len <= kQuadKeys &&
+                        (float)len > rule.per_slot * (float)*n_isect;
+  if (!on_quads) {
+    if (quad == 0) {
+      track_tile<1>(tile, proj, vals, ranges, cam, cfg, tiles_x, obs_rgb, obs_depth, prm, ts, sh.t);
+      write_tile_partial(sh.t, tile, pose_part, loss_part);
+    }
+  } else {
+    QuadTrackSmem& s = sh.q;
+    const int tile_x0 = (tile % tiles_x) * cfg.tile_w, tile_y0 = (tile / tiles_x) * cfg.tile_h;
+    const QuadPix tp = quad_pixel(quad, tile_x0, tile_y0, cfg.tile_w);
+    const bool inside = tp.px < cam.width && tp.py < cam.height;
+    const float xt = (float)tile_x0 + 0.5f - cam.cx;
+    const float yt = (float)tile_y0 + 0.5f - cam.cy;
+    const float rx = (tp.px + 0.5f - cam.cx) / cam.fx, ry = (tp.py + 0.5f - cam.cy) / cam.fy;
+    // the quadrant's keys, in any order
+    if (threadIdx.x == 0) s.cnt = 0;
+    __syncthreads();
+    for (int i0 = 0; i0 < len; i0 += kTileThreads) {
+      const int i = i0 + (int)threadIdx.x;
+      unsigned long long key = 0ull;
+      bool hit = false;
+      if (i < len) {
+        key = ts.seg_keys[start + i];
+        const uint32_t id = min((uint32_t)(key & 0xFFFFFFFFull), (uint32_t)(ts.n - 1));
+        const float4 r7 = proj[(size_t)id * (kProjFloats / 4) + 7];
+        hit = quad_mask(r7.z, r7.w, tp.x0, tp.y0) != 0u;
+      }
+      const uint32_t b = __ballot_sync(0xffffffffu, hit);
+      int o = 0;
+      if (lane == 0 && b) o = atomicAdd(&s.cnt, __popc(b));
+      o = __shfl_sync(0xffffffffu, o, 0);
+      if (hit) s.keys[o + __popc(b & ((1u << lane) - 1u))] = key;
+    }
+    __syncthreads();
+    const int n = s.cnt;
+    // counting ranks costs n^2 / 256 comparisons a thread, the network
+    // log^2(n) / 2 barriers: about even at 768 keys
+    if (n <= kRankPer * kTileThreads) {
+      rank_ids(s.keys, n, s.ids, ts.n);
+    } else {
+      bitonic_sort(s.keys, n);
+      for (int i = threadIdx.x; i < n; i += kTileThreads)
+        s.ids[i] = min((uint32_t)(s.keys[i] & 0xFFFFFFFFull), (uint32_t)(ts.n - 1));
+      __syncthreads();
+    }
+    auto stage = [&](int b, int cnt) {   // entries b .. b + cnt - 1; returns the warp's hits
+      if ((int)threadIdx.x < cnt) {
+        stage_record_to<kBwdVec4>(proj, s.ids[b + threadIdx.x], xt, yt, s.st.rec[threadIdx.x]);
+        const float4 r6 = s.st.rec[threadIdx.x][6];
+        s.st.mask[threadIdx.x] = (uint8_t)quad_mask(r6.z, r6.w, tp.x0, tp.y0);
+      }
+      __syncthreads();
+      return quad_hits(s.st, cnt);
+    };
+    QuadFwd st = quad_fwd_init(inside);
+    int nh = 0, staged = 0;   // the batch in shared memory
+    for (int b = 0; b < n; b += kQuadBatch) {
+      if (__syncthreads_count(!st.done) == 0) break;
+      nh = stage(b, min(kQuadBatch, n - b));
+      staged = b;
+      quad_blend(s.st, nh, tp, cam, cfg, st, [&](int j) { return (uint32_t)(b + j + 1); });
+    }
+    const QuadOut o = quad_gather(st);
+    const float inv = 1.f / (float)(cam.width * cam.height);
+    PixLoss L;
+    L.loss = 0.f;
+    L.g_rgb[0] = L.g_rgb[1] = L.g_rgb[2] = 0.f;
+    L.g_depth = L.g_opac = 0.f;
+    if (inside) {
+      const size_t p = (size_t)tp.py * cam.width + tp.px;
+      L = tracking_pixel_loss(o.C, o.D, o.N, 1.f - st.T,
+                              f3(obs_rgb[3 * p], obs_rgb[3 * p + 1], obs_rgb[3 * p + 2]),
+                              obs_depth[p], rx, ry, inv, prm);
+    }
+    PixGrad pg;
+    pg.Tf = st.T;
+    pg.nl = st.last;
+    pg.gC = f3(L.g_rgb[0], L.g_rgb[1], L.g_rgb[2]);
+    pg.gN = f3(0.f, 0.f, 0.f);
+    pg.gD = L.g_depth;
+    pg.gO = L.g_opac;
+    QuadBwd bw;
+    bw.T = st.T;
+    bw.acc = 0.f;
+    bw.sG = bw.szG = f3(0.f, 0.f, 0.f);
+    for (int b = staged; b >= 0 && n > 0; b -= kQuadBatch) {
+      if (b != staged) {
+        __syncthreads();
+        nh = stage(b, kQuadBatch);
+      }
+      quad_replay(s.st, nh, b, tp, cam, cfg, pg, rx, ry, cam.fx * cam.fy, bw);
+    }
+    const F3 th = cross3(f3(rx, ry, 1.f), bw.szG);
+    if ((lane & 3) == 0) {
+      s.out[0][tp.slot] = bw.sG.x;
+      s.out[1][tp.slot] = bw.sG.y;
+      s.out[2][tp.slot] = bw.sG.z;
+      s.out[3][tp.slot] = th.x;
+      s.out[4][tp.slot] = th.y;
+      s.out[5][tp.slot] = th.z;
+      s.out[6][tp.slot] = L.loss * inv;
+    }
+    __syncthreads();
+    // the quadrant's two 8 x 4 blocks, each summed over its lanes as a warp
+    // of the plain form sums them
+    for (int v = warp; v < 14; v += kTileThreads / 32) {
+      const int c = v >> 1, half = v & 1;
+      float x = s.out[c][32 * half + lane];
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+      // block (8 x 4) of the tile: row 2 (quadrant row) + half
+      const int per_row = cfg.tile_w >> 3;
+      const size_t part = (size_t)rank * kTileParts +
+                          (2 * (quad / per_row) + half) * per_row + quad % per_row;
+      if (lane == 0) ts.quad_part[part * 7 + c] = x;
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s.cnt = (int)atomicAdd(ts.quad_done + rank, 1u);
+    __syncthreads();
+    if (s.cnt == kQuads - 1) {
+      __threadfence();
+      if (threadIdx.x < 7) {
+        float v = 0.f;
+        for (int w = 0; w < kTileParts; ++w)
+          v += __ldcg(ts.quad_part + ((size_t)rank * kTileParts + w) * 7 + threadIdx.x);
+        if (threadIdx.x < 6)
+          pose_part[(size_t)tile * 6 + threadIdx.x] = v;
+        else
+          loss_part[tile] = v;
+      }
+      if (threadIdx.x == 0) ts.quad_done[rank] = 0u;   // for the next iteration
+    }
+  }
+  track_finish(pose_part, loss_part, n_tiles, ts, prm, status, &s_last, sh.red);
 }
 
 // Per-surfel reduction of the (tile, region, surfel) partials in emission
@@ -494,22 +840,31 @@ int validate_tile_cfg(const gs2d_camera* cam, const gs2d_config* cfg) {
   return GS2D_OK;
 }
 
-// Tile grids of at most this many tiles run the grouped one-pixel loops
-// (-1: twice the device's SM count, i.e. at most two blocks per SM).
+// gs2d_set_grouped_tiles: grids of at most this many tiles run on quadrants
+// (quad.cuh); -1: the library's own rule.
 static int g_grouped_max_tiles = -1;
 
-// Whether a one-pixel tile kernel over n_tiles tiles takes the grouped loops.
+static int sm_count() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 0;
+  return sms;
+}
+
+// Whether the forward pass of a one-pixel grid of n_tiles tiles runs on
+// quadrants: up to two tiles per SM.
 static bool use_grouped(int px_per_thread, int n_tiles) {
   if (px_per_thread != 1) return false;
-  int limit = g_grouped_max_tiles;
-  if (limit < 0) {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      return false;
-    limit = 2 * sms;
-  }
-  return n_tiles <= limit;
+  return n_tiles <= (g_grouped_max_tiles < 0 ? 2 * sm_count() : g_grouped_max_tiles);
+}
+
+static SplitRule split_rule(int n_tiles) {
+  if (g_grouped_max_tiles >= 0)
+    return SplitRule{n_tiles <= g_grouped_max_tiles ? n_tiles : 0, 0, 0, 0.f};
+  const int sms = max(sm_count(), 1), slots = 4 * sms;
+  if (n_tiles <= 2 * sms) return SplitRule{n_tiles, 0, 80, 1.25f / slots};
+  return SplitRule{min(sms / 2, n_tiles), 1, 80, 1.75f / slots};
 }
 
 int render_fwd_launch(const float* proj, const gs2d_bins* bins, const gs2d_camera* cam,
@@ -524,9 +879,9 @@ int render_fwd_launch(const float* proj, const gs2d_bins* bins, const gs2d_camer
   if (reinterpret_cast<uintptr_t>(proj) & 15) return GS2D_ERR_INVALID_ARG;
   const int tx = gs2d_tiles_x(cam, cfg), ty = gs2d_tiles_y(cam, cfg);
   if (use_grouped(cfg->px_per_thread, tx * ty))
-    render_fwd_kernel<false, 1, kGroup><<<tx * ty, kTileThreads, 0, st>>>(
+    render_fwd_quad_kernel<<<tx * ty * kQuads, kTileThreads, 0, st>>>(
         reinterpret_cast<const float4*>(proj), bins->vals, bins->tile_ranges, *cam, *cfg, tx, rgb,
-        depth, normal, opacity, t_final, n_last, nullptr, gate);
+        depth, normal, opacity, t_final, n_last, gate);
   else
     GS2D_DISPATCH_P(cfg->px_per_thread, render_fwd_kernel<false, P><<<tx * ty, kTileThreads, 0, st>>>(
         reinterpret_cast<const float4*>(proj), bins->vals, bins->tile_ranges, *cam, *cfg, tx, rgb,
@@ -534,6 +889,11 @@ int render_fwd_launch(const float* proj, const gs2d_bins* bins, const gs2d_camer
   GS2D_LAUNCH_CHECK();
   return GS2D_OK;
 }
+
+#define GS2D_TRACK_TILE(P)                                                                      \
+  track_tile_kernel<P><<<tx * ty, kTileThreads, 0, st>>>(                                       \
+      reinterpret_cast<const float4*>(proj), bins->vals, bins->tile_ranges, *cam, *cfg, tx,     \
+      obs_rgb, obs_depth, *prm, loss_part, pose_part, ts, status)
 
 int track_tile_launch(const float* proj, const gs2d_bins* bins, const gs2d_camera* cam,
                       const gs2d_config* cfg, const float* obs_rgb, const float* obs_depth,
@@ -545,14 +905,19 @@ int track_tile_launch(const float* proj, const gs2d_bins* bins, const gs2d_camer
       !loss_part || !pose_part || !ts.pose || !ts.adam || !ts.counter || !status)
     return GS2D_ERR_INVALID_ARG;
   const int tx = gs2d_tiles_x(cam, cfg), ty = gs2d_tiles_y(cam, cfg);
-  if (use_grouped(cfg->px_per_thread, tx * ty))
-    track_tile_kernel<1, kGroup><<<tx * ty, kTileThreads, 0, st>>>(
-        reinterpret_cast<const float4*>(proj), bins->vals, bins->tile_ranges, *cam, *cfg, tx,
-        obs_rgb, obs_depth, *prm, loss_part, pose_part, ts, status);
-  else
-    GS2D_DISPATCH_P(cfg->px_per_thread, track_tile_kernel<P><<<tx * ty, kTileThreads, 0, st>>>(
-        reinterpret_cast<const float4*>(proj), bins->vals, bins->tile_ranges, *cam, *cfg, tx,
-        obs_rgb, obs_depth, *prm, loss_part, pose_part, ts, status));
+  if (cfg->px_per_thread == 1) {
+    if (!bins->n_isect || !ts.order || !ts.quad_part || !ts.quad_done) return GS2D_ERR_INVALID_ARG;
+    const SplitRule rule = split_rule(tx * ty);
+    track_quad_kernel<<<tx * ty + (kQuads - 1) * rule.split, kTileThreads, 0, st>>>(
+        reinterpret_cast<const float4*>(proj), bins->vals, bins->tile_ranges, bins->n_isect, *cam,
+        *cfg, tx, tx * ty, obs_rgb, obs_depth, *prm, loss_part, pose_part, rule, ts, status);
+  } else {
+    switch (cfg->px_per_thread) {
+      case 2: GS2D_TRACK_TILE(2); break;
+      case 3: GS2D_TRACK_TILE(3); break;
+      default: GS2D_TRACK_TILE(4); break;
+    }
+  }
   GS2D_LAUNCH_CHECK();
   return GS2D_OK;
 }

@@ -199,12 +199,7 @@ struct HitLists {
   int count[kTileThreads / 32];  // each warp's hit count of the last staged batch
 };
 
-// kG > 1 (one pixel per thread, no counting): the warp's hits are taken kG at
-// a time -- their records loaded and their (pixel, surfel) pairs evaluated
-// independently, then blended in list order -- so a pixel's walk keeps kG
-// evaluations in flight instead of one.  Same evaluations, same order, same
-// results; pairs after a pixel's stop are evaluated and dropped.
-template <int kStride, bool kCount, int P, int kG = 1>
+template <int kStride, bool kCount, int P>
 __device__ __forceinline__ void fwd_tile(const float4* __restrict__ proj,
                                          const uint32_t* ids, int start, int end,
                                          float xt, float yt, int tile_x0, int tile_y0,
@@ -248,48 +243,7 @@ __device__ __forceinline__ void fwd_tile(const float4* __restrict__ proj,
     const int cnt_b = min(kTileThreads, end - b);
     const int nh = warp_hit_list(hl.mask, hl.list[warp], cnt_b, warp, lane);
     if (lane == 0) hl.count[warp] = nh;
-    if (P == 1 && kG > 1 && !kCount && !all_done) {
-      FwdState& q = st[0];
-      for (int h0 = 0; h0 < nh && !all_done; h0 += kG) {
-        int jg[kG];
-        float ag[kG], zg[kG], cg[kG];
-        bool hg[kG];
-#pragma unroll
-        for (int g = 0; g < kG; ++g) {
-          // past the end: re-evaluate the last hit, never blended
-          jg[g] = hl.list[warp][min(h0 + g, nh - 1)];
-          const float4 r0 = s_rec[jg[g]][0], r1 = s_rec[jg[g]][1], r2 = s_rec[jg[g]][2];
-          Eval e;
-          hg[g] = eval_pair(r0, r1, r2, tp.lx, tp.ly, cam.near_z, cfg.cutoff_r2, cfg.alpha_min,
-                            cfg.alpha_max, e) &&
-                  h0 + g < nh;
-          ag[g] = e.a;
-          zg[g] = e.z;
-          cg[g] = r2.w;
-        }
-#pragma unroll
-        for (int g = 0; g < kG; ++g) {
-          if (!hg[g]) continue;
-          const float Tn = q.T * (1.f - ag[g]);
-          if (Tn < cfg.t_min) {
-            all_done = true;
-            break;
-          }
-          const float4 r3 = s_rec[jg[g]][3];
-          const float tnz = s_rec[jg[g]][4].x;
-          const float w = ag[g] * q.T;
-          q.C.x = fmaf(w, cg[g], q.C.x);
-          q.C.y = fmaf(w, r3.x, q.C.y);
-          q.C.z = fmaf(w, r3.y, q.C.z);
-          q.D = fmaf(w, zg[g], q.D);
-          q.N.x = fmaf(w, r3.z, q.N.x);
-          q.N.y = fmaf(w, r3.w, q.N.y);
-          q.N.z = fmaf(w, tnz, q.N.z);
-          q.T = Tn;
-          q.last = (uint32_t)(b + jg[g] + 1 - start);
-        }
-      }
-    } else if (P == 1 && !all_done) {
+    if (P == 1 && !all_done) {
       // one pixel: stop at its saturation
       FwdState& q = st[0];
       for (int h = 0; h < nh; ++h) {
@@ -447,13 +401,11 @@ __device__ __forceinline__ void pose_pair(const Eval& e, const float4 r2, const 
 // and z Gv; with q = s (u d_u + v d_v), s = -G dL/dG, the pair's
 // Gv = beta n - q, beta = (q . r + gz) / (n . r).  kNormal adds the normal
 // image's term t_nc x w gN per pair (tracking has no normal gradient).
-// kG > 1 (one pixel per thread): hits are taken kG at a time, their pairs
-// evaluated independently and then replayed in back-to-front order (as in
-// fwd_tile).  staged: the tile's whole list (at most one batch) is still
+// staged: the tile's whole list (at most one batch) is still
 // staged in sm.rec with the per-warp hit lists of fwd_tile<kBwdVec4> in hl
 // (the fused tracking kernel), so neither is rebuilt; entries past a
 // pixel's last blended one are skipped per pixel as always.
-template <bool kNormal, int P, int kG = 1>
+template <bool kNormal, int P>
 __device__ __forceinline__ void bwd_tile_pose(const float4* __restrict__ proj,
                                               const uint32_t* ids, int start, int end,
                                               float xt, float yt, int tile_x0, int tile_y0,
@@ -512,30 +464,6 @@ __device__ __forceinline__ void bwd_tile_pose(const float4* __restrict__ proj,
       nh = warp_hit_list(hl.mask, hl.list[warp], cnt, warp, lane);
     }
     if (!any_inside) continue;
-    if (P == 1 && kG > 1) {
-      for (int h0 = nh - 1; h0 >= 0; h0 -= kG) {
-        int jg[kG];
-        bool vg[kG];
-        Eval eg[kG];
-        float4 r2g[kG];
-#pragma unroll
-        for (int g = 0; g < kG; ++g) {
-          // before the start: re-evaluate the first hit, never replayed
-          jg[g] = hl.list[warp][max(h0 - g, 0)];
-          const float4 r0 = sm.rec[jg[g]][0], r1 = sm.rec[jg[g]][1];
-          r2g[g] = sm.rec[jg[g]][2];
-          vg[g] = eval_pair(r0, r1, r2g[g], tp.lx, lyk[0], cam.near_z, cfg.cutoff_r2,
-                            cfg.alpha_min, cfg.alpha_max, eg[g]) &&
-                  h0 - g >= 0 && bstart + jg[g] - start < (int)pg[0].nl;
-        }
-#pragma unroll
-        for (int g = 0; g < kG; ++g)
-          if (vg[g])
-            pose_pair<kNormal>(eg[g], r2g[g], sm.rec[jg[g]], pg[0], rx, ryk[0], fxfy,
-                               cfg.alpha_max, gOT[0], T[0], acc[0], sG, szG[0], sN[0]);
-      }
-      continue;
-    }
     for (int h = nh - 1; h >= 0; --h) {
       const int jj = hl.list[warp][h];
       const int jrel = bstart + jj - start;
@@ -566,9 +494,8 @@ __device__ __forceinline__ void bwd_tile_pose(const float4* __restrict__ proj,
   pr[5] += th.z;
 }
 
-// Block sum of a per-thread 6-vector, written by threads 0..5.
-__device__ __forceinline__ void block_sum6(const float (&pr)[6], float (*s_pose)[6],
-                                           float* __restrict__ out) {
+// Warp sums of a per-thread 6-vector.
+__device__ __forceinline__ void warp_sum6(const float (&pr)[6], float (*s_pose)[6]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
@@ -577,6 +504,12 @@ __device__ __forceinline__ void block_sum6(const float (&pr)[6], float (*s_pose)
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     if (lane == 0) s_pose[warp][i] = v;
   }
+}
+
+// Block sum of a per-thread 6-vector, written by threads 0..5.
+__device__ __forceinline__ void block_sum6(const float (&pr)[6], float (*s_pose)[6],
+                                           float* __restrict__ out) {
+  warp_sum6(pr, s_pose);
   __syncthreads();
   if (threadIdx.x < 6) {
     float v = 0.f;

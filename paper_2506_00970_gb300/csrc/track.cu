@@ -44,13 +44,15 @@ cudaError_t record_timing_event(cudaEvent_t ev, cudaStream_t st) {
 // binning counters, and the moments when they live in the workspace (a
 // caller-owned AdamW state is left as the caller passed it).
 __global__ void track_reset_kernel(float* adam, uint32_t* counter, int32_t* status,
-                                   uint32_t* sort_zero, size_t sort_zero_words) {
+                                   uint32_t* sort_zero, size_t sort_zero_words,
+                                   uint32_t* quad_done, int n_tiles) {
   if (adam && threadIdx.x < 16) adam[threadIdx.x] = 0.f;
   if (threadIdx.x == 0) {
     *counter = 0u;
     *status = 0;
   }
   for (size_t i = threadIdx.x; i < sort_zero_words; i += blockDim.x) sort_zero[i] = 0u;
+  for (int i = threadIdx.x; i < n_tiles; i += blockDim.x) quad_done[i] = 0u;
 }
 
 struct TrackWs {
@@ -60,8 +62,8 @@ struct TrackWs {
   int32_t *ranges, *n_isect, *order;
   void* sort_ws;
   size_t sort_bytes;
-  float *loss_part, *pose_part, *adam;
-  uint32_t* counter;
+  float *loss_part, *pose_part, *quad_part, *adam;
+  uint32_t *counter, *quad_done;
   size_t bytes;
 };
 
@@ -84,6 +86,8 @@ TrackWs carve_track_ws(void* base, int n, size_t cap, const gs2d_camera* cam,
   w.sort_ws = c.take<char>(w.sort_bytes);
   w.loss_part = c.take<float>((size_t)nt);
   w.pose_part = c.take<float>((size_t)nt * 6);
+  w.quad_part = c.take<float>((size_t)nt * 8 * 7);
+  w.quad_done = c.take<uint32_t>((size_t)nt);
   w.adam = c.take<float>(16);
   w.counter = c.take<uint32_t>(1);
   w.bytes = align_up(c.off, 256);
@@ -154,7 +158,8 @@ int gs2d_track_step(const gs2d_surfels* s, const gs2d_camera* cam, const gs2d_co
                    &zero_begin, &zero_words);
   float* adam = adam_state ? adam_state : w.adam;
   track_reset_kernel<<<1, 256, 0, st>>>(adam_state ? nullptr : w.adam, w.counter, status,
-                                        zero_begin, zero_words);
+                                        zero_begin, zero_words, w.quad_done,
+                                        gs2d_tiles_x(cam, cfg) * gs2d_tiles_y(cam, cfg));
   GS2D_LAUNCH_CHECK();
   gs2d_bins bins;
   bins.keys = nullptr;
@@ -191,7 +196,7 @@ int gs2d_track_step(const gs2d_surfels* s, const gs2d_camera* cam, const gs2d_co
     const bool timed = g_timer.used < g_timer.capacity && it % g_timer.every == 0;
     if (timed) GS2D_CUDA_TRY(record_timing_event(g_timer.start[g_timer.used], st));
     TrackStep ts{pose, adam, loss_hist, pose_hist, grad_hist, it, w.counter, zero_begin,
-                 zero_words, w.order, seg_keys, seg_tmp, s->n};
+                 zero_words, w.order, seg_keys, seg_tmp, s->n, w.quad_part, w.quad_done};
     r = track_tile_launch(w.proj, &bins, cam, cfg, obs_rgb, obs_depth, prm, w.loss_part,
                           w.pose_part, ts, status, st);
     if (r) return r;

@@ -62,20 +62,20 @@ __device__ __forceinline__ void record_converged(const float* __restrict__ pose,
     for (int k = 0; k < 6; ++k) grad_hist[6 * iter + k] = 0.f;
 }
 
-// Block-wide (256 threads): sum the n_part partials in a fixed order (L1 is
-// bypassed: other blocks wrote them), then thread 0 takes the AdamW step
+// Block-wide (256 threads): sum the partials of n_tiles tiles in a fixed order
+// (L1 is bypassed: other blocks wrote them), then thread 0 takes the AdamW step
 // (tau is zero before the step, so weight decay has no effect) and retracts.
 // Records the loss and the gradient at the pre-update pose and the updated
 // pose.  A non-finite loss or gradient leaves the pose and the moments as
 // they were and records GS2D_ERR_NONFINITE.  adam = m[6], v[6], step, done.
 __device__ __forceinline__ void reduce_and_step(const float* __restrict__ pose_part,
-                                const float* __restrict__ loss_part, int n_part,
+                                const float* __restrict__ loss_part, int n_tiles,
                                 float* __restrict__ pose, float* __restrict__ adam,
                                 const gs2d_track_params& prm, float* __restrict__ loss_hist,
                                 float* __restrict__ pose_hist, float* __restrict__ grad_hist,
                                 int iter, int32_t* __restrict__ status, float (*s)[256]) {
   float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  for (int b = threadIdx.x; b < n_part; b += 256) {
+  for (int b = threadIdx.x; b < n_tiles; b += 256) {
 #pragma unroll
     for (int c = 0; c < 6; ++c) acc[c] += __ldcg(pose_part + (size_t)b * 6 + c);
     acc[6] += __ldcg(loss_part + b);

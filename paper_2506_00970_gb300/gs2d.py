@@ -359,8 +359,8 @@ def gs2d_render_count(proj, bins: Bins, cam: Camera, cfg: Config, counts, stream
 
 
 def gs2d_set_grouped_tiles(max_tiles: int):
-    """Tile grids of at most max_tiles tiles run the grouped one-pixel
-    compositing loops (-1: twice the SM count, the default; 0: never)."""
+    """Tile grids of at most max_tiles tiles run the grouped form of the
+    one-pixel compositing (-1: the library's rule, the default; 0: never)."""
     lib().gs2d_set_grouped_tiles(int(max_tiles))
 
 

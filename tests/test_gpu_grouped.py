@@ -92,3 +92,45 @@ def test_grouped_tracking_frame_is_bit_identical(torch_cuda, case):
     assert hist[0][0][0] > 0
     for x, y in zip(hist[0], hist[1]):
         np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("w,h,f,tile", [
+    (160, 120, 150.0, (16, 16)),     # lists of a few batches
+    (112, 84, 105.0, (16, 16)),      # quadrants of more than 768 keys
+    (64, 48, 60.0, (16, 16)),        # segments too long for the quadrant form
+    (101, 77, 95.0, (8, 32)),        # the other tile shapes, ragged image
+    (101, 77, 95.0, (32, 8)),
+    (333, 251, 275.0, (16, 16)),     # more tiles than may split, some of them long
+])
+def test_grouped_forms_agree_over_list_lengths_and_shapes(torch_cuda, w, h, f, tile):
+    """Forward images and a short tracking call, whole tiles against quadrants
+    and against the library's choice per tile: bit-identical."""
+    torch = torch_cuda
+    from paper_2506_00970_gb300 import gs2d
+    cam = scenes.Camera(f, f, w / 2, h / 2, w, h)
+    s = scenes.room_scene(3, 200_000)
+    ds = gs2d.DeviceSurfels(s)
+    gt = scenes.room_pose(11)
+    ccam, cfg = gs2d.camera(cam), gs2d.default_config(tile)
+    prm = gs2d.default_track_params(stop_tol=0.0)
+    cap = 8 * s.n
+    obs, res = None, []
+    for limit in (0, 1 << 30, -1):
+        gs2d.gs2d_set_grouped_tiles(limit)
+        r = gs2d.Rasterizer(cam, s.n, tile=tile)
+        out = {k: v.clone() for k, v in r.forward(ds, gs2d.pose_tensor(gt)).items()}
+        if obs is None:
+            obs = out["rgb"], out["depth"] / out["opacity"].clamp_min(1e-6)
+        ws = torch.empty(gs2d.gs2d_track_workspace(s.n, cap, ccam, cfg), dtype=torch.uint8,
+                         device="cuda")
+        pose = gs2d.pose_tensor(scenes.perturb_pose(gt, 0.02, 1.0, seed=7))
+        lh, gh = torch.zeros(4, device="cuda"), torch.zeros(4, 6, device="cuda")
+        gs2d.gs2d_track_step(ds, ccam, cfg, prm, pose, *obs, 4, cap, lh, None, ws, grad_hist=gh)
+        torch.cuda.synchronize()
+        assert int(gs2d.gs2d_track_status(ws).item()) == 0
+        res.append(dict(out, loss=lh, grad=gh, pose=pose))
+    gs2d.gs2d_set_grouped_tiles(-1)
+    assert float(res[0]["loss"][0]) > 0
+    for other in res[1:]:
+        for k in res[0]:
+            assert torch.equal(res[0][k], other[k]), k
