@@ -67,229 +67,220 @@ __global__ void __launch_bounds__(256) sum_parts_kernel(const float* __restrict_
 // pixels whose own and 4-neighbour opacities exceed 0.5.  The normal term's
 // gradient w.r.t. the depth of pixel q collects the four stencils that use
 // q, recomputed here (a gather, so no atomics).
-// Tiles of 32 x 8 pixels; a block strides over tiles in a fixed order.
-// Phase 0 stages D/O and O of the tile and a two-pixel ring in shared
-// memory; phase 1 evaluates the normal term once for every position of the
-// tile and its one-pixel edge ring (the four neighbours' stencils read it);
-// phase 2 forms each pixel's outputs, gathering the neighbours' gradients
-// w.r.t. its back-projected point from there.
-constexpr int kMapTW = 32, kMapTH = 8;
-constexpr int kMapRW = kMapTW + 2, kMapRH = kMapTH + 2;  // with the ring
-constexpr int kMapSW = kMapTW + 4, kMapSH = kMapTH + 4;  // with two rings
-struct MapSmem {
-  float dh[kMapSH][kMapSW];     // D / max(O, 1e-6); 0 outside the image
-  float op[kMapSH][kMapSW];     // O; 0 outside the image
-  float g[kMapRH][kMapRW][12];  // dL_n / dX of the four stencil points
-  float ln[kMapTH][kMapTW];     // L_n of the tile's own pixels
-  float gn[kMapTH][kMapTW][3];  // dL_n / dN_r of the tile's own pixels
-  bool ok[kMapRH][kMapRW];
+//
+// A warp takes a strip of 28 columns and R rows: a lane per column (two halo
+// columns on each side) loads the depths and opacities of R + 4 rows at once
+// and walks down them, keeping the normal term of the last two in registers;
+// left and right neighbours come by shuffles.  Nothing is staged in shared
+// memory and there is no block barrier.  Replaces 32 x 8 tiles with three
+// barrier-separated phases over two rings in shared memory, which took ~650
+// instructions a pixel (31 us at 1200x680, 197 us for eight such views, 7.9
+// us at 160x120).  R = 4: 24, 140 and 11.8 us; taller strips repeat fewer
+// halo rows but chain more latencies (R = 6: 21, 147, 14.5 us; R = 16: 45 us
+// at 1200x680); R = 2 where R = 4 would leave fewer than eight warps per SM
+// (160x120: 8.8 us).
+constexpr int kStripW = 28;        // output columns of a strip
+constexpr int kStripRows = 4;      // and rows
+constexpr int kStripRowsSmall = 2;
+constexpr int kLossWarps = kLossThreads / 32;
+
+__host__ __device__ inline int strips_along(int n, int step) { return (n + step - 1) / step; }
+inline int strip_rows(long long px) {
+  return px >= 8ll * 152 * kStripW * kStripRows ? kStripRows : kStripRowsSmall;
+}
+
+struct MapLossImages {
+  const float *rgb, *depth, *normal, *opac, *obs_rgb, *obs_depth;
+  float *g_rgb, *g_depth, *g_normal, *g_opac;
 };
 
-// Pixel ray (x', y', 1) of pixel (px, py) with the reciprocal focal lengths
-// (ifx, ify) = (1/fx, 1/fy) taken once per kernel.
-__device__ __forceinline__ F3 ray_of(const gs2d_camera& cam, float ifx, float ify, int px, int py) {
-  return f3((px + 0.5f - cam.cx) * ifx, (py + 0.5f - cam.cy) * ify, 1.f);
-}
-// Normal term at pixel (px, py), staged at (sx, sy) of the two-ring arrays:
-// returns L_n (false if invalid: border pixel, own or a 4-neighbour's
-// opacity <= 0.5, degenerate cross product) and the gradients of L_n w.r.t.
-// X(p+ex), X(p-ex), X(p+ey), X(p-ey) and N_r(p).
-__device__ bool ln_eval(const MapSmem& sm, const float* __restrict__ normal,
-                        const gs2d_camera& cam, float ifx, float ify, int px, int py, int sx,
-                        int sy, float& Ln, F3 g[4], F3& gNr) {
+// Gradients of the strip with first output pixel (x0, y0); returns the lane's
+// sum of the loss terms (unscaled).  (ifx, ify) = (1/fx, 1/fy), taken once
+// per kernel: the pixel ray is ((px + 0.5 - cx) ifx, (py + 0.5 - cy) ify, 1).
+template <int R>
+__device__ __forceinline__ float mapping_loss_strip(int x0, int y0,
+                                                    const MapLossImages& im,
+                                                    const gs2d_camera& cam, float ifx, float ify,
+                                                    float inv, float w_l1, float w_d, float w_n) {
   const int W = cam.width, H = cam.height;
-  if (px < 1 || py < 1 || px > W - 2 || py > H - 2) return false;
-  if (!(sm.op[sy][sx] > 0.5f && sm.op[sy][sx - 1] > 0.5f && sm.op[sy][sx + 1] > 0.5f &&
-        sm.op[sy - 1][sx] > 0.5f && sm.op[sy + 1][sx] > 0.5f))
-    return false;
-  const int i = py * W + px;
-  const F3 Xr = sm.dh[sy][sx + 1] * ray_of(cam, ifx, ify, px + 1, py);
-  const F3 Xl = sm.dh[sy][sx - 1] * ray_of(cam, ifx, ify, px - 1, py);
-  const F3 Xd = sm.dh[sy + 1][sx] * ray_of(cam, ifx, ify, px, py + 1);
-  const F3 Xu = sm.dh[sy - 1][sx] * ray_of(cam, ifx, ify, px, py - 1);
-  const F3 gx = 0.5f * (Xr - Xl), gy = 0.5f * (Xd - Xu);
-  const F3 n = cross3(gx, gy);
-  const float n2 = dot3(n, n);
-  if (!(n2 > 0.f)) return false;
-  const float inn = rsqrtf(n2);  // 1 / |n|
-  const F3 ND = inn * n;
-  const F3 Nr = f3(normal[3 * i], normal[3 * i + 1], normal[3 * i + 2]);
-  const float dp = dot3(ND, Nr);
-  Ln = 1.f - dp;
-  gNr = (-1.f) * ND;
-  // dLn/dn = -(Nr - ND (ND . Nr)) / |n|
-  const F3 gn = (-inn) * (Nr - dp * ND);
-  const F3 ggx = cross3(gy, gn), ggy = cross3(gn, gx);
-  g[0] = 0.5f * ggx;
-  g[1] = (-0.5f) * ggx;
-  g[2] = 0.5f * ggy;
-  g[3] = (-0.5f) * ggy;
-  return true;
-}
-
-// One 32 x 8 tile of the mapping loss at (x0, y0): gradients written for
-// its pixels, this thread's pixel's loss terms added to acc (unscaled).
-__device__ __forceinline__ void mapping_loss_tile(
-    MapSmem& sm, int x0, int y0, const float* __restrict__ rgb, const float* __restrict__ depth,
-    const float* __restrict__ normal, const float* __restrict__ opac,
-    const float* __restrict__ obs_rgb, const float* __restrict__ obs_depth,
-    const gs2d_camera& cam, float ifx, float ify, float inv, float w_l1, float w_d, float w_n,
-    float* __restrict__ g_rgb, float* __restrict__ g_depth, float* __restrict__ g_normal,
-    float* __restrict__ g_opac, float& acc) {
-  const int W = cam.width, H = cam.height;
-  __syncthreads();
-  // phase 0: D/O and O on the tile and two rings
-  for (int e = threadIdx.x; e < kMapSW * kMapSH; e += blockDim.x) {
-    const int sy = e / kMapSW, sx = e % kMapSW;
-    const int px = x0 + sx - 2, py = y0 + sy - 2;
-    float d = 0.f, o = 0.f;
-    if (px >= 0 && py >= 0 && px < W && py < H) {
-      const int i = py * W + px;
-      o = opac[i];
-      d = depth[i] / fmaxf(o, 1e-6f);
+  const int lane = threadIdx.x & 31;
+  const int px = x0 + lane - 2;
+  const bool in_x = px >= 0 && px < W;
+  const bool out_x = lane >= 2 && lane < 2 + kStripW && px < W;
+  const float rxl = ((px - 1) + 0.5f - cam.cx) * ifx, rxc = (px + 0.5f - cam.cx) * ifx,
+              rxr = ((px + 1) + 0.5f - cam.cx) * ifx;
+  // D / max(O, 1e-6), O and D of rows y0 - 2 .. y0 + R + 1 (0 outside
+  // the image)
+  constexpr int kR = R + 4;
+  float dv[kR], ov[kR], Dv[kR];
+#pragma unroll
+  for (int k = 0; k < kR; ++k) {
+    const int y = y0 - 2 + k;
+    ov[k] = Dv[k] = 0.f;
+    if (in_x && y >= 0 && y < H) {
+      const int i = y * W + px;
+      ov[k] = __ldg(im.opac + i);
+      Dv[k] = __ldg(im.depth + i);
     }
-    sm.dh[sy][sx] = d;
-    sm.op[sy][sx] = o;
   }
-  __syncthreads();
-  // phase 1: the normal term on the tile and its ring
-  for (int e = threadIdx.x; e < kMapRW * kMapRH; e += blockDim.x) {
-    const int ry = e / kMapRW, rx = e % kMapRW;
-    const int px = x0 + rx - 1, py = y0 + ry - 1;
-    const bool tile_px = rx >= 1 && rx <= kMapTW && ry >= 1 && ry <= kMapTH;
-    const bool ring = !tile_px && !((rx == 0 || rx == kMapRW - 1) && (ry == 0 || ry == kMapRH - 1));
-    float Ln = 0.f;
-    F3 g4[4], gNr = f3(0.f, 0.f, 0.f);
+#pragma unroll
+  for (int k = 0; k < kR; ++k) dv[k] = Dv[k] / fmaxf(ov[k], 1e-6f);
+  // row q = e - 1: its normal term, dL_n / dN_r and dL_n / dX from its left
+  // and right stencils; and the vertical part of row q - 1
+  bool ok_q = false, ok_u = false;
+  float ln_q = 0.f;
+  F3 gn_q = f3(0.f, 0.f, 0.f), hx_q = gn_q, gy_q = gn_q, gy_u = gn_q;
+  float acc = 0.f;
+#pragma unroll
+  for (int k = 1; k < kR - 1; ++k) {
+    const int e = y0 - 2 + k;
+    const float du = dv[k - 1], dc = dv[k], dd = dv[k + 1];   // rows e - 1, e, e + 1
+    const float ou = ov[k - 1], oc = ov[k], od = ov[k + 1];
+    // the normal term at (px, e): false if invalid (border pixel, own or a
+    // 4-neighbour's opacity <= 0.5, degenerate cross product)
+    const float dl = __shfl_up_sync(0xffffffffu, dc, 1), dr = __shfl_down_sync(0xffffffffu, dc, 1);
+    const float ol = __shfl_up_sync(0xffffffffu, oc, 1), orr = __shfl_down_sync(0xffffffffu, oc, 1);
     bool ok = false;
-    if ((tile_px || ring) && px >= 0 && py >= 0 && px < W && py < H)
-      ok = ln_eval(sm, normal, cam, ifx, ify, px, py, rx + 1, ry + 1, Ln, g4, gNr);
-    sm.ok[ry][rx] = ok;
-    if (ok)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        sm.g[ry][rx][3 * k] = g4[k].x;
-        sm.g[ry][rx][3 * k + 1] = g4[k].y;
-        sm.g[ry][rx][3 * k + 2] = g4[k].z;
+    float Ln = 0.f;
+    F3 gNr = f3(0.f, 0.f, 0.f), ggx = gNr, ggy = gNr;
+    if (lane >= 1 && lane <= 30 && px >= 1 && e >= 1 && px <= W - 2 && e <= H - 2 && oc > 0.5f &&
+        ol > 0.5f && orr > 0.5f && ou > 0.5f && od > 0.5f) {
+      const int i = e * W + px;
+      const float ryu = ((e - 1) + 0.5f - cam.cy) * ify, ryc = (e + 0.5f - cam.cy) * ify,
+                  ryd = ((e + 1) + 0.5f - cam.cy) * ify;
+      const F3 Xr = dr * f3(rxr, ryc, 1.f), Xl = dl * f3(rxl, ryc, 1.f);
+      const F3 Xd = dd * f3(rxc, ryd, 1.f), Xu = du * f3(rxc, ryu, 1.f);
+      const F3 gx = 0.5f * (Xr - Xl), gy = 0.5f * (Xd - Xu);
+      const F3 n = cross3(gx, gy);
+      const float n2 = dot3(n, n);
+      if (n2 > 0.f) {
+        ok = true;
+        const float inn = rsqrtf(n2);  // 1 / |n|
+        const F3 ND = inn * n;
+        const F3 Nr = f3(__ldg(im.normal + 3 * i), __ldg(im.normal + 3 * i + 1),
+                         __ldg(im.normal + 3 * i + 2));
+        const float dp = dot3(ND, Nr);
+        Ln = 1.f - dp;
+        gNr = (-1.f) * ND;
+        // dLn/dn = -(Nr - ND (ND . Nr)) / |n|
+        const F3 gn = (-inn) * (Nr - dp * ND);
+        // dL_n / dX(p + ex) = 0.5 ggx, of X(p - ex) the negative; ggy alike
+        ggx = cross3(gy, gn);
+        ggy = cross3(gn, gx);
       }
-    if (tile_px) {
-      sm.ln[ry - 1][rx - 1] = ok ? Ln : 0.f;
-      sm.gn[ry - 1][rx - 1][0] = ok ? gNr.x : 0.f;
-      sm.gn[ry - 1][rx - 1][1] = ok ? gNr.y : 0.f;
-      sm.gn[ry - 1][rx - 1][2] = ok ? gNr.z : 0.f;
     }
-  }
-  __syncthreads();
-  // phase 2: one pixel per thread
-  const int lx = threadIdx.x % kMapTW, ly = threadIdx.x / kMapTW;
-  const int px = x0 + lx, py = y0 + ly;
-  if (px < W && py < H) {
-    const int i = py * W + px;
-    const float O = sm.op[ly + 2][lx + 2];
-    const float Oc = fmaxf(O, 1e-6f);
-    const float D = depth[i];
-    const float Dh = sm.dh[ly + 2][lx + 2];
-    const float d0 = rgb[3 * i] - obs_rgb[3 * i];
-    const float d1 = rgb[3 * i + 1] - obs_rgb[3 * i + 1];
-    const float d2 = rgb[3 * i + 2] - obs_rgb[3 * i + 2];
-    const float dd = Dh - obs_depth[i];
-    acc += w_l1 * (fabsf(d0) + fabsf(d1) + fabsf(d2)) + w_d * fabsf(dd);
-    const float sl = w_l1 * inv;
-    g_rgb[3 * i] = sgnf(d0) * sl;
-    g_rgb[3 * i + 1] = sgnf(d1) * sl;
-    g_rgb[3 * i + 2] = sgnf(d2) * sl;
-    float gDh = w_d * sgnf(dd) * inv;
-    // own normal term
-    const int ry = ly + 1, rx = lx + 1;
-    if (sm.ok[ry][rx]) acc += w_n * sm.ln[ly][lx];
-    const float sn = w_n * inv;
-    g_normal[3 * i] = sn * sm.gn[ly][lx][0];
-    g_normal[3 * i + 1] = sn * sm.gn[ly][lx][1];
-    g_normal[3 * i + 2] = sn * sm.gn[ly][lx][2];
-    // stencils of the four neighbours that read X(q): p = q-ex uses X(p+ex)
-    // (slot 0), p = q+ex uses X(p-ex) (1), p = q-ey uses X(p+ey) (2),
-    // p = q+ey uses X(p-ey) (3)
-    const F3 rq = ray_of(cam, ifx, ify, px, py);
-    const int nb[4][3] = {{rx - 1, ry, 0}, {rx + 1, ry, 1}, {rx, ry - 1, 2}, {rx, ry + 1, 3}};
-    F3 gX = f3(0.f, 0.f, 0.f);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int qx = nb[k][0], qy = nb[k][1], sl2 = nb[k][2];
-      if (sm.ok[qy][qx])
-        gX = gX + f3(sm.g[qy][qx][3 * sl2], sm.g[qy][qx][3 * sl2 + 1], sm.g[qy][qx][3 * sl2 + 2]);
+    // dL_n / dX(px, e) from the stencils of the left (uses X(p + ex)) and
+    // right (X(p - ex)) neighbours
+    const bool okl = __shfl_up_sync(0xffffffffu, (int)ok, 1) != 0;
+    const bool okr = __shfl_down_sync(0xffffffffu, (int)ok, 1) != 0;
+    const F3 gl = f3(__shfl_up_sync(0xffffffffu, ggx.x, 1), __shfl_up_sync(0xffffffffu, ggx.y, 1),
+                     __shfl_up_sync(0xffffffffu, ggx.z, 1));
+    const F3 gr = f3(__shfl_down_sync(0xffffffffu, ggx.x, 1),
+                     __shfl_down_sync(0xffffffffu, ggx.y, 1),
+                     __shfl_down_sync(0xffffffffu, ggx.z, 1));
+    F3 hx = f3(0.f, 0.f, 0.f);
+    if (okl) hx = hx + 0.5f * gl;
+    if (okr) hx = hx + (-0.5f) * gr;
+    const int q = e - 1;
+    if (k >= 3 && q < H && out_x) {
+      const int i = q * W + px;
+      const float O = ou, Dh = du;
+      const float Oc = fmaxf(O, 1e-6f);
+      const float D = Dv[k - 1];
+      const float d0 = __ldg(im.rgb + 3 * i) - __ldg(im.obs_rgb + 3 * i);
+      const float d1 = __ldg(im.rgb + 3 * i + 1) - __ldg(im.obs_rgb + 3 * i + 1);
+      const float d2 = __ldg(im.rgb + 3 * i + 2) - __ldg(im.obs_rgb + 3 * i + 2);
+      const float ddp = Dh - __ldg(im.obs_depth + i);
+      acc += w_l1 * (fabsf(d0) + fabsf(d1) + fabsf(d2)) + w_d * fabsf(ddp);
+      const float sl = w_l1 * inv;
+      im.g_rgb[3 * i] = sgnf(d0) * sl;
+      im.g_rgb[3 * i + 1] = sgnf(d1) * sl;
+      im.g_rgb[3 * i + 2] = sgnf(d2) * sl;
+      float gDh = w_d * sgnf(ddp) * inv;
+      // own normal term
+      if (ok_q) acc += w_n * ln_q;
+      const float sn = w_n * inv;
+      im.g_normal[3 * i] = sn * gn_q.x;
+      im.g_normal[3 * i + 1] = sn * gn_q.y;
+      im.g_normal[3 * i + 2] = sn * gn_q.z;
+      // and the stencils above (uses X(p + ey)) and below (X(p - ey))
+      F3 gX = hx_q;
+      if (ok_u) gX = gX + 0.5f * gy_u;
+      if (ok) gX = gX + (-0.5f) * ggy;
+      const F3 rq = f3(rxc, (q + 0.5f - cam.cy) * ify, 1.f);
+      gDh += w_n * inv * dot3(gX, rq);
+      im.g_depth[i] = gDh / Oc;
+      im.g_opac[i] = O > 1e-6f ? -gDh * D / (O * O) : 0.f;
     }
-    gDh += w_n * inv * dot3(gX, rq);
-    g_depth[i] = gDh / Oc;
-    g_opac[i] = O > 1e-6f ? -gDh * D / (O * O) : 0.f;
+    ok_u = ok_q;
+    gy_u = gy_q;
+    ok_q = ok;
+    ln_q = Ln;
+    gn_q = gNr;
+    hx_q = hx;
+    gy_q = ggy;
   }
+  return acc;
 }
 
-__global__ void __launch_bounds__(kLossThreads) mapping_loss_kernel(
-    const float* __restrict__ rgb, const float* __restrict__ depth, const float* __restrict__ normal,
-    const float* __restrict__ opac, const float* __restrict__ obs_rgb,
-    const float* __restrict__ obs_depth, gs2d_camera cam, float w_l1, float w_d, float w_n,
-    float* __restrict__ g_rgb, float* __restrict__ g_depth, float* __restrict__ g_normal,
-    float* __restrict__ g_opac, float* __restrict__ part) {
-  __shared__ float s[kLossThreads / 32];
-  __shared__ MapSmem sm;
-  const int W = cam.width, H = cam.height, P = W * H;
-  const float inv = 1.f / (float)P;
-  const int tiles_x = (W + kMapTW - 1) / kMapTW, tiles_y = (H + kMapTH - 1) / kMapTH;
+template <int R>
+__global__ void __launch_bounds__(kLossThreads, 4) mapping_loss_kernel(
+    MapLossImages im, gs2d_camera cam, float w_l1, float w_d, float w_n,
+    float* __restrict__ part) {
+  __shared__ float s[kLossWarps];
+  const int strips_x = strips_along(cam.width, kStripW);
+  const int n = strips_x * strips_along(cam.height, R);
+  const float inv = 1.f / (float)(cam.width * cam.height);
   const float ifx = 1.f / cam.fx, ify = 1.f / cam.fy;
   float acc = 0.f;
-  for (int tile = blockIdx.x; tile < tiles_x * tiles_y; tile += gridDim.x)
-    mapping_loss_tile(sm, (tile % tiles_x) * kMapTW, (tile / tiles_x) * kMapTH, rgb, depth, normal,
-                      opac, obs_rgb, obs_depth, cam, ifx, ify, inv, w_l1, w_d, w_n, g_rgb,
-                      g_depth, g_normal, g_opac, acc);
+  for (int k = blockIdx.x * kLossWarps + (threadIdx.x >> 5); k < n; k += gridDim.x * kLossWarps)
+    acc += mapping_loss_strip<R>((k % strips_x) * kStripW, (k / strips_x) * R, im, cam, ifx,
+                              ify, inv, w_l1, w_d, w_n);
   const float t = block_sum256(acc, s);
   if (threadIdx.x == 0) part[blockIdx.x] = t * inv;
 }
 
 // The mapping loss of many views in one launch: work items are the views'
-// 32 x 8 tiles in view order; each tile's loss terms are summed per warp
-// into part[item * 8 + warp] (no block barrier beyond the tile's own), and
-// mapping_loss_batch_sum_kernel adds each view's items in order.
+// strips in view order; each strip's loss terms are summed over its warp
+// into part[item], and mapping_loss_batch_sum_kernel adds each view's items
+// in order.
 struct LossViewDev {
   gs2d_camera cam;
-  const float *rgb, *depth, *normal, *opac, *obs_rgb, *obs_depth;
-  float *g_rgb, *g_depth, *g_normal, *g_opac;
-  int tiles_x, item0, n_items;
+  MapLossImages im;
+  int strips_x, item0, n_items;
 };
 struct LossTable {
   int n_views, n_items;
   LossViewDev v[GS2D_MAX_VIEWS];
 };
-constexpr int kLossWarps = kLossThreads / 32;
 
-__global__ void __launch_bounds__(kLossThreads) mapping_loss_batch_kernel(const LossTable tab,
-                                                                          float w_d, float w_n,
-                                                                          float* __restrict__ part) {
-  __shared__ MapSmem sm;
-  for (int item = blockIdx.x; item < tab.n_items; item += gridDim.x) {
+template <int R>
+__global__ void __launch_bounds__(kLossThreads, 4) mapping_loss_batch_kernel(
+    const LossTable tab, float w_d, float w_n, float* __restrict__ part) {
+  for (int item = blockIdx.x * kLossWarps + (threadIdx.x >> 5); item < tab.n_items;
+       item += gridDim.x * kLossWarps) {
     int v = 0;
     while (v + 1 < tab.n_views && item >= tab.v[v + 1].item0) ++v;
     const LossViewDev& V = tab.v[v];
-    const int tile = item - V.item0;
+    const int k = item - V.item0;
     const float inv = 1.f / (float)(V.cam.width * V.cam.height);
-    float acc = 0.f;
-    mapping_loss_tile(sm, (tile % V.tiles_x) * kMapTW, (tile / V.tiles_x) * kMapTH, V.rgb, V.depth,
-                      V.normal, V.opac, V.obs_rgb, V.obs_depth, V.cam, 1.f / V.cam.fx,
-                      1.f / V.cam.fy, inv, 1.f, w_d, w_n, V.g_rgb, V.g_depth, V.g_normal, V.g_opac,
-                      acc);
+    float acc = mapping_loss_strip<R>((k % V.strips_x) * kStripW, (k / V.strips_x) * R, V.im,
+                                   V.cam, 1.f / V.cam.fx, 1.f / V.cam.fy, inv, 1.f, w_d, w_n);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if ((threadIdx.x & 31) == 0) part[(size_t)item * kLossWarps + (threadIdx.x >> 5)] = acc;
+    if ((threadIdx.x & 31) == 0) part[item] = acc;
   }
 }
 
-// loss_out[v] = inv_v x the sum of view v's per-warp partials: thread t adds
+// loss_out[v] = inv_v x the sum of view v's strip partials: thread t adds
 // entries t, t + 256, ... in order, then a fixed tree over the threads.
 __global__ void __launch_bounds__(256) mapping_loss_batch_sum_kernel(const LossTable tab,
                                                                      const float* __restrict__ part,
                                                                      float* __restrict__ loss_out) {
   __shared__ float s[256];
   const LossViewDev& V = tab.v[blockIdx.x];
-  const float* p = part + (size_t)V.item0 * kLossWarps;
-  const int n = V.n_items * kLossWarps;
+  const float* p = part + V.item0;
+  const int n = V.n_items;
   float a = 0.f;
 #pragma unroll 8
   for (int e = threadIdx.x; e < n; e += 256) a += p[e];
@@ -361,9 +352,10 @@ size_t gs2d_mapping_loss_batch_workspace(const gs2d_loss_view* views, int n_view
   for (int v = 0; v < n_views; ++v) {
     const gs2d_camera& c = views[v].cam;
     if (c.width <= 0 || c.height <= 0) return 0;
-    items += (size_t)((c.width + kMapTW - 1) / kMapTW) * ((c.height + kMapTH - 1) / kMapTH);
+    // sized for the smaller strips
+    items += (size_t)strips_along(c.width, kStripW) * strips_along(c.height, kStripRowsSmall);
   }
-  return align_up(items * kLossWarps * sizeof(float), 256);
+  return align_up(items * sizeof(float), 256);
 }
 
 int gs2d_mapping_loss_batch(const gs2d_loss_view* views, int n_views, float w_d, float w_n,
@@ -372,7 +364,9 @@ int gs2d_mapping_loss_batch(const gs2d_loss_view* views, int n_views, float w_d,
   if (!views || n_views <= 0 || n_views > GS2D_MAX_VIEWS || !loss_out) return GS2D_ERR_INVALID_ARG;
   LossTable tab;
   tab.n_views = n_views;
-  long long items = 0;
+  long long items = 0, px = 0;
+  for (int v = 0; v < n_views; ++v) px += (long long)views[v].cam.width * views[v].cam.height;
+  const int rows = strip_rows(px);
   for (int v = 0; v < n_views; ++v) {
     const gs2d_loss_view& x = views[v];
     if (!x.rgb || !x.depth || !x.normal || !x.opacity || !x.obs_rgb || !x.obs_depth || !x.g_rgb ||
@@ -381,20 +375,13 @@ int gs2d_mapping_loss_batch(const gs2d_loss_view* views, int n_views, float w_d,
     if (x.cam.width <= 0 || x.cam.height <= 0) return GS2D_ERR_INVALID_ARG;
     LossViewDev& d = tab.v[v];
     d.cam = x.cam;
-    d.rgb = x.rgb;
-    d.depth = x.depth;
-    d.normal = x.normal;
-    d.opac = x.opacity;
-    d.obs_rgb = x.obs_rgb;
-    d.obs_depth = x.obs_depth;
-    d.g_rgb = x.g_rgb;
-    d.g_depth = x.g_depth;
-    d.g_normal = x.g_normal;
-    d.g_opac = x.g_opacity;
-    d.tiles_x = (x.cam.width + kMapTW - 1) / kMapTW;
+    d.im = MapLossImages{x.rgb,     x.depth, x.normal,  x.opacity,  x.obs_rgb,
+                         x.obs_depth, x.g_rgb, x.g_depth, x.g_normal, x.g_opacity};
+    d.strips_x = strips_along(x.cam.width, kStripW);
     d.item0 = (int)items;
-    d.n_items = d.tiles_x * ((x.cam.height + kMapTH - 1) / kMapTH);
-    items += d.n_items;
+    const long long mine = (long long)d.strips_x * strips_along(x.cam.height, rows);
+    d.n_items = (int)mine;
+    items += mine;
     if (items > 0x7FFFFFFF / kLossWarps) return GS2D_ERR_INVALID_ARG;
   }
   tab.n_items = (int)items;
@@ -410,14 +397,15 @@ int gs2d_mapping_loss_batch(const gs2d_loss_view* views, int n_views, float w_d,
   GS2D_CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return GS2D_ERR_CUDA;
   if (!slots[dev]) {
-    int per_sm = 0, sms = 0;
-    GS2D_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mapping_loss_batch_kernel,
-                                                                kLossThreads, 0));
+    int sms = 0;
     GS2D_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    slots[dev] = max(1, per_sm) * max(1, sms);
+    slots[dev] = 4 * max(1, sms);   // the launch bounds' blocks per SM
   }
-  mapping_loss_batch_kernel<<<min(slots[dev], tab.n_items), kLossThreads, 0, st>>>(tab, w_d, w_n,
-                                                                                  part);
+  const int blocks = min(slots[dev], strips_along(tab.n_items, kLossWarps));
+  if (rows == kStripRows)
+    mapping_loss_batch_kernel<kStripRows><<<blocks, kLossThreads, 0, st>>>(tab, w_d, w_n, part);
+  else
+    mapping_loss_batch_kernel<kStripRowsSmall><<<blocks, kLossThreads, 0, st>>>(tab, w_d, w_n, part);
   GS2D_LAUNCH_CHECK();
   mapping_loss_batch_sum_kernel<<<n_views, 256, 0, st>>>(tab, part, loss_out);
   GS2D_LAUNCH_CHECK();
@@ -446,11 +434,19 @@ int gs2d_mapping_loss_ssim(const float* rgb, const float* depth, const float* no
   if (!workspace || ws_bytes < need) return GS2D_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   float* part = static_cast<float*>(workspace);
-  mapping_loss_kernel<<<kLossBlocks, kLossThreads, 0, st>>>(
-      rgb, depth, normal, opacity, obs_rgb, obs_depth, *cam, 1.f - w_ssim, w_d, w_n, g_rgb,
-      g_depth, g_normal, g_opacity, part);
+  const int rows = strip_rows((long long)cam->width * cam->height);
+  const int strips = strips_along(cam->width, kStripW) * strips_along(cam->height, rows);
+  const int blocks = min(kLossBlocks, strips_along(strips, kLossWarps));
+  const MapLossImages im{rgb,     depth, normal,  opacity,  obs_rgb,
+                         obs_depth, g_rgb, g_depth, g_normal, g_opacity};
+  if (rows == kStripRows)
+    mapping_loss_kernel<kStripRows><<<blocks, kLossThreads, 0, st>>>(im, *cam, 1.f - w_ssim, w_d,
+                                                                     w_n, part);
+  else
+    mapping_loss_kernel<kStripRowsSmall><<<blocks, kLossThreads, 0, st>>>(im, *cam, 1.f - w_ssim,
+                                                                          w_d, w_n, part);
   GS2D_LAUNCH_CHECK();
-  sum_parts_kernel<<<1, 256, 0, st>>>(part, kLossBlocks, loss_out, nullptr);
+  sum_parts_kernel<<<1, 256, 0, st>>>(part, blocks, loss_out, nullptr);
   GS2D_LAUNCH_CHECK();
   if (w_ssim > 0.f)
     return ssim_launch(rgb, obs_rgb, cam->height, cam->width, w_ssim, g_rgb, loss_out,

@@ -23,15 +23,28 @@
 // (the window is symmetric, so the adjoint filter is the same filter).
 //
 // One block per 32 x 32 output tile and channel.  It stages x and y on the
-// tile plus a 10-pixel ring in shared memory, filters the five moment maps
-// separably (rows, then columns) on the tile plus a 5-pixel ring, evaluates
+// tile plus a 10-pixel ring in shared memory and filters the five moment maps
+// separably on the tile plus a 5-pixel ring (columns, then rows), evaluates
 // S and the three G maps there (zero outside the image), filters those
-// separably down to the tile and writes the gradient.  Everything between
-// the image reads and the gradient write stays in shared memory: per pixel
-// and channel the kernel reads x and y and adds one gradient value.  The
-// per-block loss sums are reduced in a fixed order (deterministic).
+// separably down to the tile (rows, then columns) and writes the gradient.
+// Everything between the image reads and the gradient write stays in shared
+// memory: per pixel and channel the kernel reads x and y and adds one
+// gradient value.  The per-block loss sums are reduced in a fixed order
+// (deterministic).
+//
+// The kernel is bound by its FP32 issue, so every filter runs on pairs
+// (fma.rn.f32x2, two values per instruction): a column filter takes adjacent
+// columns, which lie side by side in a row-major map; its results are stored
+// transposed, so that the row filter that follows finds adjacent rows side by
+// side.  A thread forms four outputs along the filter from one pass over
+// their fourteen taps, and the products x^2, y^2, d^2 once per tap instead of
+// once per tap and output.  Six outputs per thread in 192 threads left too
+// few warps to cover the phases' barriers.  1200x680, three channels: 81 us
+// with one value per instruction, 72 us with pairs in 192 threads, 68 us
+// so.
 #include <cmath>
 
+#include "f32x2.cuh"
 #include "gs2d_common.cuh"
 #include "gs2d_internal.h"
 
@@ -41,206 +54,242 @@ constexpr int kSsimT = 32;                 // output tile edge
 constexpr int kSsimR = 5;                  // window radius
 constexpr int kSsimA = kSsimT + 4 * kSsimR;  // 52: staged edge (two rings)
 constexpr int kSsimB = kSsimT + 2 * kSsimR;  // 42: moment / G map edge
-constexpr int kSsimThreads = 256;
+constexpr int kSsimThreads = 288;
 constexpr float kSsimC1 = 0.0001f, kSsimC2 = 0.0009f;
 
 struct SsimWin {
   float g[2 * kSsimR + 1];  // normalised 1D Gaussian; the window is g g^T
 };
 
-// Shared memory (floats).  Region A: x and y (2 x 52 x 52, rows of 52), later
-// the three G maps (3 x 42 rows of 44).  Region B: the five row-filtered
-// moment maps (5 x 52 rows of 44), later the three row-filtered G maps
-// (3 x 42 rows of 32).  Row strides are multiples of 4 floats so a thread
-// reads 16 consecutive taps as four float4; each region has a little slack
-// for the taps past the last row that only padding outputs use.
-constexpr int kSsimBP = 44;                       // padded row of the 42-wide maps
-constexpr int kSsimSmemA = 3 * kSsimB * kSsimBP + 16;
-constexpr int kSsimSmemB = 5 * kSsimA * kSsimBP + 2 * kSsimBP + 16;
+// Shared memory (floats).  Region A: x and y (2 x 52 rows of 52), later the
+// three G maps, transposed (3 x 42 columns of 46 rows).  Region B: the five
+// column-filtered moment maps, transposed (5 x 52 columns of 46 rows), later
+// the three row-filtered G maps (3 x 42 rows of 36).  Pitches are even (pairs
+// of floats are read) and spread a warp's stores over the banks (two-way
+// conflicts at most).
+constexpr int kSsimBP = 46;                       // pitch of the 42-row transposed maps
+constexpr int kSsimFP = 36;                       // pitch of the 32-column filtered G maps
+constexpr int kSsimSmemA = 3 * kSsimB * kSsimBP;
+// two columns of slack: the last group of a filter reads past the 52 columns
+// (rows) for outputs beyond the 42, which are dropped
+constexpr int kSsimSmemB = (5 * kSsimA + 2) * kSsimBP;
 constexpr size_t kSsimSmemBytes = (size_t)(kSsimSmemA + kSsimSmemB) * sizeof(float);
-static_assert(2 * kSsimA * kSsimA + 16 <= kSsimSmemA, "x and y fit region A");
-static_assert(3 * kSsimB * kSsimT <= kSsimSmemB, "filtered G maps fit region B");
-constexpr int kSsimRB = 4;                        // outputs per thread along a row or column
+static_assert((2 * kSsimA + 2) * kSsimA <= kSsimSmemA, "x, y and two rows of slack fit region A");
+static_assert(3 * kSsimB * kSsimFP <= kSsimSmemB, "filtered G maps fit region B");
+static_assert(kSsimSmemA % 4 == 0 && kSsimFP % 4 == 0, "16-byte stores");
+constexpr int kSsimM = 4;                         // outputs per thread of a filter
+constexpr int kSsimGM = (kSsimB + kSsimM - 1) / kSsimM;   // 11 groups of the moment filters
+constexpr int kSsimGG = kSsimT / kSsimM;                  // 8 groups of the G row filter
+constexpr int kSsimC = 2;                         // outputs per thread of the last filter
+constexpr int kSsimTaps = 2 * kSsimR + 1;
 
-__device__ __forceinline__ void load16(const float* p, float (&v)[16]) {
-  const float4* q = reinterpret_cast<const float4*>(p);
+// acc[o] += sum over taps t of w_t v[o + t], fed one value at a time: i is
+// the index of v (taps i - o of the outputs it reaches).
+template <int kOut, int kMaps>
+__device__ __forceinline__ void filter_tap(const F2 (&w)[kSsimR + 1], const F2 (&v)[kMaps], int i,
+                                           F2 (&acc)[kMaps][kOut]) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float4 t = q[i];
-    v[4 * i] = t.x;
-    v[4 * i + 1] = t.y;
-    v[4 * i + 2] = t.z;
-    v[4 * i + 3] = t.w;
+  for (int o = 0; o < kOut; ++o) {
+    const int t = i - o;
+    if (t < 0 || t >= kSsimTaps) continue;
+    const F2 g = w[t <= kSsimR ? t : 2 * kSsimR - t];
+#pragma unroll
+    for (int k = 0; k < kMaps; ++k) acc[k][o] = fma2(g, v[k], acc[k][o]);
   }
 }
 
-__global__ void __launch_bounds__(kSsimThreads) ssim_kernel(const float* __restrict__ x,
+__global__ void __launch_bounds__(kSsimThreads, 3) ssim_kernel(const float* __restrict__ x,
                                                            const float* __restrict__ y, int H,
                                                            int W, float weight, SsimWin win,
                                                            float* __restrict__ g_x,
                                                            float* __restrict__ part) {
   extern __shared__ float4 smem4[];
-  float* sa = reinterpret_cast<float*>(smem4);    // x, y [52][52]  ->  G [3][42][44]
-  float* sb = sa + kSsimSmemA;                    // M [5][52][44]  ->  F [3][42][32]
+  float* sa = reinterpret_cast<float*>(smem4);    // x, y [52][52]  ->  G [3][42 q][46 r]
+  float* sb = sa + kSsimSmemA;                    // M [5][52 q][46 r]  ->  F [3][42 r][36 q]
   __shared__ float s_red[kSsimThreads / 32];
   const int c = blockIdx.z;
   const int tx0 = blockIdx.x * kSsimT, ty0 = blockIdx.y * kSsimT;
   const int ax0 = tx0 - 2 * kSsimR, ay0 = ty0 - 2 * kSsimR;   // staged origin
-  // stage x, y (zero outside the image) and clear the slack; unrolled so
-  // that several loads of each thread are in flight
-#pragma unroll 4
-  for (int e = threadIdx.x; e < kSsimA * kSsimA; e += kSsimThreads) {
-    const int r = e / kSsimA, q = e % kSsimA;
-    const int py = ay0 + r, px = ax0 + q;
-    float vx = 0.f, vy = 0.f;
-    if (px >= 0 && py >= 0 && px < W && py < H) {
-      const size_t i = ((size_t)py * W + px) * 3 + c;
-      vx = x[i];
-      vy = y[i];
-    }
-    sa[e] = vx;
-    sa[kSsimA * kSsimA + e] = vy;
-  }
-  if (threadIdx.x < 16) sa[2 * kSsimA * kSsimA + threadIdx.x] = 0.f;
-  __syncthreads();
-  // row filter of the five moments (x, d = x - y, x^2, y^2, d^2): outputs
-  // M[k][r][q0 .. q0 + 3], r in [0, 52), q0 = 4 g, g in [0, 11)
-  constexpr int kG1 = (kSsimB + kSsimRB - 1) / kSsimRB;   // 11 groups along a row
-  for (int e = threadIdx.x; e < kSsimA * kG1; e += kSsimThreads) {
-    const int r = e / kG1, q0 = (e % kG1) * kSsimRB;
-    float xa[16], ya[16];
-    load16(sa + r * kSsimA + q0, xa);
-    load16(sa + kSsimA * kSsimA + r * kSsimA + q0, ya);
-    float m[5][kSsimRB];
+  F2 w[kSsimR + 1];
 #pragma unroll
-    for (int o = 0; o < kSsimRB; ++o) {
-      float mx = 0.f, md = 0.f, exx = 0.f, eyy = 0.f, edd = 0.f;
-#pragma unroll
-      for (int t = 0; t <= 2 * kSsimR; ++t) {
-        const float a = xa[o + t], b = ya[o + t], w = win.g[t];
-        const float d = a - b;
-        const float wa = w * a, wb = w * b, wd = w * d;
-        mx += wa;
-        md += wd;
-        exx = fmaf(wa, a, exx);
-        eyy = fmaf(wb, b, eyy);
-        edd = fmaf(wd, d, edd);
+  for (int t = 0; t <= kSsimR; ++t) w[t] = dup2(win.g[t]);
+  // stage x, y (zero outside the image), a warp per row: the lanes' columns
+  // and offsets are the same in every row
+  {
+    constexpr int kW = kSsimThreads / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int qa = lane, qb = lane + 32;
+    const bool ia = ax0 + qa >= 0 && ax0 + qa < W;
+    const bool ib = qb < kSsimA && ax0 + qb >= 0 && ax0 + qb < W;
+    const float* px = x + ((ptrdiff_t)ay0 * W + ax0 + qa) * 3 + c;
+    const float* py = y + ((ptrdiff_t)ay0 * W + ax0 + qa) * 3 + c;
+#pragma unroll 3
+    for (int r = warp; r < kSsimA; r += kW) {
+      const bool in = ay0 + r >= 0 && ay0 + r < H;
+      const ptrdiff_t o = (ptrdiff_t)r * W * 3;
+      const float xa = in && ia ? __ldg(px + o) : 0.f, ya = in && ia ? __ldg(py + o) : 0.f;
+      const float xb = in && ib ? __ldg(px + o + 96) : 0.f, yb = in && ib ? __ldg(py + o + 96) : 0.f;
+      float* d = sa + r * kSsimA + qa;
+      d[0] = xa;
+      d[kSsimA * kSsimA] = ya;
+      if (qb < kSsimA) {
+        d[32] = xb;
+        d[kSsimA * kSsimA + 32] = yb;
       }
-      m[0][o] = mx;
-      m[1][o] = md;
-      m[2][o] = exx;
-      m[3][o] = eyy;
-      m[4][o] = edd;
     }
+  }
+  __syncthreads();
+  // column filter of the five moments (x, d = x - y, x^2, y^2, d^2) of the
+  // columns 2 p, 2 p + 1: M[k][q][r0 .. r0 + 3] (rows 42, 43 land in the padding)
+  for (int e = threadIdx.x; e < (kSsimA / 2) * kSsimGM; e += kSsimThreads) {
+    const int p = e % (kSsimA / 2), r0 = (e / (kSsimA / 2)) * kSsimM;
+    const float* sx = sa + r0 * kSsimA + 2 * p;
+    const float* sy = sx + kSsimA * kSsimA;
+    F2 acc[5][kSsimM];
 #pragma unroll
     for (int k = 0; k < 5; ++k)
-      *reinterpret_cast<float4*>(sb + (k * kSsimA + r) * kSsimBP + q0) =
-          make_float4(m[k][0], m[k][1], m[k][2], m[k][3]);
-  }
-  __syncthreads();
-  // column filter, S and the G maps on the 42 x 42 region (origin tile - 5):
-  // rows r0 .. r0 + 3 of column q per thread; x and y are dead, so the G
-  // maps take region A
-  const float up = -weight / (3.f * (float)H * (float)W);
-  float loss = 0.f;
-  for (int e = threadIdx.x; e < kSsimB * kG1; e += kSsimThreads) {
-    const int q = e % kSsimB, r0 = (e / kSsimB) * kSsimRB;
-    float m[5][kSsimRB];
+#pragma unroll
+      for (int o = 0; o < kSsimM; ++o) acc[k][o] = dup2(0.f);
+#pragma unroll
+    for (int i = 0; i < kSsimM + 2 * kSsimR; ++i) {
+      const F2 a = load2(sx + i * kSsimA), b = load2(sy + i * kSsimA);
+      const F2 d = sub2(a, b);
+      const F2 v[5] = {a, d, mul2(a, a), mul2(b, b), mul2(d, d)};
+      filter_tap(w, v, i, acc);
+    }
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-      const float* col = sb + (k * kSsimA + r0) * kSsimBP + q;
-      float v[kSsimRB + 2 * kSsimR];
+      float* col = sb + (k * kSsimA + 2 * p) * kSsimBP + r0;
 #pragma unroll
-      for (int t = 0; t < kSsimRB + 2 * kSsimR; ++t) v[t] = col[t * kSsimBP];
-#pragma unroll
-      for (int o = 0; o < kSsimRB; ++o) {
-        float a = 0.f;
-#pragma unroll
-        for (int t = 0; t <= 2 * kSsimR; ++t) a = fmaf(win.g[t], v[o + t], a);
-        m[k][o] = a;
+      for (int o = 0; o < kSsimM; o += 2) {
+        const float2 u = split2(acc[k][o]), v = split2(acc[k][o + 1]);
+        *reinterpret_cast<float2*>(col + o) = make_float2(u.x, v.x);
+        *reinterpret_cast<float2*>(col + kSsimBP + o) = make_float2(u.y, v.y);
       }
-    }
-#pragma unroll
-    for (int o = 0; o < kSsimRB; ++o) {
-      const int r = r0 + o;
-      if (r >= kSsimB) break;
-      const int py = ty0 - kSsimR + r, px = tx0 - kSsimR + q;
-      float g0 = 0.f, g1 = 0.f, g2 = 0.f;
-      if (px >= 0 && py >= 0 && px < W && py < H) {
-        const float mx = m[0][o], md = m[1][o], my = mx - md;
-        const float b1 = fmaf(mx, mx, fmaf(my, my, kSsimC1));
-        const float b2 = (m[2][o] - mx * mx) + (m[3][o] - my * my) + kSsimC2;
-        const float vd = m[4][o] - md * md;
-        const float ib1 = 1.f / b1, ib2 = 1.f / b2;
-        const float p1 = md * md * ib1, q1 = vd * ib2;   // 1 - P, 1 - Q
-        const float P = 1.f - p1, Q = 1.f - q1;
-        if (r >= kSsimR && r < kSsimR + kSsimT && q >= kSsimR && q < kSsimR + kSsimT)
-          loss += p1 + q1 - p1 * q1;                      // 1 - S
-        const float dmx = 2.f * (mx + my) * (Q * p1 * ib1 - P * q1 * ib2);
-        const float dmd = Q * (-2.f * ib1) * (md + my * p1) + P * (2.f * ib2) * (md + my * q1);
-        g0 = up * (dmx + dmd);
-        g1 = up * P * q1 * ib2;
-        g2 = -up * P * ib2;
-      }
-      sa[(0 * kSsimB + r) * kSsimBP + q] = g0;
-      sa[(1 * kSsimB + r) * kSsimBP + q] = g1;
-      sa[(2 * kSsimB + r) * kSsimBP + q] = g2;
     }
   }
   __syncthreads();
-  // row filter of the G maps: F[k][r][q0 .. q0 + 3], r in [0, 42), q0 = 4 g
-  constexpr int kG2 = kSsimT / kSsimRB;   // 8 groups along an output row
-  for (int e = threadIdx.x; e < kSsimB * kG2; e += kSsimThreads) {
-    const int r = e / kG2, q0 = (e % kG2) * kSsimRB;
+  // row filter of the rows 2 p, 2 p + 1, then S and the G maps at their
+  // columns q0 .. q0 + 3 of the 42 x 42 region (origin tile - 5); x and y are
+  // dead, so the G maps take region A
+  const float up = -weight / (3.f * (float)H * (float)W);
+  float loss = 0.f;
+  for (int e = threadIdx.x; e < (kSsimB / 2) * kSsimGM; e += kSsimThreads) {
+    const int p = e % (kSsimB / 2), q0 = (e / (kSsimB / 2)) * kSsimM;
+    F2 acc[5][kSsimM];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      float v[16];
-      load16(sa + (k * kSsimB + r) * kSsimBP + q0, v);
-      float f[kSsimRB];
+    for (int k = 0; k < 5; ++k)
 #pragma unroll
-      for (int o = 0; o < kSsimRB; ++o) {
-        float a = 0.f;
+      for (int o = 0; o < kSsimM; ++o) acc[k][o] = dup2(0.f);
 #pragma unroll
-        for (int t = 0; t <= 2 * kSsimR; ++t) a = fmaf(win.g[t], v[o + t], a);
-        f[o] = a;
+    for (int i = 0; i < kSsimM + 2 * kSsimR; ++i) {
+      F2 v[5];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) v[k] = load2(sb + (k * kSsimA + q0 + i) * kSsimBP + 2 * p);
+      filter_tap(w, v, i, acc);
+    }
+#pragma unroll
+    for (int o = 0; o < kSsimM; ++o) {
+      const int q = q0 + o, px = tx0 - kSsimR + q, py = ty0 - kSsimR + 2 * p;
+      if (q >= kSsimB) break;
+      const F2 mx = acc[0][o], md = acc[1][o], my = sub2(mx, md);
+      const F2 one = dup2(1.f);
+      const F2 b1 = fma2(mx, mx, fma2(my, my, dup2(kSsimC1)));
+      const F2 b2 = add2(add2(sub2(acc[2][o], mul2(mx, mx)), sub2(acc[3][o], mul2(my, my))),
+                         dup2(kSsimC2));
+      const F2 vd = sub2(acc[4][o], mul2(md, md));
+      const F2 ib1 = recip2(b1), ib2 = recip2(b2);
+      const F2 p1 = mul2(mul2(md, md), ib1), q1 = mul2(vd, ib2);   // 1 - P, 1 - Q
+      const F2 P = sub2(one, p1), Q = sub2(one, q1);
+      const F2 dmx = mul2(mul2(dup2(2.f), add2(mx, my)),
+                          sub2(mul2(mul2(Q, p1), ib1), mul2(mul2(P, q1), ib2)));
+      const F2 dmd = fma2(mul2(mul2(Q, dup2(-2.f)), ib1), fma2(my, p1, md),
+                          mul2(mul2(mul2(P, dup2(2.f)), ib2), fma2(my, q1, md)));
+      const F2 u2 = dup2(up), Pi = mul2(mul2(u2, P), ib2);
+      const float2 g0 = split2(mul2(u2, add2(dmx, dmd))), g1 = split2(mul2(Pi, q1));
+      const float2 g2 = split2(Pi), l = split2(sub2(add2(p1, q1), mul2(p1, q1)));   // 1 - S
+      const bool in_x = px >= 0 && px < W;
+      const bool i0 = in_x && py >= 0 && py < H, i1 = in_x && py + 1 >= 0 && py + 1 < H;
+      if (q >= kSsimR && q < kSsimR + kSsimT) {
+        if (i0 && 2 * p >= kSsimR && 2 * p < kSsimR + kSsimT) loss += l.x;
+        if (i1 && 2 * p + 1 >= kSsimR && 2 * p + 1 < kSsimR + kSsimT) loss += l.y;
       }
-      *reinterpret_cast<float4*>(sb + (k * kSsimB + r) * kSsimT + q0) =
-          make_float4(f[0], f[1], f[2], f[3]);
+      float* g = sa + q * kSsimBP + 2 * p;
+      *reinterpret_cast<float2*>(g) = make_float2(i0 ? g0.x : 0.f, i1 ? g0.y : 0.f);
+      *reinterpret_cast<float2*>(g + kSsimB * kSsimBP) =
+          make_float2(i0 ? g1.x : 0.f, i1 ? g1.y : 0.f);
+      *reinterpret_cast<float2*>(g + 2 * kSsimB * kSsimBP) =
+          make_float2(i0 ? -g2.x : 0.f, i1 ? -g2.y : 0.f);
     }
   }
-  __syncthreads();
-  // column filter to the tile (rows r0 .. r0 + 3 of column q) and the gradient
   if (g_x) {
-    for (int e = threadIdx.x; e < kSsimT * kG2; e += kSsimThreads) {
-      const int q = e % kSsimT, r0 = (e / kSsimT) * kSsimRB;
-      const int px = tx0 + q;
-      float f[3][kSsimRB];
+    __syncthreads();
+    // row filter of the G maps, a map per item, rows 2 p, 2 p + 1:
+    // F[k][r][q0 .. q0 + 3]
+    for (int e = threadIdx.x; e < 3 * (kSsimB / 2) * kSsimGG; e += kSsimThreads) {
+      const int k = e / ((kSsimB / 2) * kSsimGG), j = e % ((kSsimB / 2) * kSsimGG);
+      const int p = j % (kSsimB / 2), q0 = (j / (kSsimB / 2)) * kSsimM;
+      F2 acc[1][kSsimM];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const float* col = sb + (k * kSsimB + r0) * kSsimT + q;
-        float v[kSsimRB + 2 * kSsimR];
+      for (int o = 0; o < kSsimM; ++o) acc[0][o] = dup2(0.f);
 #pragma unroll
-        for (int t = 0; t < kSsimRB + 2 * kSsimR; ++t) v[t] = col[t * kSsimT];
+      for (int i = 0; i < kSsimM + 2 * kSsimR; ++i) {
+        const F2 v[1] = {load2(sa + (k * kSsimB + q0 + i) * kSsimBP + 2 * p)};
+        filter_tap(w, v, i, acc);
+      }
+      float2 u[kSsimM];
 #pragma unroll
-        for (int o = 0; o < kSsimRB; ++o) {
-          float a = 0.f;
+      for (int o = 0; o < kSsimM; ++o) u[o] = split2(acc[0][o]);
+      float* row = sb + (k * kSsimB + 2 * p) * kSsimFP + q0;
+      *reinterpret_cast<float4*>(row) = make_float4(u[0].x, u[1].x, u[2].x, u[3].x);
+      *reinterpret_cast<float4*>(row + kSsimFP) = make_float4(u[0].y, u[1].y, u[2].y, u[3].y);
+    }
+    __syncthreads();
+    // column filter to the tile (rows r0, r0 + 1 of columns 2 p, 2 p + 1) and
+    // the gradient
+    for (int e = threadIdx.x; e < (kSsimT / 2) * (kSsimT / kSsimC); e += kSsimThreads) {
+      const int p = e % (kSsimT / 2), r0 = (e / (kSsimT / 2)) * kSsimC;
+      const int px = tx0 + 2 * p;
+      // the pixels' x, y and gradient so far, in flight during the filter
+      float xv[kSsimC][2], yv[kSsimC][2], gv[kSsimC][2];
+      bool in[kSsimC][2];
 #pragma unroll
-          for (int t = 0; t <= 2 * kSsimR; ++t) a = fmaf(win.g[t], v[o + t], a);
-          f[k][o] = a;
+      for (int o = 0; o < kSsimC; ++o)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          in[o][h] = ty0 + r0 + o < H && px + h < W;
+          const size_t i = ((size_t)(ty0 + r0 + o) * W + px + h) * 3 + c;
+          xv[o][h] = in[o][h] ? __ldg(x + i) : 0.f;
+          yv[o][h] = in[o][h] ? __ldg(y + i) : 0.f;
+          gv[o][h] = in[o][h] ? g_x[i] : 0.f;
+        }
+      F2 acc[3][kSsimC];
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int o = 0; o < kSsimC; ++o) acc[k][o] = dup2(0.f);
+#pragma unroll
+      for (int i = 0; i < kSsimC + 2 * kSsimR; ++i) {
+        F2 v[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) v[k] = load2(sb + (k * kSsimB + r0 + i) * kSsimFP + 2 * p);
+        filter_tap(w, v, i, acc);
+      }
+#pragma unroll
+      for (int o = 0; o < kSsimC; ++o) {
+        const float2 f0 = split2(acc[0][o]), f1 = split2(acc[1][o]), f2 = split2(acc[2][o]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (!in[o][h]) continue;
+          const size_t i = ((size_t)(ty0 + r0 + o) * W + px + h) * 3 + c;
+          g_x[i] = gv[o][h] + fmaf(2.f * xv[o][h], h ? f1.y : f1.x,
+                                   fmaf(2.f * (xv[o][h] - yv[o][h]), h ? f2.y : f2.x,
+                                        h ? f0.y : f0.x));
         }
       }
-      if (px >= W) continue;
-#pragma unroll
-      for (int o = 0; o < kSsimRB; ++o) {
-        const int py = ty0 + r0 + o;
-        if (py >= H) break;
-        const size_t i = ((size_t)py * W + px) * 3 + c;
-        const float xv = x[i], yv = y[i];
-        g_x[i] += fmaf(2.f * xv, f[1][o], fmaf(2.f * (xv - yv), f[2][o], f[0][o]));
-      }
     }
   }
-  const float t = block_sum256(loss, s_red);
+  const float t = block_sum<kSsimThreads>(loss, s_red);
   if (threadIdx.x == 0)
     part[(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = t;
 }
@@ -248,9 +297,10 @@ __global__ void __launch_bounds__(kSsimThreads) ssim_kernel(const float* __restr
 // loss[0] += scale * (fixed-order sum of the block partials)
 __global__ void ssim_sum_kernel(const float* __restrict__ part, int n, float scale,
                                 float* __restrict__ loss) {
-  __shared__ float s_red[kSsimThreads / 32];
+  __shared__ float s_red[8];
   float a = 0.f;
-  for (int i = threadIdx.x; i < n; i += kSsimThreads) a += part[i];
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += 256) a += part[i];
   const float t = block_sum256(a, s_red);
   if (threadIdx.x == 0) loss[0] += scale * t;
 }
@@ -291,7 +341,7 @@ int ssim_launch(const float* x, const float* y, int height, int width, float wei
   ssim_kernel<<<grid, kSsimThreads, kSsimSmemBytes, st>>>(x, y, height, width, weight,
                                                           ssim_window(), g_x, part);
   GS2D_LAUNCH_CHECK();
-  ssim_sum_kernel<<<1, kSsimThreads, 0, st>>>(part, (int)(grid.x * grid.y * grid.z),
+  ssim_sum_kernel<<<1, 256, 0, st>>>(part, (int)(grid.x * grid.y * grid.z),
                                               weight / (3.f * (float)height * (float)width), loss);
   GS2D_LAUNCH_CHECK();
   return GS2D_OK;
