@@ -89,6 +89,14 @@ inline int strip_rows(long long px) {
   return px >= 8ll * 152 * kStripW * kStripRows ? kStripRows : kStripRowsSmall;
 }
 
+__device__ __forceinline__ F3 cross_rn(F3 a, F3 b) {
+  return f3(fmaf(a.y, b.z, -__fmul_rn(a.z, b.y)), fmaf(a.z, b.x, -__fmul_rn(a.x, b.z)),
+            fmaf(a.x, b.y, -__fmul_rn(a.y, b.x)));
+}
+__device__ __forceinline__ F3 fma_rn(float s, F3 a, F3 b) {
+  return f3(fmaf(s, a.x, b.x), fmaf(s, a.y, b.y), fmaf(s, a.z, b.z));
+}
+
 struct MapLossImages {
   const float *rgb, *depth, *normal, *opac, *obs_rgb, *obs_depth;
   float *g_rgb, *g_depth, *g_normal, *g_opac;
@@ -97,6 +105,9 @@ struct MapLossImages {
 // Gradients of the strip with first output pixel (x0, y0); returns the lane's
 // sum of the loss terms (unscaled).  (ifx, ify) = (1/fx, 1/fy), taken once
 // per kernel: the pixel ray is ((px + 0.5 - cx) ifx, (py + 0.5 - cy) ify, 1).
+// Every product that is added to something is an explicit fmaf or __fmul_rn,
+// so that the single-view and the batched kernel round alike and their
+// gradients agree bit for bit, whatever the compiler would contract in each.
 template <int R>
 __device__ __forceinline__ float mapping_loss_strip(int x0, int y0,
                                                     const MapLossImages& im,
@@ -148,10 +159,12 @@ __device__ __forceinline__ float mapping_loss_strip(int x0, int y0,
       const int i = e * W + px;
       const float ryu = ((e - 1) + 0.5f - cam.cy) * ify, ryc = (e + 0.5f - cam.cy) * ify,
                   ryd = ((e + 1) + 0.5f - cam.cy) * ify;
-      const F3 Xr = dr * f3(rxr, ryc, 1.f), Xl = dl * f3(rxl, ryc, 1.f);
-      const F3 Xd = dd * f3(rxc, ryd, 1.f), Xu = du * f3(rxc, ryu, 1.f);
-      const F3 gx = 0.5f * (Xr - Xl), gy = 0.5f * (Xd - Xu);
-      const F3 n = cross3(gx, gy);
+      // half the differences of the neighbours' back-projected points
+      const F3 gx = 0.5f * f3(fmaf(dr, rxr, -__fmul_rn(dl, rxl)), fmaf(dr, ryc, -__fmul_rn(dl, ryc)),
+                              dr - dl);
+      const F3 gy = 0.5f * f3(fmaf(dd, rxc, -__fmul_rn(du, rxc)), fmaf(dd, ryd, -__fmul_rn(du, ryu)),
+                              dd - du);
+      const F3 n = cross_rn(gx, gy);
       const float n2 = dot3(n, n);
       if (n2 > 0.f) {
         ok = true;
@@ -163,10 +176,10 @@ __device__ __forceinline__ float mapping_loss_strip(int x0, int y0,
         Ln = 1.f - dp;
         gNr = (-1.f) * ND;
         // dLn/dn = -(Nr - ND (ND . Nr)) / |n|
-        const F3 gn = (-inn) * (Nr - dp * ND);
+        const F3 gn = (-inn) * f3(fmaf(-dp, ND.x, Nr.x), fmaf(-dp, ND.y, Nr.y), fmaf(-dp, ND.z, Nr.z));
         // dL_n / dX(p + ex) = 0.5 ggx, of X(p - ex) the negative; ggy alike
-        ggx = cross3(gy, gn);
-        ggy = cross3(gn, gx);
+        ggx = cross_rn(gy, gn);
+        ggy = cross_rn(gn, gx);
       }
     }
     // dL_n / dX(px, e) from the stencils of the left (uses X(p + ex)) and
@@ -179,8 +192,8 @@ __device__ __forceinline__ float mapping_loss_strip(int x0, int y0,
                      __shfl_down_sync(0xffffffffu, ggx.y, 1),
                      __shfl_down_sync(0xffffffffu, ggx.z, 1));
     F3 hx = f3(0.f, 0.f, 0.f);
-    if (okl) hx = hx + 0.5f * gl;
-    if (okr) hx = hx + (-0.5f) * gr;
+    if (okl) hx = fma_rn(0.5f, gl, hx);
+    if (okr) hx = fma_rn(-0.5f, gr, hx);
     const int q = e - 1;
     if (k >= 3 && q < H && out_x) {
       const int i = q * W + px;
@@ -191,24 +204,24 @@ __device__ __forceinline__ float mapping_loss_strip(int x0, int y0,
       const float d1 = __ldg(im.rgb + 3 * i + 1) - __ldg(im.obs_rgb + 3 * i + 1);
       const float d2 = __ldg(im.rgb + 3 * i + 2) - __ldg(im.obs_rgb + 3 * i + 2);
       const float ddp = Dh - __ldg(im.obs_depth + i);
-      acc += w_l1 * (fabsf(d0) + fabsf(d1) + fabsf(d2)) + w_d * fabsf(ddp);
+      acc += fmaf(w_l1, fabsf(d0) + fabsf(d1) + fabsf(d2), __fmul_rn(w_d, fabsf(ddp)));
       const float sl = w_l1 * inv;
       im.g_rgb[3 * i] = sgnf(d0) * sl;
       im.g_rgb[3 * i + 1] = sgnf(d1) * sl;
       im.g_rgb[3 * i + 2] = sgnf(d2) * sl;
-      float gDh = w_d * sgnf(ddp) * inv;
+      float gDh = __fmul_rn(w_d * sgnf(ddp), inv);
       // own normal term
-      if (ok_q) acc += w_n * ln_q;
+      if (ok_q) acc = fmaf(w_n, ln_q, acc);
       const float sn = w_n * inv;
       im.g_normal[3 * i] = sn * gn_q.x;
       im.g_normal[3 * i + 1] = sn * gn_q.y;
       im.g_normal[3 * i + 2] = sn * gn_q.z;
       // and the stencils above (uses X(p + ey)) and below (X(p - ey))
       F3 gX = hx_q;
-      if (ok_u) gX = gX + 0.5f * gy_u;
-      if (ok) gX = gX + (-0.5f) * ggy;
+      if (ok_u) gX = fma_rn(0.5f, gy_u, gX);
+      if (ok) gX = fma_rn(-0.5f, ggy, gX);
       const F3 rq = f3(rxc, (q + 0.5f - cam.cy) * ify, 1.f);
-      gDh += w_n * inv * dot3(gX, rq);
+      gDh = fmaf(sn, dot3(gX, rq), gDh);
       im.g_depth[i] = gDh / Oc;
       im.g_opac[i] = O > 1e-6f ? -gDh * D / (O * O) : 0.f;
     }
