@@ -43,14 +43,11 @@ int project_launch(const gs2d_surfels* s, const gs2d_camera* cam, const float* p
 // (used only by the full backward) are not computed.  flags:
 // kSortPreZeroed -- the caller has zeroed the counter region
 // (sort_zero_region) since the last binning, so no init launch;
-// kSortLongInBlock -- tiles with segments over 2048 keys are sorted by their
-// own 256-thread block (chunks + merges) instead of a separate launch.
 // kSortPreScanned -- a fused projection already counted and scanned the
 // tiles (implies pre-zeroed counters; no emission offsets);
 // kSortInTileKernel -- no per-tile sort launch: the tile kernel that reads
 // the bins sorts each tile's segment itself (sort_seg_args).
-constexpr unsigned kSortPreZeroed = 1u, kSortLongInBlock = 2u, kSortPreScanned = 4u,
-                   kSortInTileKernel = 8u;
+constexpr unsigned kSortPreZeroed = 1u, kSortPreScanned = 4u, kSortInTileKernel = 8u;
 // Binning of several views, one launch per stage (sort.cu): the workspace
 // is a 256-byte header followed by each view's gs2d_bin_sort workspace.
 size_t bin_sort_batch_bytes(const gs2d_view* views, int n_views, int n);

@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(256) project_fused_kernel(
     }
     // tile counts of the warp's rectangles, walked cooperatively
     warp_tile_walk(k, tx0, ty0, tx1, fz.tiles_x, fz.n_tiles, s_walk[threadIdx.x >> 5],
-                   [&](int, int t) { atomicAdd(local ? s_hist + t : fz.tile_count + t, 1u); });
+                   [&](int, int t, int) { atomicAdd(local ? s_hist + t : fz.tile_count + t, 1u); });
     __syncthreads();
     const int valid = min((int)blockDim.x, my1 - base);
     float4* dst = proj + (size_t)base * (kProjFloats / 4);
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(256) project_fused_kernel(
       s_key[threadIdx.x] = key;
       __syncwarp();
       warp_tile_walk(k, tx0, ty0, tx1, fz.tiles_x, fz.n_tiles, s_walk[threadIdx.x >> 5],
-                     [&](int owner, int t) {
+                     [&](int owner, int t, int) {
                        const uint32_t pos = atomicAdd(s_hist + t, 1u);
                        if ((long long)pos < fz.capacity) fz.seg_keys[pos] = wkey[owner];
                      });

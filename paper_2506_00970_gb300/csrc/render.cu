@@ -275,39 +275,11 @@ struct TrackSmem {
   uint32_t ids[kSegSmem];
 };
 
-// Ranks of n (distinct) keys of shared memory by counting, several keys per
-// thread (at most kRankPer): two barriers instead of a bitonic network's
-// stages; ids[rank] = the key's id, clamped below n_ids.  a has room for one
-// key more.
-constexpr int kRankPer = 3;
-__device__ __forceinline__ void rank_ids(unsigned long long* a, int n, uint32_t* ids, int n_ids) {
-  unsigned long long k[kRankPer];
-  int r[kRankPer];
-#pragma unroll
-  for (int c = 0; c < kRankPer; ++c) {
-    const int i = (int)threadIdx.x + c * kTileThreads;
-    k[c] = i < n ? a[i] : 0ull;
-    r[c] = 0;
-  }
-  if (threadIdx.x == 0) a[n] = ~0ull;   // pairs of keys are read
-  __syncthreads();
-  if (n <= kTileThreads) {
-    if ((int)threadIdx.x < n)
-      for (int j = 0; j < n; j += 2) {
-        const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(a + j);
-        r[0] += (int)(kk.x < k[0]) + (int)(kk.y < k[0]);
-      }
-  } else {
-    for (int j = 0; j < n; j += 2) {
-      const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(a + j);
-#pragma unroll
-      for (int c = 0; c < kRankPer; ++c) r[c] += (int)(kk.x < k[c]) + (int)(kk.y < k[c]);
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < kRankPer; ++c)
-    if ((int)threadIdx.x + c * kTileThreads < n)
-      ids[r[c]] = min((uint32_t)(k[c] & 0xFFFFFFFFull), (uint32_t)(n_ids - 1));
+// The ids of n sorted keys, clamped below n_ids.
+__device__ __forceinline__ void key_ids(const unsigned long long* keys, int n, uint32_t* ids,
+                                        int n_ids) {
+  for (int i = threadIdx.x; i < n; i += kTileThreads)
+    ids[i] = min((uint32_t)(keys[i] & 0xFFFFFFFFull), (uint32_t)(n_ids - 1));
   __syncthreads();
 }
 
@@ -346,17 +318,15 @@ __device__ __forceinline__ void track_tile(
     const int len = end - start;
     unsigned long long* keys = reinterpret_cast<unsigned long long*>(&sm.rec[0][0]);
     static_assert(sizeof(sm.rec) >= kSegSmem * sizeof(unsigned long long), "sort area");
-    if (len <= kTileThreads) {
-      if ((int)threadIdx.x < len) keys[threadIdx.x] = ts.seg_keys[start + threadIdx.x];
-      rank_ids(keys, len, s_ids, ts.n);
-      ids = s_ids;
-    } else if (len <= kSegSmem) {
+    constexpr int kTwice = (int)(sizeof(sm.rec) / (2 * sizeof(unsigned long long)));
+    if (len <= kSegSmem) {
       for (int i = threadIdx.x; i < len; i += kTileThreads) keys[i] = ts.seg_keys[start + i];
       __syncthreads();
-      bitonic_sort(keys, len);
-      for (int i = threadIdx.x; i < len; i += kTileThreads)
-        s_ids[i] = min((uint32_t)(keys[i] & 0xFFFFFFFFull), (uint32_t)(ts.n - 1));
-      __syncthreads();
+      if (len <= kTwice)   // room for two copies
+        keys = merge_sort(keys, keys + kTwice, len);
+      else
+        bitonic_sort(keys, len);
+      key_ids(keys, len, s_ids, ts.n);
       ids = s_ids;
     } else {
       sort_long_segment<kSegSmem>(tile, proj, ts.n, tiles_x, ranges, ts.seg_keys, ts.seg_tmp,
@@ -480,7 +450,7 @@ constexpr int kQuadKeys = 3072;
 struct QuadTrackSmem {
   union {
     QuadStage<kBwdVec4> st;
-    unsigned long long keys[kQuadKeys + 2];
+    unsigned long long keys[kQuadKeys];
   };
   uint32_t ids[kQuadKeys];
   float out[7][64];     // per pixel: the pose 6-vector and the loss
@@ -576,16 +546,12 @@ __global__ void __launch_bounds__(kTileThreads, 4) track_quad_kernel(
     }
     __syncthreads();
     const int n = s.cnt;
-    // counting ranks costs n^2 / 256 comparisons a thread, the network
-    // log^2(n) / 2 barriers: about even at 768 keys
-    if (n <= kRankPer * kTileThreads) {
-      rank_ids(s.keys, n, s.ids, ts.n);
-    } else {
+    unsigned long long* sorted = s.keys;
+    if (n <= kQuadKeys / 2)   // room for two copies
+      sorted = merge_sort(s.keys, s.keys + kQuadKeys / 2, n);
+    else
       bitonic_sort(s.keys, n);
-      for (int i = threadIdx.x; i < n; i += kTileThreads)
-        s.ids[i] = min((uint32_t)(s.keys[i] & 0xFFFFFFFFull), (uint32_t)(ts.n - 1));
-      __syncthreads();
-    }
+    key_ids(sorted, n, s.ids, ts.n);
     auto stage = [&](int b, int cnt) {   // entries b .. b + cnt - 1; returns the warp's hits
       if ((int)threadIdx.x < cnt) {
         stage_record_to<kBwdVec4>(proj, s.ids[b + threadIdx.x], xt, yt, s.st.rec[threadIdx.x]);

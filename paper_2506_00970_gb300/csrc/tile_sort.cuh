@@ -1,9 +1,10 @@
 // Device code of the per-tile depth sort (step 4 of the binning in sort.cu),
 // shared by the binning's sort kernels and by the fused tracking kernel,
 // whose blocks sort their own tile's segment before rendering it: a segment
-// of at most kSegSmem keys is sorted in shared memory by a bitonic network;
-// a longer one in kSegSmem-key chunks whose sorted runs are then merged in
-// global memory.
+// of at most kSegSmem keys is sorted in shared memory by runs and merges; a
+// longer one likewise where shared memory holds two copies of it, else in
+// chunks (a bitonic network each) whose sorted runs are then merged in global
+// memory.
 #pragma once
 
 #include "gs2d_common.cuh"
@@ -56,6 +57,53 @@ __device__ inline void bitonic_sort(unsigned long long* a, int len) {
   }
 }
 
+// Ascending sort of n distinct keys of shared memory by the whole block, a
+// and b two buffers of n keys; returns the one that holds the result (visible
+// to the block).  Warps sort runs of 32 keys in registers (a bitonic network
+// by shuffles); then runs are merged two by two, every key finding its place
+// as its index in its own run plus the number of smaller keys in the other
+// (a binary search), from one buffer into the other.  log2(n / 32) barriers
+// instead of the log2(n)^2 / 2 of a bitonic network in shared memory, which
+// spent its time on them (80 tiles of ~300 to 1300 keys at 160x120, 27 -> 19
+// us; larger grids are bound by the outputs' gathers).
+static __device__ __noinline__ unsigned long long* merge_sort(unsigned long long* a, unsigned long long* b,
+                                                 int n) {
+  const int lane = threadIdx.x & 31;
+  for (int r0 = (int)(threadIdx.x & ~31u); r0 < n; r0 += blockDim.x) {
+    const int i = r0 + lane;
+    unsigned long long k = i < n ? a[i] : ~0ull;
+#pragma unroll
+    for (int size = 2; size <= 32; size <<= 1) {
+#pragma unroll
+      for (int j = size >> 1; j > 0; j >>= 1) {
+        const unsigned long long o = __shfl_xor_sync(0xffffffffu, k, j);
+        const bool low = ((lane & j) == 0) == ((lane & size) == 0 || size == 32);
+        k = ((k < o) == low) ? k : o;
+      }
+    }
+    if (i < n) a[i] = k;
+  }
+  __syncthreads();
+  for (int w = 32; w < n; w <<= 1) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const unsigned long long k = a[i];
+      const int other = (i & ~(w - 1)) ^ w;          // the sibling run
+      const int len = min(w, n - other);
+      const unsigned long long* q = a + other - 1;   // q[m]: its m-th key
+      int m = 0;                                     // keys below k
+      if (len > 0)
+        for (int step = w; step > 0; step >>= 1)
+          if (m + step <= len && q[m + step] < k) m += step;
+      b[(i & ~(2 * w - 1)) + (i & (w - 1)) + m] = k;
+    }
+    __syncthreads();
+    unsigned long long* t = a;
+    a = b;
+    b = t;
+  }
+  return a;
+}
+
 __device__ __forceinline__ void write_outputs(const unsigned long long* a, int len, int start, int t,
                                               int tiles_x, int n, const float4* __restrict__ proj,
                                               const uint32_t* __restrict__ surfel_off,
@@ -90,10 +138,10 @@ __device__ __forceinline__ int co_rank(const unsigned long long* A, int la, cons
   return lo;
 }
 
-// Segments longer than kSegSmem: chunks of kLongChunk keys are sorted in
-// shared memory by 1024 threads, then adjacent sorted runs are merged in
-// global memory (seg_keys <-> seg_tmp), each thread producing a contiguous
-// span of the output located by a co-rank search.
+// Segments longer than kSegSmem: up to half of kChunkKeys in shared memory;
+// longer ones in chunks of kChunkKeys sorted there, then adjacent sorted runs
+// are merged in global memory (seg_keys <-> seg_tmp), each thread producing a
+// contiguous span of the output located by a co-rank search.
 // One long segment (tile t) by the whole block.
 template <int kChunkKeys>
 __device__ void sort_long_segment(int t, const float4* __restrict__ proj, int n, int tiles_x,
@@ -109,6 +157,13 @@ __device__ void sort_long_segment(int t, const float4* __restrict__ proj, int n,
   if (len <= kSegSmem) return;
   unsigned long long* src = seg_keys + start;
   unsigned long long* dst = seg_tmp + start;
+  if (len <= kChunkKeys / 2) {
+    for (int i = threadIdx.x; i < len; i += blockDim.x) s_keys[i] = src[i];
+    __syncthreads();
+    write_outputs(merge_sort(s_keys, s_keys + kChunkKeys / 2, len), len, start, t, tiles_x, n, proj,
+                  surfel_off, vals, emit, keys64);
+    return;
+  }
   const int chunks = (len + kChunkKeys - 1) / kChunkKeys;
   for (int c = 0; c < chunks; ++c) {
     const int c0 = c * kChunkKeys, cl = min(kChunkKeys, len - c0);

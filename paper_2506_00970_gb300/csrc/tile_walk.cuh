@@ -24,8 +24,9 @@ struct WalkScratch {
   int tx0[32], ty0[32], rw[32];
 };
 
-// Calls fn(owner_lane, tile) for every pair of the warp's rectangles (tile
-// ids clamped to n_tiles - 1, as everywhere in the binning).  Every lane of
+// Calls fn(owner_lane, tile, k) for every pair of the warp's rectangles (tile
+// ids clamped to n_tiles - 1, as everywhere in the binning; k the pair's
+// row-major position in the owner's rectangle).  Every lane of
 // the warp must call it, with k = 0 when its surfel covers no tile.
 template <class F>
 __device__ __forceinline__ void warp_tile_walk(int k, int tx0, int ty0, int tx1, int tiles_x,
@@ -56,9 +57,9 @@ __device__ __forceinline__ void warp_tile_walk(int k, int tx0, int ty0, int tx1,
     int rw = ws.rw[o], x0 = ws.tx0[o], y0 = ws.ty0[o];
     int left = ws.inc[o] - idx;  // pairs of the owner's rectangle from idx on
     const int off = idx - (o ? ws.inc[o - 1] : 0);
-    int row = off / rw, col = off - row * rw;
-    for (; idx < stop; ++idx) {
-      fn(o, min((y0 + row) * tiles_x + x0 + col, n_tiles - 1));
+    int row = off / rw, col = off - row * rw, pos = off;
+    for (; idx < stop; ++idx, ++pos) {
+      fn(o, min((y0 + row) * tiles_x + x0 + col, n_tiles - 1), pos);
       if (--left == 0) {
         // next lane with a non-empty rectangle (exists while idx + 1 < total)
         if (idx + 1 >= stop) break;
@@ -71,6 +72,7 @@ __device__ __forceinline__ void warp_tile_walk(int k, int tx0, int ty0, int tx1,
         left = ws.inc[o] - ws.inc[o - 1];
         row = 0;
         col = 0;
+        pos = -1;
       } else if (++col == rw) {
         col = 0;
         ++row;
