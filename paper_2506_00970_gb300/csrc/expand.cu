@@ -15,8 +15,8 @@
 //                  quaternion and state at n_map + rank; optionally its
 //                  voxel is inserted into the table.
 // A block's first index is the sum of the counts of the blocks before it,
-// formed by the block itself (a scan launch more only beyond kExSelfSum
-// blocks).
+// formed by the block itself (a scan launch more only beyond kSelfSumBlocks
+// blocks, 4.2M pixels).
 // Voxel table: open addressing with linear probing over 64-bit keys, every
 // probe loop bounded by the capacity.
 #include "gs2d_common.cuh"
@@ -30,9 +30,6 @@ constexpr int kExThreads = 256;
 constexpr int kExPer = 4;                          // pixels per thread in the selection
 constexpr int kExBlock = kExThreads * kExPer;
 constexpr int kExWords = kExBlock / 32;            // mask words per block
-// Blocks that sum the counts before them themselves: 4096 counts are 16 KB
-// from L2, ~1 us; a scan launch costs 4-5 us (4096 blocks = 4.2M pixels).
-constexpr int kExSelfSum = 4096;
 constexpr unsigned long long kEmptyKey = ~0ull;
 constexpr int kVoxBits = 21;
 constexpr int kVoxHalf = 1 << (kVoxBits - 1);
@@ -137,7 +134,7 @@ __global__ void __launch_bounds__(kExThreads) ps_select_kernel(
 }
 
 // exclusive scan of nb block counts in place; *total = the sum (only for
-// more than kExSelfSum blocks)
+// more than kSelfSumBlocks blocks)
 __global__ void __launch_bounds__(kExThreads) select_scan_kernel(int32_t* __restrict__ blk, int nb,
                                                                 int32_t* __restrict__ total) {
   __shared__ int s_w[kExThreads / 32];
@@ -151,40 +148,6 @@ __global__ void __launch_bounds__(kExThreads) select_scan_kernel(int32_t* __rest
     carry += t;
   }
   if (threadIdx.x == 0) *total = carry;
-}
-
-// This block's exclusive prefix of the block counts and their total, summed
-// by the block itself (nb <= kExSelfSum), or read after select_scan_kernel.
-// s: 2 x 8 ints; every thread calls it.
-__device__ __forceinline__ void block_base(const int32_t* __restrict__ blk, int nb,
-                                           const int32_t* __restrict__ scanned_total, int* s,
-                                           int* base, int* total) {
-  if (scanned_total) {
-    *base = blk[blockIdx.x];
-    *total = *scanned_total;
-    return;
-  }
-  int before = 0, all = 0;
-  for (int b = threadIdx.x; b < nb; b += kExThreads) {
-    const int v = blk[b];
-    all += v;
-    if (b < (int)blockIdx.x) before += v;
-  }
-  before = __reduce_add_sync(0xffffffffu, before);
-  all = __reduce_add_sync(0xffffffffu, all);
-  if ((threadIdx.x & 31) == 0) {
-    s[threadIdx.x >> 5] = before;
-    s[8 + (threadIdx.x >> 5)] = all;
-  }
-  __syncthreads();
-  before = all = 0;
-#pragma unroll
-  for (int w = 0; w < kExThreads / 32; ++w) {
-    before += s[w];
-    all += s[8 + w];
-  }
-  *base = before;
-  *total = all;
 }
 
 // ---------------------------------------------------------------------------
@@ -606,7 +569,7 @@ int gs2d_expand(const float* rgb, const float* depth, const gs2d_camera* cam, co
   cudaStream_t s = (cudaStream_t)stream;
   const ExWs w = carve_expand(workspace, P);
   const int nb = (P + kExBlock - 1) / kExBlock;
-  const bool scan = nb > kExSelfSum;
+  const bool scan = nb > kSelfSumBlocks;
   ps_select_kernel<<<nb, kExThreads, 0, s>>>(depth, u_keep, prm->ratio, P, w.mask, w.blk);
   GS2D_LAUNCH_CHECK();
   if (scan) {

@@ -161,3 +161,10 @@ def test_map_prune_and_compact(torch_cuda, n):
         assert np.array_equal(getattr(st_o, nm).cpu().numpy()[:k], e), nm
     if n:
         assert np.array_equal(new_index.cpu().numpy()[:n], idx)
+
+
+def test_passes_beyond_their_shared_and_self_summed_sizes(torch_cuda):
+    """More keyframe increments than fit in shared memory, and more compaction
+    blocks than sum the counts before them themselves."""
+    test_map_correct(torch_cuda, 10_000, 700)
+    test_map_prune_and_compact(torch_cuda, 4_300_001)
