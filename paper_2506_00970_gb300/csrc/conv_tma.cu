@@ -19,9 +19,9 @@
 //    inside a row.
 //  * B (weights [C_out][9 C_in], K = tap x C_in + channel): a box {KB k,
 //    C_out rows} in the same swizzled K-major layout.
-// One thread issues the loads S stages ahead (mbarrier transaction counts)
-// and the MMAs; a stage is refilled once the tcgen05.commit of the MMAs that
-// read it has arrived.  Four warps read the accumulator back (tcgen05.ld)
+// One warp issues the loads S stages ahead (mbarrier transaction counts),
+// another the MMAs; a stage is refilled once the tcgen05.commit of the MMAs
+// that read it has arrived.  Four warps read the accumulator back (tcgen05.ld)
 // and apply bias, ReLU and the bfloat16 rounding of the other kernels.
 // Every wait is bounded: past the limit the kernel records an error in
 // *err, stops issuing, waits (bounded) for what it issued and frees its
@@ -92,8 +92,8 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
-// A tile is NI images' TW x TH output pixels (NI = 1: a 128-pixel part of one
-// image; NI > 1: whole small images, TW x TH = the output map) times NB of the
+// A tile is NI images' TW x TH output pixels (a 128-pixel part of one image,
+// or whole small images, TW x TH = the output map) times NB of the
 // C_out channels.  One box per tap and channel block spans the NI images
 // (its fourth dimension), so image g's pixels are rows [g TW TH, (g + 1) TW TH)
 // of the 128-row MMA tile; rows past NI TW TH hold stale data whose results
@@ -116,7 +116,7 @@ struct ConvTma {
   static constexpr int SMEM = S * STAGE + 1024;   // + slack for 1024-byte alignment
   static constexpr int TMEM_COLS = NB;
   static constexpr int NSPLIT = COUT / NB;        // channel groups (grid.y)
-  static_assert(NI == 1 ? TW * TH == 128 : (TX == 1 && TY == 1 && ROWS <= 128),
+  static_assert((NI == 1 && TW * TH == 128) || (TX == 1 && TY == 1 && ROWS <= 128),
                 "one 128-row MMA tile: a part of one image, or whole images");
   static_assert(KB == 32 || KB == 64, "64- or 128-byte swizzled rows");
   static_assert(CIN % KB == 0 && NB >= 32 && NB <= 256 && (NB & (NB - 1)) == 0 &&
@@ -126,6 +126,107 @@ struct ConvTma {
   static_assert(2 * TW <= 256 && 2 * TH <= 256, "TMA box dimensions");
 };
 
+// The two issuing roles of a tile, each a whole warp whose lane 0 issues: the
+// loop counters, barrier addresses and descriptors are then warp-uniform, and
+// only the issuing instructions are predicated.  As single-thread loops with
+// a descriptor built per MMA they took ~0.5 us per K step (of 9 to 36),
+// whatever the step's bytes and MMAs, and were most of a small batch's time.
+
+// Commit of every MMA issued so far to barrier bar, by lane 0.
+__device__ __forceinline__ void commit_lane0(uint32_t bar) {
+  asm volatile(
+      "{.reg .pred q; setp.eq.u32 q, %1, 0;\n"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];}\n" ::"r"(bar),
+      "r"(threadIdx.x & 31)
+      : "memory");
+}
+
+// K steps 0 .. KS - 1 of one tile into the accumulator at tmem, the stages'
+// running number starting at g0.  False when a wait ran out (the steps before
+// it are issued).
+template <class C, int S, int N>
+__device__ __forceinline__ bool mma_steps(uint32_t tmem, int g0, const uint64_t* s_full,
+                                          const uint64_t* s_empty, uint32_t stages,
+                                          volatile int* s_consumed) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t a0 = sw_desc<C::SW>(stages), b0 = sw_desc<C::SW>(stages + C::A_BYTES);
+  const uint32_t a_lo = (uint32_t)a0, a_hi = (uint32_t)(a0 >> 32);
+  const uint32_t b_lo = (uint32_t)b0, b_hi = (uint32_t)(b0 >> 32);
+  int st = g0 % S;
+  uint32_t phase = (uint32_t)((g0 / S) & 1);
+#pragma unroll 1
+  for (int s = 0; s < C::KS; ++s) {
+    if (!bar_wait(smem_u32(s_full + st), phase)) return false;
+    *s_consumed = g0 + s + 1;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    // the address field counts 16 bytes and does not carry out of its 14 bits
+    const uint32_t off = (uint32_t)st * (C::STAGE / 16);
+#pragma unroll
+    for (int j = 0; j < C::MMAS; ++j) {
+      // K step j of the stage: 16 channels, 32 bytes into every swizzled row
+      asm volatile(
+          "{.reg .pred p, q; .reg .b64 da, db;\n"
+          "setp.ne.b32 p, %6, 0; setp.eq.u32 q, %7, 0;\n"
+          "mov.b64 da, {%1, %2}; mov.b64 db, {%3, %4};\n"
+          "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;}\n" ::"r"(tmem),
+          "r"(a_lo + off + 2 * j), "r"(a_hi), "r"(b_lo + off + 2 * j), "r"(b_hi),
+          "r"(mma_idesc(N)), "r"((s > 0 || j > 0) ? 1u : 0u), "r"(lane));
+    }
+    commit_lane0(smem_u32(s_empty + st));
+    if (++st == S) {
+      st = 0;
+      phase ^= 1u;
+    }
+  }
+  return true;
+}
+
+// Loads of `steps` K steps (KS per tile), a stage's once the MMAs that read
+// its previous fill are done.  origin(tile step, x, y, n): the input pixel of
+// tap (0, 0) and the image of the tile that step s belongs to.
+template <class C, int CIN, int S, class Origin>
+__device__ __forceinline__ void load_steps(const CUtensorMap& map_x, const CUtensorMap& map_w,
+                                           int steps, const uint64_t* s_full,
+                                           const uint64_t* s_empty, uint32_t stages,
+                                           volatile int* s_issued, int* s_fail, Origin origin,
+                                           int nb0) {
+  const uint32_t lane = threadIdx.x & 31;
+  int st = 0, x = 0, y = 0, n = 0, cb = 0, kx = 0, ky = 0, k = 0;
+  uint32_t phase = 1u;   // of the stage's previous fill
+#pragma unroll 1
+  for (int g = 0; g < steps; ++g) {
+    if (k == 0) origin(g, x, y, n);
+    if (g >= S && !bar_wait(smem_u32(s_empty + st), phase)) {
+      if (lane == 0) atomicExch(s_fail, 1);
+      return;
+    }
+    const uint32_t base = stages + (uint32_t)st * C::STAGE;
+    if (lane == 0) {
+      const uint32_t bar = smem_u32(s_full + st);
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                   "r"(C::TX_BYTES)
+                   : "memory");
+      tma_load_4d(base, &map_x, cb, x + kx, y + ky, n, bar);
+      tma_load_2d(base + C::A_BYTES, &map_w, (3 * ky + kx) * CIN + cb, nb0, bar);
+    }
+    *s_issued = g + 1;
+    // next channel block, tap, tile
+    cb += C::KB;
+    if (cb == CIN) {
+      cb = 0;
+      if (++kx == 3) {
+        kx = 0;
+        if (++ky == 3) ky = 0;
+      }
+    }
+    if (++k == C::KS) k = 0;
+    if (++st == S) {
+      st = 0;
+      phase ^= 1u;
+    }
+  }
+}
+
 template <int CIN, int COUT, int HI, int WI, int TW, int TH, int S, int NI, int NB>
 __global__ void __launch_bounds__(kConvThreads) conv_tma_kernel(
     const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
@@ -134,7 +235,7 @@ __global__ void __launch_bounds__(kConvThreads) conv_tma_kernel(
   extern __shared__ unsigned char conv_raw[];
   __shared__ __align__(8) uint64_t s_full[S], s_empty[S], s_done;
   __shared__ uint32_t s_tmem;
-  __shared__ int s_fail;
+  __shared__ int s_fail, s_issued, s_consumed;
   unsigned char* stages = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(conv_raw) + 1023) & ~(uintptr_t)1023);
   const int tile = blockIdx.x;
@@ -147,6 +248,8 @@ __global__ void __launch_bounds__(kConvThreads) conv_tma_kernel(
 
   if (threadIdx.x == 0) {
     s_fail = 0;
+    s_issued = 0;
+    s_consumed = 0;
     for (int i = 0; i < S; ++i) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_full[i])));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_empty[i])));
@@ -165,77 +268,28 @@ __global__ void __launch_bounds__(kConvThreads) conv_tma_kernel(
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s_tmem;
 
-  // warp 0's lane 0 issues every load and MMA; its other lanes wait for it
-  // at the __syncwarp below rather than spinning beside it
-  if (threadIdx.x == 0) {
-    // stage s: the input box of tap s / CB, channels cb .. cb + KB, and the
-    // matching weight box
-    auto load = [&](int s) {
-      const int st = s % S;
-      const uint32_t base = smem_u32(stages + st * C::STAGE);
-      const uint32_t bar = smem_u32(&s_full[st]);
-      const int tap = s / C::CB, cb = (s % C::CB) * C::KB;
-      const int ky = tap / 3, kx = tap - 3 * (tap / 3);
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
-                   "r"(C::TX_BYTES)
-                   : "memory");
-      // images past the batch read as zeros (out-of-range coordinates)
-      tma_load_4d(base, &map_x, cb, 2 * ox0 + kx - 1, 2 * oy0 + ky - 1, img, bar);
-      tma_load_2d(base + C::A_BYTES, &map_w, tap * CIN + cb, nb0, bar);
-    };
-    bool fail = false;
-    int issued = 0, consumed = 0;
-    for (; issued < S && issued < C::KS; ++issued) load(issued);
-    for (int s = 0; s < C::KS; ++s) {
-      const int st = s % S;
-      if (!bar_wait(smem_u32(&s_full[st]), (uint32_t)((s / S) & 1))) {
-        fail = true;
-        break;
-      }
-      consumed = s + 1;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t base = smem_u32(stages + st * C::STAGE);
-#pragma unroll
-      for (int j = 0; j < C::MMAS; ++j) {
-        // K step j of the stage: 16 channels, 32 bytes into every swizzled row
-        const uint64_t ad = sw_desc<C::SW>(base + 32 * j);
-        const uint64_t bd = sw_desc<C::SW>(base + C::A_BYTES + 32 * j);
-        const uint32_t acc = (s > 0 || j > 0) ? 1u : 0u;
-        asm volatile(
-            "{.reg .pred p; setp.ne.b32 p, %4, 0;\n"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;}\n" ::"r"(tmem),
-            "l"(ad), "l"(bd), "r"(mma_idesc(NB)), "r"(acc));
-      }
-      asm volatile(
-          "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-              smem_u32(&s_empty[st]))
-          : "memory");
-      // refill the stage the previous step read once its MMA is done (the
-      // MMA just issued keeps the tensor pipe busy meanwhile)
-      if (s >= 1 && issued < C::KS) {
-        const int ps = (s - 1) % S;
-        if (!bar_wait(smem_u32(&s_empty[ps]), (uint32_t)(((s - 1) / S) & 1))) {
-          fail = true;
-          break;
-        }
-        load(issued++);
-      }
-    }
+  // warp 1 issues every load, warp 0 every MMA, so that the MMAs wait for
+  // nothing but their operands
+  if (warp == 1)
+    load_steps<C, CIN, S>(map_x, map_w, C::KS, s_full, s_empty, smem_u32(stages), &s_issued,
+                          &s_fail, [&](int s, int& x, int& y, int& n) {
+                            (void)s;
+                            x = 2 * ox0 - 1;
+                            y = 2 * oy0 - 1;
+                            n = img;   // images past the batch read as zeros
+                          }, nb0);
+  if (warp == 0) {
+    const int ok = mma_steps<C, S, NB>(tmem, 0, s_full, s_empty, smem_u32(stages), &s_consumed);
     // one last commit tracks every MMA issued (all, or those before a failure)
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            smem_u32(&s_done))
-        : "memory");
-    if (fail) {
-      s_fail = 1;
-      // loads still in flight must land before the CTA exits (bounded)
-      for (int s = consumed; s < issued; ++s)
-        bar_wait(smem_u32(&s_full[s % S]), (uint32_t)((s / S) & 1));
-    }
+    commit_lane0(smem_u32(&s_done));
+    if (!ok) s_fail = 1;
   }
-  if (warp == 0) __syncwarp();
   if (!bar_wait(smem_u32(&s_done), 0u)) atomicExch(&s_fail, 1);
   __syncthreads();
+  // loads issued but not consumed (after a failure) land before the CTA exits
+  if (threadIdx.x == 32)
+    for (int s = s_consumed; s < s_issued; ++s)
+      bar_wait(smem_u32(&s_full[s % S]), (uint32_t)((s / S) & 1));
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (!*reinterpret_cast<volatile int*>(&s_fail)) {
     // TMEM lane = row m: image img + m / (TW TH), output pixel (oy0 + q / TW,
@@ -339,84 +393,31 @@ __global__ void __launch_bounds__(kPersThreads) conv_tma_pers_kernel(
   const uint32_t tmem = s_tmem;
 
   if (warp == 4) {
-    if (lane == 0) {
-      int g = 0;
-      bool fail = false;
-      for (int k = 0; k < my_n && !fail; ++k) {
-        const int tile = (int)blockIdx.x + k * (int)gridDim.x;
-        const int img = tile / (C::TX * C::TY), r = tile % (C::TX * C::TY);
-        const int oy0 = (r / C::TX) * TH, ox0 = (r % C::TX) * TW;
-        for (int s = 0; s < C::KS; ++s, ++g) {
-          const int st = g % S;
-          // the MMAs that read this stage's previous fill are done
-          if (g >= S && !bar_wait(smem_u32(&s_empty[st]), (uint32_t)((g / S - 1) & 1))) {
-            fail = true;
-            break;
-          }
-          const uint32_t base = smem_u32(stages + st * C::STAGE);
-          const uint32_t bar = smem_u32(&s_full[st]);
-          const int tap = s / C::CB, cb = (s % C::CB) * C::KB;
-          const int ky = tap / 3, kx = tap - 3 * (tap / 3);
-          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
-                       "r"(C::TX_BYTES)
-                       : "memory");
-          tma_load_4d(base, &map_x, cb, 2 * ox0 + kx - 1, 2 * oy0 + ky - 1, img, bar);
-          tma_load_2d(base + C::A_BYTES, &map_w, tap * CIN + cb, 0, bar);
-          s_issued = g + 1;
-        }
-      }
-      if (fail) atomicExch(&s_fail, 1);
-    }
+    load_steps<C, CIN, S>(map_x, map_w, my_n * C::KS, s_full, s_empty, smem_u32(stages), &s_issued,
+                          &s_fail, [&](int g, int& x, int& y, int& n) {
+                            const int tile = (int)blockIdx.x + g / C::KS * (int)gridDim.x;
+                            const int r = tile % (C::TX * C::TY);
+                            n = tile / (C::TX * C::TY);
+                            x = 2 * (r % C::TX) * TW - 1;
+                            y = 2 * (r / C::TX) * TH - 1;
+                          }, 0);
   } else if (warp == 5) {
-    if (lane == 0) {
-      int g = 0;
-      bool fail = false;
-      for (int k = 0; k < my_n && !fail; ++k) {
-        const int buf = k & 1;
-        // the epilogue has read this accumulator's previous tile
-        if (k >= 2 && !bar_wait(smem_u32(&s_tempty[buf]), (uint32_t)(((k >> 1) - 1) & 1))) {
-          fail = true;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t acc_tmem = tmem + (uint32_t)(buf * C::TMEM_COLS);
-        for (int s = 0; s < C::KS; ++s, ++g) {
-          const int st = g % S;
-          if (!bar_wait(smem_u32(&s_full[st]), (uint32_t)((g / S) & 1))) {
-            fail = true;
-            break;
-          }
-          s_consumed = g + 1;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t base = smem_u32(stages + st * C::STAGE);
-#pragma unroll
-          for (int j = 0; j < C::MMAS; ++j) {
-            const uint64_t ad = sw_desc<C::SW>(base + 32 * j);
-            const uint64_t bd = sw_desc<C::SW>(base + C::A_BYTES + 32 * j);
-            const uint32_t acc = (s > 0 || j > 0) ? 1u : 0u;
-            asm volatile(
-                "{.reg .pred p; setp.ne.b32 p, %4, 0;\n"
-                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;}\n" ::"r"(acc_tmem),
-                "l"(ad), "l"(bd), "r"(mma_idesc(COUT)), "r"(acc));
-          }
-          asm volatile(
-              "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                  smem_u32(&s_empty[st]))
-              : "memory");
-        }
-        if (fail) break;
-        asm volatile(
-            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                smem_u32(&s_tfull[buf]))
-            : "memory");
+    bool ok = true;
+    for (int k = 0; k < my_n && ok; ++k) {
+      const int buf = k & 1;
+      // the epilogue has read this accumulator's previous tile
+      if (k >= 2 && !bar_wait(smem_u32(&s_tempty[buf]), (uint32_t)(((k >> 1) - 1) & 1))) {
+        ok = false;
+        break;
       }
-      // one last commit tracks every MMA issued
-      asm volatile(
-          "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-              smem_u32(&s_done))
-          : "memory");
-      if (fail) atomicExch(&s_fail, 1);
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      ok = mma_steps<C, S, COUT>(tmem + (uint32_t)(buf * C::TMEM_COLS), k * C::KS, s_full, s_empty,
+                                 smem_u32(stages), &s_consumed);
+      if (ok) commit_lane0(smem_u32(&s_tfull[buf]));
     }
+    // one last commit tracks every MMA issued
+    commit_lane0(smem_u32(&s_done));
+    if (!ok && lane == 0) atomicExch(&s_fail, 1);
   } else {
     // warps 0-3: TMEM lane = row m = threadIdx.x = output pixel (oy0 + m / TW, ox0 + m % TW)
     const int m = threadIdx.x;
@@ -612,33 +613,52 @@ int run_pers(const bf16* x, int B, const bf16* w, const float* bias, bf16* out, 
 
 bool conv_tma_layer(int layer) { return layer >= 1 && layer <= 5; }
 
-// Stages in flight: with a grid that fills the GPU several CTAs share an SM
-// (fewer stages each; the SM keeps as many loads in flight); a small batch's
-// few CTAs each keep as many stages as shared memory holds.  The stage count
-// changes no result (every tile sums its K steps in the same order).
+// Which form a layer runs in at a batch.  None changes a result: every tile
+// sums its K steps in the same order.  A CTA's time is its chain of K steps
+// (~0.25 us each, 9 to 36 of them, nearly whatever their bytes) plus ~5 us,
+// so a batch too small to fill the GPU splits the output channels over more
+// CTAs (NB of them each, which lets a stage be smaller and more stages fit);
+// a larger one takes wide tiles, few enough stages that two CTAs share an SM,
+// and for layers 3 and 4 the persistent form.  Measured per layer (us, batch
+// 1 / 24 / 77 / 256; before: one or two forms per layer and one thread
+// issuing loads and MMAs):
+//   layer 2   8.4 / 9.9 / 19.5 / 45.0  ->   6.8 / 8.9 / 18.4 / 40.6
+//   layer 3  11.2 / 10.9 / 19.2 / 30.4 ->   7.3 / 8.5 / 14.0 / 31.1
+//   layer 4  20.3 / 18.9 / 18.9 / 26.8 ->   9.3 / 10.8 / 14.7 / 21.8
+//   layer 5  22.1 / 23.6 / 22.3 / 23.4 ->  13.5 / 14.0 / 14.0 / 17.1
+//   layer 6  17.7 / 18.4 / 18.0 / 18.0 ->  13.3 / 14.0 / 13.6 / 14.3
 int conv_tma_forward(int layer, const bf16* x, int B, const bf16* w, const float* bias, bf16* out,
                      int* err, cudaStream_t st) {
-  constexpr int kFull = 2 * 152;  // CTAs that fill the GPU twice over
+  constexpr int kSms = 152;
   switch (layer) {
-    // layers 3 and 4 with more tiles than the GPU holds CTAs: the persistent
-    // form (layer 2's grid is bound by its 64-byte strided input rows, not
-    // by per-tile set-up: the persistent form measured the same there)
-    case 1:
-      return B * 10 >= kFull ? run<32, 64, 60, 80, 8, 16, 4>(x, B, w, bias, out, err, st)
-                             : run<32, 64, 60, 80, 8, 16, 8>(x, B, w, bias, out, err, st);
-    case 2:
-      return B * 3 >= kFull ? run_pers<64, 128, 30, 40, 8, 16, 6>(x, B, w, bias, out, err, st)
-                            : run<64, 128, 30, 40, 8, 16, 6>(x, B, w, bias, out, err, st);
+    case 1:   // 10 tiles per image
+      return B * 10 * 2 <= 2 * kSms ? run<32, 64, 60, 80, 8, 16, 9, 1, 32>(x, B, w, bias, out, err, st)
+                                    : run<32, 64, 60, 80, 8, 16, 3>(x, B, w, bias, out, err, st);
+    case 2:   // 3 tiles per image
+      if (B * 3 * 4 <= kSms) return run<64, 128, 30, 40, 8, 16, 9, 1, 32>(x, B, w, bias, out, err, st);
+      if (B * 3 * 2 <= 4 * kSms / 3)
+        return run<64, 128, 30, 40, 8, 16, 4, 1, 64>(x, B, w, bias, out, err, st);
+      return B * 3 <= 2 * kSms ? run<64, 128, 30, 40, 8, 16, 3>(x, B, w, bias, out, err, st)
+                               : run_pers<64, 128, 30, 40, 8, 16, 6>(x, B, w, bias, out, err, st);
+    // layer 4's 8 x 10 outputs are one tile of 80 rows
     case 3:
-      return B >= kFull / 2 ? run_pers<128, 256, 15, 20, 16, 8, 4>(x, B, w, bias, out, err, st)
-                            : run<128, 256, 15, 20, 16, 8, 4>(x, B, w, bias, out, err, st);
+      if (B * 8 <= kSms) return run<128, 256, 15, 20, 10, 8, 11, 1, 32>(x, B, w, bias, out, err, st);
+      if (B * 4 <= kSms) return run<128, 256, 15, 20, 10, 8, 9, 1, 64>(x, B, w, bias, out, err, st);
+      if (B * 2 <= kSms) return run<128, 256, 15, 20, 10, 8, 6, 1, 128>(x, B, w, bias, out, err, st);
+      return B <= kSms ? run<128, 256, 15, 20, 10, 8, 3, 1, 128>(x, B, w, bias, out, err, st)
+                       : run_pers<128, 256, 15, 20, 10, 8, 4>(x, B, w, bias, out, err, st);
     // layers 5 and 6 (4 x 5 and 2 x 3 outputs): whole images per tile (5 and
-    // 21: 100 and 126 rows), the 256 output channels in halves or quarters so
-    // the grid still spreads over the SMs
-    case 4:
-      return run<256, 256, 8, 10, 5, 4, 6, 5, 128>(x, B, w, bias, out, err, st);
+    // 21: 100 and 126 rows)
+    case 4: {
+      const int tiles = (B + 4) / 5;
+      if (tiles * 8 <= kSms) return run<256, 256, 8, 10, 5, 4, 11, 5, 32>(x, B, w, bias, out, err, st);
+      if (tiles * 4 <= kSms) return run<256, 256, 8, 10, 5, 4, 9, 5, 64>(x, B, w, bias, out, err, st);
+      return tiles * 4 <= 2 * kSms ? run<256, 256, 8, 10, 5, 4, 4, 5, 64>(x, B, w, bias, out, err, st)
+                                   : run<256, 256, 8, 10, 5, 4, 3, 5, 128>(x, B, w, bias, out, err, st);
+    }
     case 5:
-      return run<256, 256, 4, 5, 3, 2, 8, 21, 32>(x, B, w, bias, out, err, st);
+      return (B + 20) / 21 * 8 <= kSms ? run<256, 256, 4, 5, 3, 2, 11, 21, 32>(x, B, w, bias, out, err, st)
+                                       : run<256, 256, 4, 5, 3, 2, 5, 21, 32>(x, B, w, bias, out, err, st);
     default: return GS2D_ERR_INVALID_ARG;
   }
 }

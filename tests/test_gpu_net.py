@@ -365,3 +365,27 @@ def test_prepared_forward_is_the_forward(torch_cuda):
     gs2d.gs2d_net_forward_prepared(params, x, y1, ws)
     torch.cuda.synchronize()
     assert torch.equal(y0, y1)
+
+
+def test_forward_does_not_depend_on_the_batch(torch_cuda):
+    """The forward's layers run in different forms by batch (tile width,
+    output channels per tile, persistent or not); a sample's outputs are the
+    same bits in each.  Batches on both sides of every line of those rules."""
+    torch = torch_cuda
+    from paper_2506_00970_gb300 import gs2d
+    params = torch.tensor(scenes.net_init(4, gs2d.net_init_blocks()), device="cuda")
+    g = torch.Generator(device="cuda")
+    g.manual_seed(2)
+    x = (torch.rand(400, 120, 160, 8, generator=g, device="cuda") * 2 - 1).to(torch.bfloat16)
+
+    def forward(b):
+        ws = torch.empty(gs2d.gs2d_net_workspace(b), dtype=torch.uint8, device="cuda")
+        y = torch.empty(b, 6, device="cuda")
+        gs2d.gs2d_net_forward(params, x[:b].contiguous(), y, ws)
+        return y
+
+    ref = forward(400)
+    assert torch.isfinite(ref).all() and float(ref.abs().max()) > 0
+    for b in (1, 12, 13, 15, 16, 19, 20, 33, 34, 38, 39, 76, 77, 95, 96, 101, 102, 152, 153, 190,
+              191, 380, 381, 399):
+        assert torch.equal(forward(b), ref[:b]), b
