@@ -54,36 +54,72 @@ __device__ __forceinline__ int length_bucket(uint32_t len) {
   const int oct = 31 - __clz(len);  // >= 4
   return 16 + (oct - 4) * 8 + (int)((len >> (oct - 3)) & 7u);  // <= 239
 }
+// One block; its threads take eight items at a time so that their loads are
+// in flight together: 45,800 items 68 -> 53 us, 25,800 items 30 -> 26 us.
+// The rest is the atomics' (a warp's items of one bucket, matched and counted
+// together, took 68 and 34 us).
+constexpr int kOrderPer = 8;
 __global__ void __launch_bounds__(kOrderThreads) order_items_kernel(ViewTable tab,
                                                                   int32_t* __restrict__ order) {
   __shared__ uint32_t hist[kOrderBuckets];
+  __shared__ int s_first[GS2D_MAX_VIEWS + 1];
+  __shared__ const int2* s_ranges[GS2D_MAX_VIEWS];
+  __shared__ bool s_dead[GS2D_MAX_VIEWS];
   for (int b = threadIdx.x; b < kOrderBuckets; b += blockDim.x) hist[b] = 0u;
-  __syncthreads();
-  for (int v = 0; v < tab.n_views; ++v) {
-    const ViewDev& V = tab.v[v];
-    const bool dead = V.status && *V.status;
-    for (int t = threadIdx.x; t < V.n_tiles; t += blockDim.x) {
-      const uint32_t len = dead ? 0u : (uint32_t)max(V.ranges[2 * t + 1] - V.ranges[2 * t], 0);
-      atomicAdd(&hist[length_bucket(len)], 1u);
+  for (int v = threadIdx.x; v <= tab.n_views; v += blockDim.x) {
+    s_first[v] = v < tab.n_views ? tab.v[v].item0 : tab.n_items;
+    if (v < tab.n_views) {
+      s_ranges[v] = reinterpret_cast<const int2*>(tab.v[v].ranges);
+      s_dead[v] = tab.v[v].status && *tab.v[v].status;
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) {  // exclusive scan, longest bucket first
+  auto buckets = [&](int base, int (&bk)[kOrderPer]) {
+    int2 r[kOrderPer];
+    int v = 0;
+#pragma unroll
+    for (int k = 0; k < kOrderPer; ++k) {
+      const int i = base + k * kOrderThreads;
+      r[k] = make_int2(0, 0);
+      bk[k] = i < tab.n_items ? 0 : -1;
+      if (i < tab.n_items) {
+        while (i >= s_first[v + 1]) ++v;
+        if (!s_dead[v]) r[k] = s_ranges[v][i - s_first[v]];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kOrderPer; ++k)
+      if (bk[k] == 0) bk[k] = length_bucket((uint32_t)max(r[k].y - r[k].x, 0));
+  };
+  int bk[kOrderPer];
+  for (int base = threadIdx.x; base < tab.n_items; base += kOrderPer * kOrderThreads) {
+    buckets(base, bk);
+#pragma unroll
+    for (int k = 0; k < kOrderPer; ++k)
+      if (bk[k] >= 0) atomicAdd(&hist[bk[k]], 1u);
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {  // exclusive scan, longest bucket first
     uint32_t run = 0u;
-    for (int b = kOrderBuckets - 1; b >= 0; --b) {
+    for (int b0 = kOrderBuckets - 32; b0 >= 0; b0 -= 32) {
+      const int b = b0 + 31 - (int)threadIdx.x;
       const uint32_t c = hist[b];
-      hist[b] = run;
-      run += c;
+      uint32_t inc = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+        if ((int)threadIdx.x >= o) inc += t;
+      }
+      hist[b] = run + inc - c;
+      run += __shfl_sync(0xffffffffu, inc, 31);
     }
   }
   __syncthreads();
-  for (int v = 0; v < tab.n_views; ++v) {
-    const ViewDev& V = tab.v[v];
-    const bool dead = V.status && *V.status;
-    for (int t = threadIdx.x; t < V.n_tiles; t += blockDim.x) {
-      const uint32_t len = dead ? 0u : (uint32_t)max(V.ranges[2 * t + 1] - V.ranges[2 * t], 0);
-      order[atomicAdd(&hist[length_bucket(len)], 1u)] = V.item0 + t;
-    }
+  for (int base = threadIdx.x; base < tab.n_items; base += kOrderPer * kOrderThreads) {
+    buckets(base, bk);
+#pragma unroll
+    for (int k = 0; k < kOrderPer; ++k)
+      if (bk[k] >= 0) order[atomicAdd(&hist[bk[k]], 1u)] = base + k * kOrderThreads;
   }
 }
 
@@ -190,7 +226,7 @@ struct BatchWs {
   uint32_t* queue;        // [2] fwd, bwd work counters
   int32_t* order;         // [items] heavy-first work order
   float* partials[GS2D_MAX_VIEWS];
-  float* pose_part;       // [max parts * 6]
+  float* pose_part[GS2D_MAX_VIEWS];  // [parts * 6] per view
   size_t bytes;
 };
 
@@ -204,14 +240,12 @@ BatchWs carve_batch_ws(void* base, const gs2d_view* views, int n_views, int n) {
     items += (size_t)max(view_tiles(views[v], &tx), 0);
   }
   w.order = c.take<int32_t>(items > 0 ? items : 1);
-  int max_parts = 1;
   for (int v = 0; v < n_views; ++v) {
     const size_t cap = views[v].bins.capacity > 0 ? views[v].bins.capacity : 1;
     w.partials[v] = c.take<float>(cap * bwd_regions(views[v].cfg) * 16);
     const int m = views[v].active ? views[v].n_active : n;
-    max_parts = max(max_parts, (m + 255) / 256);
+    w.pose_part[v] = c.take<float>((size_t)max(1, (m + 255) / 256) * 6);
   }
-  w.pose_part = c.take<float>((size_t)max_parts * 6);
   w.bytes = align_up(c.off, 256);
   return w;
 }
@@ -405,24 +439,39 @@ int gs2d_render_bwd_batch(const gs2d_view* views, int n_views, const gs2d_surfel
   if (grid <= 0) return GS2D_ERR_CUDA;
   bwd_batch_kernel<<<grid, kBwdWarps * 32, 0, st>>>(tab, Q, w.queue + 1, w.order);
   GS2D_LAUNCH_CHECK();
-  // surfels outside every view's subset receive zero: clear, then add view by view
-  GS2D_CUDA_TRY(cudaMemsetAsync(d_mu, 0, sizeof(float) * 3 * s->n, st));
-  GS2D_CUDA_TRY(cudaMemsetAsync(d_quat, 0, sizeof(float) * 4 * s->n, st));
-  GS2D_CUDA_TRY(cudaMemsetAsync(d_scale, 0, sizeof(float) * 2 * s->n, st));
-  GS2D_CUDA_TRY(cudaMemsetAsync(d_opac, 0, sizeof(float) * s->n, st));
-  GS2D_CUDA_TRY(cudaMemsetAsync(d_rgb, 0, sizeof(float) * 3 * s->n, st));
-  for (int v = 0; v < n_views; ++v) {
-    const gs2d_view& x = views[v];
-    const int m = x.active ? x.n_active : s->n;
-    r = surfel_grad_launch(s, x.active, m, 1, x.pose, x.tiles_per_surfel, x.bins.surfel_off, Q,
-                           x.proj, w.partials[v], d_mu, d_quat, d_scale, d_opac, d_rgb, w.pose_part,
-                           x.bins.status, st);
-    if (r) return r;
-    if (x.d_pose6) {
-      r = pose_reduce_launch(w.pose_part, (m + 255) / 256, x.d_pose6, x.bins.status, st);
-      if (r) return r;
-    }
+  // runs of views that draw every surfel go in one launch, which sums their
+  // gradients in registers; a view of a subset goes by itself and adds its
+  // own.  Without a run at the head the outputs are cleared first: surfels
+  // outside every view's subset receive zero.
+  if (views[0].active) {
+    GS2D_CUDA_TRY(cudaMemsetAsync(d_mu, 0, sizeof(float) * 3 * s->n, st));
+    GS2D_CUDA_TRY(cudaMemsetAsync(d_quat, 0, sizeof(float) * 4 * s->n, st));
+    GS2D_CUDA_TRY(cudaMemsetAsync(d_scale, 0, sizeof(float) * 2 * s->n, st));
+    GS2D_CUDA_TRY(cudaMemsetAsync(d_opac, 0, sizeof(float) * s->n, st));
+    GS2D_CUDA_TRY(cudaMemsetAsync(d_rgb, 0, sizeof(float) * 3 * s->n, st));
   }
+  PoseReduceTable pt;
+  pt.n = 0;
+  for (int v = 0; v < n_views;) {
+    const int first = v;
+    const int32_t* active = views[first].active;
+    const int m = active ? views[first].n_active : s->n;
+    GradTable t;
+    t.n = 0;
+    do {
+      const gs2d_view& x = views[v];
+      t.v[t.n++] = GradView{x.pose, x.tiles_per_surfel, x.bins.surfel_off, x.proj, w.partials[v],
+                            w.pose_part[v], x.bins.status};
+      if (x.d_pose6)
+        pt.v[pt.n++] = PoseReduceView{w.pose_part[v], (m + 255) / 256, x.d_pose6, x.bins.status};
+      ++v;
+    } while (!active && v < n_views && !views[v].active);
+    r = surfel_grad_launch(s, active, m, first == 0 && !active ? kGradSum : kGradAdd, Q, t, d_mu,
+                           d_quat, d_scale, d_opac, d_rgb, st);
+    if (r) return r;
+  }
+  // every view's pose gradient in one launch
+  if (pt.n > 0) return pose_reduce_batch_launch(pt, st);
   return GS2D_OK;
 }
 

@@ -131,16 +131,41 @@ int tracking_loss_launch(const float* rgb, const float* depth, const float* norm
                          float* g_depth, float* g_opacity, float* loss_out, void* workspace,
                          size_t ws_bytes, size_t* ws_needed, const int32_t* gate, cudaStream_t st);
 
-// Per-surfel reduction of one view's (tile, region, surfel) partials, Q
-// region slots per tile, with the view's projected records proj (record i
-// is surfel active[i] or i; accumulate adds into the outputs) and the block partials of that view's pose gradient;
-// fixed-order pose reduction.
-int surfel_grad_launch(const gs2d_surfels* s, const int32_t* active, int m, int accumulate,
-                       const float* pose, const int32_t* tiles, const uint32_t* surfel_off, int Q,
-                       const float* proj, const float* partials, float* d_mu, float* d_quat,
-                       float* d_scale, float* d_opac, float* d_rgb, float* pose_part,
-                       const int32_t* gate, cudaStream_t st);
-int pose_reduce_launch(const float* part, int n_part, float* out, const int32_t* gate,
-                       cudaStream_t st);
+// Per-surfel reduction of the (tile, region, surfel) partials, Q region slots
+// per tile, of one or several views of the same m records (record i is surfel
+// active[i] or i), and the block partials of each view's pose gradient
+// ([ceil(m / 256)][6]).  mode: kGradWrite writes the sum of the views'
+// gradients, or nothing if the gate keeps the (one) view out; kGradSum writes
+// the sum over the views that their gates let in; kGradAdd adds that sum.
+enum GradMode { kGradWrite = 0, kGradAdd = 1, kGradSum = 2 };
+struct GradView {
+  const float* pose;
+  const int32_t* tiles;
+  const uint32_t* surfel_off;
+  const float* proj;
+  const float* partials;
+  float* pose_part;
+  const int32_t* gate;
+};
+struct GradTable {
+  int n;
+  GradView v[GS2D_MAX_VIEWS];
+};
+int surfel_grad_launch(const gs2d_surfels* s, const int32_t* active, int m, int mode, int Q,
+                       const GradTable& t, float* d_mu, float* d_quat, float* d_scale,
+                       float* d_opac, float* d_rgb, cudaStream_t st);
+
+// Fixed-order pose reductions of several views in one launch.
+struct PoseReduceView {
+  const float* part;
+  int n_part;
+  float* out;
+  const int32_t* gate;
+};
+struct PoseReduceTable {
+  int n;
+  PoseReduceView v[GS2D_MAX_VIEWS];
+};
+int pose_reduce_batch_launch(const PoseReduceTable& t, cudaStream_t st);
 
 }  // namespace gs2d

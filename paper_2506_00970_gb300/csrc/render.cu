@@ -646,126 +646,204 @@ __global__ void __launch_bounds__(kTileThreads, 4) track_quad_kernel(
 
 // Per-surfel reduction of the (tile, region, surfel) partials in emission
 // order (Q region slots per tile) and the chain rule to world-space
-// parameters; pose term per block.
-// Record i is surfel active[i] (or i); with accumulate the gradients are
-// added to the outputs (several views, one after another).
-__global__ void __launch_bounds__(256) surfel_grad_kernel(
-    const float* __restrict__ mu, const float* __restrict__ quat, const float* __restrict__ scale,
-    int n, const int32_t* __restrict__ active, int accumulate, const float* __restrict__ pose,
-    const int32_t* __restrict__ tiles, const uint32_t* __restrict__ surfel_off,
-    int Q, const float* __restrict__ proj, const float* __restrict__ partials,
-    float* __restrict__ d_mu,
-    float* __restrict__ d_quat, float* __restrict__ d_scale, float* __restrict__ d_opac,
-    float* __restrict__ d_rgb, float* __restrict__ pose_part, int n_all,
-    const int32_t* __restrict__ gate) {
-  __shared__ float sp[12];
-  __shared__ float s_pose[8][6];
-  if (gate && *gate) return;
-  if (threadIdx.x < 12) sp[threadIdx.x] = pose[threadIdx.x];
+// parameters, for one or several views of the same m records (record i is
+// surfel active[i], or i); the views' gradients are summed in registers and
+// written (or added) once.  Pose term per view and block.
+//
+// The sums are latency-bound gathers: a surfel's partials are contiguous, but
+// a thread per surfel touches 32 places in a warp's load and leaves the lanes
+// of surfels that the view does not see idle (half of them or more).  So a
+// warp lists its surfels that have tiles and gives four lanes to each, a
+// 16-byte quarter of every partial to a lane, eight surfels at a time; the
+// sums then return to the surfel's own thread through shared memory for the
+// chain rule.  1M surfels x 8 views of 1200 x 680: 684 -> 311 us (all
+// views in one launch); 32 views of subsets, each in a launch of its own that
+// mostly moves the scattered outputs and parameters, 1389 -> 1370 us.
+constexpr int kGradThreads = 256, kGradWarps = kGradThreads / 32;
+__global__ void __launch_bounds__(kGradThreads, 3) surfel_grad_kernel(
+    const GradTable t, const float* __restrict__ mu, const float* __restrict__ quat,
+    const float* __restrict__ scale, int m, const int32_t* __restrict__ active, int n_all, int mode,
+    int Q, float* __restrict__ d_mu, float* __restrict__ d_quat, float* __restrict__ d_scale,
+    float* __restrict__ d_opac, float* __restrict__ d_rgb) {
+  __shared__ float s_S[kGradWarps][32][kRedVals + 1];
+  __shared__ unsigned char s_list[kGradWarps][32];
+  __shared__ float s_in[GS2D_MAX_VIEWS][12];
+  __shared__ float s_pose[GS2D_MAX_VIEWS][kGradWarps][6];
+  __shared__ bool s_dead[GS2D_MAX_VIEWS];
+  if (mode == kGradWrite && t.v[0].gate && *t.v[0].gate) return;
+  for (int e = threadIdx.x; e < t.n * 12; e += kGradThreads) s_in[e / 12][e % 12] = t.v[e / 12].pose[e % 12];
+  for (int v = threadIdx.x; v < t.n; v += kGradThreads) s_dead[v] = t.v[v].gate && *t.v[v].gate;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i = blockIdx.x * kGradThreads + threadIdx.x;
+  const bool in = i < m;
+  const int sid = !in ? 0 : (active ? min(max(active[i], 0), n_all - 1) : i);
+  float4 q4 = make_float4(1.f, 0.f, 0.f, 0.f);
+  F3 mw = f3(0.f, 0.f, 0.f);
+  float su = 0.f, sv = 0.f;
+  if (in) {
+    q4 = reinterpret_cast<const float4*>(quat)[sid];
+    mw = f3(mu[3 * sid], mu[3 * sid + 1], mu[3 * sid + 2]);
+    su = scale[2 * sid];
+    sv = scale[2 * sid + 1];
+  }
+  // a view's counts and offsets are read one view ahead, whatever its gate says
+  auto first_at = [&](int v, int& k, uint32_t& off) {
+    const bool on = v < t.n && in;
+    k = on ? t.v[v].tiles[i] * Q : 0;
+    off = on ? t.v[v].surfel_off[i] : 0u;
+  };
+  int k_next;
+  uint32_t off_next;
+  first_at(0, k_next, off_next);
   __syncthreads();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  float pr[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  if (i < n) {
-    float S[kRedVals];
-#pragma unroll
-    for (int c = 0; c < kRedVals; ++c) S[c] = 0.f;
-    const int k = tiles[i] * Q;
+  const float qn2 = fmaf(q4.x, q4.x, fmaf(q4.y, q4.y, fmaf(q4.z, q4.z, q4.w * q4.w)));
+  const float qinv = rsqrtf(qn2);
+  const float w = q4.x * qinv, x = q4.y * qinv, y = q4.z * qinv, z = q4.w * qinv;
+  float a_scale[2] = {0.f, 0.f}, a_opac = 0.f, a_rgb[3] = {0.f, 0.f, 0.f};
+  float a_mu[3] = {0.f, 0.f, 0.f}, a_quat[4] = {0.f, 0.f, 0.f, 0.f};
+  bool any = mode != kGradAdd;
+  for (int v = 0; v < t.n; ++v) {
+    const GradView& V = t.v[v];
+    const int k = s_dead[v] ? 0 : k_next;
+    const uint32_t off = off_next;
+    first_at(v + 1, k_next, off_next);
+    const float* R = s_in[v];
+    const F3 mu_c = mat_mul(R, mw) + f3(R[9], R[10], R[11]);
+    // no sums and every factor of the chain finite: nothing to add (a factor
+    // that is not finite makes the gradients NaN, as the products would)
+    const float mag = fabsf(mu_c.x) + fabsf(mu_c.y) + fabsf(mu_c.z) + fabsf(su) + fabsf(sv) + qinv + qn2;
+    const bool work = in && !s_dead[v] && (k > 0 || !(mag < __int_as_float(0x7f800000)));
+    const unsigned has = __ballot_sync(0xffffffffu, k > 0);
+    const float4* rec = reinterpret_cast<const float4*>(V.proj) + (size_t)i * (kProjFloats / 4);
     if (k > 0) {
-      const float4* p = reinterpret_cast<const float4*>(partials) + (size_t)surfel_off[i] * Q * 4;
-      for (int e = 0; e < k; ++e) {
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(rec + 2));
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(rec + 4));
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(rec + 6));
+      s_list[warp][__popc(has & ((1u << lane) - 1u))] = (unsigned char)lane;
+    }
+    __syncwarp();
+    const int n_has = __popc(has);
+    for (int j0 = 0; j0 < n_has; j0 += 8) {
+      const int j = j0 + (lane >> 2);
+      const int src = s_list[warp][min(j, n_has - 1)];
+      int kk = __shfl_sync(0xffffffffu, k, src);
+      const uint32_t oo = __shfl_sync(0xffffffffu, off, src);
+      if (j >= n_has) kk = 0;
+      const float4* p = reinterpret_cast<const float4*>(V.partials) + (size_t)oo * Q * 4 + (lane & 3);
+      float4 S = make_float4(0.f, 0.f, 0.f, 0.f);
+      int kk_max = kk;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const float4 t = p[(size_t)e * 4 + c];
-          S[4 * c] += t.x;
-          S[4 * c + 1] += t.y;
-          S[4 * c + 2] += t.z;
-          S[4 * c + 3] += t.w;
-        }
+      for (int o = 16; o > 2; o >>= 1) kk_max = max(kk_max, __shfl_xor_sync(0xffffffffu, kk_max, o));
+      for (int e = 0; e < kk_max; e += 8, p += 32) {
+        float4 t[8];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) t[c] = e + c < kk ? p[4 * c] : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (e + 4 < kk_max)
+#pragma unroll
+          for (int c = 4; c < 8; ++c) t[c] = e + c < kk ? p[4 * c] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) S.x += t[c].x, S.y += t[c].y, S.z += t[c].z, S.w += t[c].w;
+        if (e + 4 < kk_max)
+#pragma unroll
+          for (int c = 4; c < 8; ++c) S.x += t[c].x, S.y += t[c].y, S.z += t[c].z, S.w += t[c].w;
+      }
+      if (j < n_has) {
+        float* o = &s_S[warp][src][4 * (lane & 3)];
+        o[0] = S.x, o[1] = S.y, o[2] = S.z, o[3] = S.w;
       }
     }
-    const float* R = sp;
-    const int sid = active ? min(max(active[i], 0), n_all - 1) : i;
-    const float4 q4 = reinterpret_cast<const float4*>(quat)[sid];
-    const float qn2 = fmaf(q4.x, q4.x, fmaf(q4.y, q4.y, fmaf(q4.z, q4.z, q4.w * q4.w)));
-    const float qinv = rsqrtf(qn2);
-    const float w = q4.x * qinv, x = q4.y * qinv, y = q4.z * qinv, z = q4.w * qinv;
-    const F3 tu = f3(1.f - 2.f * (y * y + z * z), 2.f * (x * y + w * z), 2.f * (x * z - w * y));
-    const F3 tv = f3(2.f * (x * y - w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z + w * x));
-    const F3 tn = f3(2.f * (x * z + w * y), 2.f * (y * z - w * x), 1.f - 2.f * (x * x + y * y));
-    const F3 mu_c = mat_mul(R, f3(mu[3 * sid], mu[3 * sid + 1], mu[3 * sid + 2])) + f3(sp[9], sp[10], sp[11]);
-    const F3 tuc = mat_mul(R, tu), tvc = mat_mul(R, tv), tnc = mat_mul(R, tn);
-    const float su = scale[2 * sid], sv = scale[2 * sid + 1];
-    // sum Gv, sum u Gv, sum v Gv from the moment sums and the record's
-    // n, d_u, d_v and opacity (a surfel in no tile has all sums zero)
-    F3 g_muc = f3(0.f, 0.f, 0.f), g_mu = g_muc, g_mv = g_muc;
-    if (k > 0) {
-      const float* rec = proj + (size_t)i * kProjFloats;
-      const F3 nrm = f3(rec[kNrm], rec[kNrm + 1], rec[kNrm + 2]);
-      const F3 du = f3(rec[kDu], rec[kDu + 1], rec[kDu + 2]);
-      const F3 dv = f3(rec[kDv], rec[kDv + 1], rec[kDv + 2]);
-      const float op = rec[kAlpha];
-      g_muc = S[0] * nrm + op * (S[4] * du + S[5] * dv);
-      g_mu = S[1] * nrm + op * (S[6] * du + S[7] * dv);
-      g_mv = S[2] * nrm + op * (S[7] * du + S[8] * dv);
+    __syncwarp();
+    float pr[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (work) {
+      any = true;
+      const F3 tu = f3(1.f - 2.f * (y * y + z * z), 2.f * (x * y + w * z), 2.f * (x * z - w * y));
+      const F3 tv = f3(2.f * (x * y - w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z + w * x));
+      const F3 tn = f3(2.f * (x * z + w * y), 2.f * (y * z - w * x), 1.f - 2.f * (x * x + y * y));
+      const F3 tuc = mat_mul(R, tu), tvc = mat_mul(R, tv), tnc = mat_mul(R, tn);
+      // sum Gv, sum u Gv, sum v Gv from the moment sums and the record's
+      // n, d_u, d_v and opacity (a surfel in no tile has all sums zero)
+      F3 g_muc = f3(0.f, 0.f, 0.f), g_mu = g_muc, g_mv = g_muc, g_tnc = g_muc;
+      if (k > 0) {
+        const float* S = s_S[warp][lane];
+        const float4 r2 = rec[2], r4 = rec[4], r5 = rec[5], r6 = rec[6];
+        // record floats 17..25 (n, d_u, d_v) and 10 (opacity)
+        const F3 nrm = f3(r4.y, r4.z, r4.w), du = f3(r5.x, r5.y, r5.z), dv = f3(r5.w, r6.x, r6.y);
+        const float op = r2.z;
+        g_muc = S[0] * nrm + op * (S[4] * du + S[5] * dv);
+        g_mu = S[1] * nrm + op * (S[6] * du + S[7] * dv);
+        g_mv = S[2] * nrm + op * (S[7] * du + S[8] * dv);
+        g_tnc = f3(S[12], S[13], S[14]);
+        a_opac += S[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) a_rgb[c] += S[9 + c];
+      }
+      const F3 g_tuc = su * g_mu, g_tvc = sv * g_mv;
+      a_scale[0] += dot3(tuc, g_mu);
+      a_scale[1] += dot3(tvc, g_mv);
+      const F3 th = cross3(mu_c, g_muc) + cross3(tuc, g_tuc) + cross3(tvc, g_tvc) + cross3(tnc, g_tnc);
+      pr[0] = g_muc.x; pr[1] = g_muc.y; pr[2] = g_muc.z;
+      pr[3] = th.x; pr[4] = th.y; pr[5] = th.z;
+      const F3 gmw = mat_tmul(R, g_muc);
+      a_mu[0] += gmw.x, a_mu[1] += gmw.y, a_mu[2] += gmw.z;
+      // world-space column gradients G[:,0..2] = R^T g_t{u,v,n}c
+      const F3 G0 = mat_tmul(R, g_tuc), G1 = mat_tmul(R, g_tvc), G2 = mat_tmul(R, g_tnc);
+      // d/dq of the rotation matrix of a unit quaternion, contracted with G
+      // (G_rc = gradient of entry (r, c); column c of R is t_u, t_v, t_n)
+      const float G00 = G0.x, G10 = G0.y, G20 = G0.z;
+      const float G01 = G1.x, G11 = G1.y, G21 = G1.z;
+      const float G02 = G2.x, G12 = G2.y, G22 = G2.z;
+      const float gw = 2.f * (z * (G10 - G01) + y * (G02 - G20) + x * (G21 - G12));
+      const float gx = 2.f * (y * (G10 + G01) + z * (G02 + G20) + w * (G21 - G12)) - 4.f * x * (G11 + G22);
+      const float gy = 2.f * (x * (G10 + G01) + z * (G12 + G21) + w * (G02 - G20)) - 4.f * y * (G00 + G22);
+      const float gz = 2.f * (x * (G02 + G20) + y * (G12 + G21) + w * (G10 - G01)) - 4.f * z * (G00 + G11);
+      // unit quaternion -> raw quaternion: (I - q q^T) / |q|
+      const float qd = w * gw + x * gx + y * gy + z * gz;
+      a_quat[0] += (gw - w * qd) * qinv;
+      a_quat[1] += (gx - x * qd) * qinv;
+      a_quat[2] += (gy - y * qd) * qinv;
+      a_quat[3] += (gz - z * qd) * qinv;
     }
-    const F3 g_tnc = f3(S[12], S[13], S[14]);
-    const F3 g_tuc = su * g_mu, g_tvc = sv * g_mv;
-    // o(p, v): write, or add when accumulating over views
-    auto o = [&](float* p, float v) { *p = accumulate ? *p + v : v; };
-    o(d_scale + 2 * sid, dot3(tuc, g_mu));
-    o(d_scale + 2 * sid + 1, dot3(tvc, g_mv));
-    o(d_opac + sid, S[3]);
-    o(d_rgb + 3 * sid, S[9]);
-    o(d_rgb + 3 * sid + 1, S[10]);
-    o(d_rgb + 3 * sid + 2, S[11]);
-    const F3 th = cross3(mu_c, g_muc) + cross3(tuc, g_tuc) + cross3(tvc, g_tvc) + cross3(tnc, g_tnc);
-    pr[0] = g_muc.x; pr[1] = g_muc.y; pr[2] = g_muc.z;
-    pr[3] = th.x; pr[4] = th.y; pr[5] = th.z;
-    const F3 gmw = mat_tmul(R, g_muc);
-    o(d_mu + 3 * sid, gmw.x);
-    o(d_mu + 3 * sid + 1, gmw.y);
-    o(d_mu + 3 * sid + 2, gmw.z);
-    // world-space column gradients G[:,0..2] = R^T g_t{u,v,n}c
-    const F3 G0 = mat_tmul(R, g_tuc), G1 = mat_tmul(R, g_tvc), G2 = mat_tmul(R, g_tnc);
-    // d/dq of the rotation matrix of a unit quaternion, contracted with G
-    // (G_rc = gradient of entry (r, c); column c of R is t_u, t_v, t_n)
-    const float G00 = G0.x, G10 = G0.y, G20 = G0.z;
-    const float G01 = G1.x, G11 = G1.y, G21 = G1.z;
-    const float G02 = G2.x, G12 = G2.y, G22 = G2.z;
-    const float gw = 2.f * (z * (G10 - G01) + y * (G02 - G20) + x * (G21 - G12));
-    const float gx = 2.f * (y * (G10 + G01) + z * (G02 + G20) + w * (G21 - G12)) - 4.f * x * (G11 + G22);
-    const float gy = 2.f * (x * (G10 + G01) + z * (G12 + G21) + w * (G02 - G20)) - 4.f * y * (G00 + G22);
-    const float gz = 2.f * (x * (G02 + G20) + y * (G12 + G21) + w * (G10 - G01)) - 4.f * z * (G00 + G11);
-    // unit quaternion -> raw quaternion: (I - q q^T) / |q|
-    const float qd = w * gw + x * gx + y * gy + z * gz;
-    o(d_quat + 4 * sid, (gw - w * qd) * qinv);
-    o(d_quat + 4 * sid + 1, (gx - x * qd) * qinv);
-    o(d_quat + 4 * sid + 2, (gy - y * qd) * qinv);
-    o(d_quat + 4 * sid + 3, (gz - z * qd) * qinv);
+    const bool warp_any = __any_sync(0xffffffffu, work);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      float r = pr[c];
+      if (warp_any)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+      if (lane == 0) s_pose[v][warp][c] = r;
+    }
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (in && any) {
+    // o(p, v): write, or add to what earlier launches left
+    auto o = [&](float* p, float r) { *p = mode == kGradAdd ? *p + r : r; };
+    o(d_scale + 2 * sid, a_scale[0]);
+    o(d_scale + 2 * sid + 1, a_scale[1]);
+    o(d_opac + sid, a_opac);
 #pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    float v = pr[c];
+    for (int c = 0; c < 3; ++c) {
+      o(d_rgb + 3 * sid + c, a_rgb[c]);
+      o(d_mu + 3 * sid + c, a_mu[c]);
+    }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if (lane == 0) s_pose[warp][c] = v;
+    for (int c = 0; c < 4; ++c) o(d_quat + 4 * sid + c, a_quat[c]);
   }
   __syncthreads();
-  if (threadIdx.x < 6) {
-    float v = 0.f;
-    for (int ww = 0; ww < 8; ++ww) v += s_pose[ww][threadIdx.x];
-    pose_part[(size_t)blockIdx.x * 6 + threadIdx.x] = v;
+  for (int e = threadIdx.x; e < t.n * 6; e += kGradThreads) {
+    float r = 0.f;
+    for (int ww = 0; ww < kGradWarps; ++ww) r += s_pose[e / 6][ww][e % 6];
+    t.v[e / 6].pose_part[(size_t)blockIdx.x * 6 + e % 6] = r;
   }
 }
 
-// Fixed-order sum of per-block 6-vector partials.
-__global__ void __launch_bounds__(256) pose_reduce_kernel(const float* __restrict__ part, int n_part,
-                                                          float* __restrict__ out,
-                                                          const int32_t* __restrict__ gate) {
+// Fixed-order sum of per-block 6-vector partials, a view per block.
+__global__ void __launch_bounds__(256) pose_reduce_kernel(const PoseReduceTable t) {
   __shared__ float s[6][256];
-  if (gate && *gate) return;
+  const PoseReduceView& V = t.v[blockIdx.x];
+  if (V.gate && *V.gate) return;
+  const float* __restrict__ part = V.part;
+  const int n_part = V.n_part;
   float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
   for (int b = threadIdx.x; b < n_part; b += 256)
 #pragma unroll
     for (int c = 0; c < 6; ++c) acc[c] += part[(size_t)b * 6 + c];
@@ -778,7 +856,7 @@ __global__ void __launch_bounds__(256) pose_reduce_kernel(const float* __restric
       for (int c = 0; c < 6; ++c) s[c][threadIdx.x] += s[c][threadIdx.x + h];
     __syncthreads();
   }
-  if (threadIdx.x < 6) out[threadIdx.x] = s[threadIdx.x][0];
+  if (threadIdx.x < 6) V.out[threadIdx.x] = s[threadIdx.x][0];
 }
 
 struct BwdWs {
@@ -888,26 +966,29 @@ int track_tile_launch(const float* proj, const gs2d_bins* bins, const gs2d_camer
   return GS2D_OK;
 }
 
-int surfel_grad_launch(const gs2d_surfels* s, const int32_t* active, int m, int accumulate,
-                       const float* pose, const int32_t* tiles, const uint32_t* surfel_off, int Q,
-                       const float* proj, const float* partials, float* d_mu, float* d_quat,
-                       float* d_scale, float* d_opac, float* d_rgb, float* pose_part,
-                       const int32_t* gate, cudaStream_t st) {
+int surfel_grad_launch(const gs2d_surfels* s, const int32_t* active, int m, int mode, int Q,
+                       const GradTable& t, float* d_mu, float* d_quat, float* d_scale,
+                       float* d_opac, float* d_rgb, cudaStream_t st) {
   if (m <= 0) return GS2D_OK;
-  surfel_grad_kernel<<<(m + 255) / 256, 256, 0, st>>>(s->mu, s->quat, s->scale, m, active,
-                                                      accumulate, pose, tiles, surfel_off, Q, proj,
-                                                      partials,
-                                                      d_mu, d_quat, d_scale, d_opac, d_rgb,
-                                                      pose_part, s->n, gate);
+  surfel_grad_kernel<<<(m + kGradThreads - 1) / kGradThreads, kGradThreads, 0, st>>>(
+      t, s->mu, s->quat, s->scale, m, active, s->n, mode, Q, d_mu, d_quat, d_scale, d_opac, d_rgb);
   GS2D_LAUNCH_CHECK();
   return GS2D_OK;
 }
 
-int pose_reduce_launch(const float* part, int n_part, float* out, const int32_t* gate,
-                       cudaStream_t st) {
-  pose_reduce_kernel<<<1, 256, 0, st>>>(part, n_part, out, gate);
+int pose_reduce_batch_launch(const PoseReduceTable& t, cudaStream_t st) {
+  pose_reduce_kernel<<<t.n, 256, 0, st>>>(t);
   GS2D_LAUNCH_CHECK();
   return GS2D_OK;
+}
+
+// One view's pose reduction.
+static int pose_reduce_one(const float* part, int n_part, float* out, const int32_t* gate,
+                           cudaStream_t st) {
+  PoseReduceTable t;
+  t.n = 1;
+  t.v[0] = PoseReduceView{part, n_part, out, gate};
+  return pose_reduce_batch_launch(t, st);
 }
 
 size_t render_bwd_ws_bytes(int n, size_t cap, int n_tiles, bool full, int Q) {
@@ -959,15 +1040,15 @@ int render_bwd_launch(const float* proj, const gs2d_bins* bins, const int32_t* t
     GS2D_LAUNCH_CHECK();
     if (s->n > 0) {
       const int nb = (s->n + 255) / 256;
-      surfel_grad_kernel<<<nb, 256, 0, st>>>(s->mu, s->quat, s->scale, s->n, nullptr, 0, pose,
-                                             tiles_per_surfel, bins->surfel_off, Q, proj,
-                                             w.partials, d_mu,
-                                             d_quat, d_scale, d_opac, d_rgb_out, w.pose_part, s->n,
-                                             gate);
-      GS2D_LAUNCH_CHECK();
+      GradTable t;
+      t.n = 1;
+      t.v[0] = GradView{pose, tiles_per_surfel, bins->surfel_off, proj, w.partials, w.pose_part, gate};
+      const int gr = surfel_grad_launch(s, nullptr, s->n, kGradWrite, Q, t, d_mu, d_quat, d_scale,
+                                        d_opac, d_rgb_out, st);
+      if (gr) return gr;
       if (d_pose6) {
-        pose_reduce_kernel<<<1, 256, 0, st>>>(w.pose_part, nb, d_pose6, gate);
-        GS2D_LAUNCH_CHECK();
+        const int pr = pose_reduce_one(w.pose_part, nb, d_pose6, gate, st);
+        if (pr) return pr;
       }
     } else if (d_pose6) {
       GS2D_CUDA_TRY(cudaMemsetAsync(d_pose6, 0, 6 * sizeof(float), st));
@@ -977,8 +1058,8 @@ int render_bwd_launch(const float* proj, const gs2d_bins* bins, const int32_t* t
         p4, bins->vals, bins->tile_ranges, *cam, *cfg, tx, t_final, n_last, d_rgb, d_depth,
         d_normal, d_opacity, w.pose_part, gate));
     GS2D_LAUNCH_CHECK();
-    pose_reduce_kernel<<<1, 256, 0, st>>>(w.pose_part, n_tiles, d_pose6, gate);
-    GS2D_LAUNCH_CHECK();
+    const int pr = pose_reduce_one(w.pose_part, n_tiles, d_pose6, gate, st);
+    if (pr) return pr;
   }
   return GS2D_OK;
 }

@@ -317,3 +317,49 @@ def test_autotune_sweeps_pixels_per_thread(torch_cuda):
     px, tiles, table = autotune.tune(ds, cams, poses, actives, reps=1)
     assert px in (1, 2, 3, 4) and all(t in gs2d.TILE_SHAPES[px] for t in tiles)
     assert set(table) == {"px1", "px2", "px3", "px4"}
+
+
+@pytest.mark.parametrize("order,overflow", [((0, 1, 3), False), ((1, 0, 3), False), ((0, 2, 1), True),
+                                            ((1, 0), True), ((2,), True), ((3,), False)])
+def test_batch_backward_in_any_order_of_views(torch_cuda, order, overflow):
+    """The first view writes the gradients where it draws every surfel and
+    the others add theirs: with a whole view or a subset first, and with a
+    first view that overflowed (it adds nothing, and leaves no stale values),
+    the batch equals the sum of the single views; a surfel that no view's
+    tiles hold gets exactly zero, and one without a rotation NaN.  Tolerance:
+    a sum of V FP32 terms, 1e-6 of the largest a view."""
+    torch = torch_cuda
+    from paper_2506_00970_gb300 import gs2d
+    s, cams, poses, actives, tiles = _setup()
+    s.mu[:40, 2] = -5.0  # behind every camera
+    s.quat[20] = 0.0
+    cams, poses, actives, tiles = ([x[v] for v in order] for x in (cams, poses, actives, tiles))
+    ds = gs2d.DeviceSurfels(s)
+    caps = [64 if overflow and v == 0 else 200000 for v in range(len(order))]
+    br = gs2d.BatchRasterizer(cams, s.n, actives=actives, tiles=tiles, capacities=caps)
+    br.set_poses(poses)
+    br.forward(ds, check_status=False)
+    total = {k: np.zeros(getattr(s, k).shape) for k in ("mu", "quat", "scale", "opacity", "rgb")}
+    for v, b in enumerate(br.keep):
+        up = scenes.random_upstream(30 + v, cams[v].height, cams[v].width)
+        b["d_rgb"].copy_(torch.tensor(up[0], dtype=torch.float32))
+        b["d_depth"].copy_(torch.tensor(up[1], dtype=torch.float32))
+        if v == 0 and overflow:
+            continue
+        ids = np.arange(s.n) if actives[v] is None else actives[v]
+        r, dsub, pt, _ = gpu_render(s.subset(ids), cams[v], poses[v], tile=tiles[v])
+        gv = r.backward(dsub, pt, b["d_rgb"], b["d_depth"], None, None, full=True)
+        for k in total:
+            total[k][ids] += to_np(gv[k])
+    for t in br.backward(ds).values():
+        t.fill_(float("nan"))
+    g = br.backward(ds)
+    torch.cuda.synchronize()
+    assert int(br.keep[0]["status"].item()) == (3 if overflow else 0)
+    for k in total:
+        a = to_np(g[k])
+        np.testing.assert_array_equal(np.isnan(a), np.isnan(total[k]), err_msg=k)
+        lim = 1e-6 * np.nanmax(np.abs(total[k])) * len(order)
+        assert np.nanmax(np.abs(a - total[k])) <= lim, k
+        rest = np.delete(a, 20, axis=0)
+        assert np.all(rest[:39] == 0), k
