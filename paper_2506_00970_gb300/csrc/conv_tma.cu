@@ -1,4 +1,5 @@
-// Forward 3x3 / stride 2 / padding 1 convolutions of the proposal network
+// 3x3 / stride 2 / padding 1 convolutions of the proposal network: the data
+// gradients of layers 3-6 (dgrad_tma_kernel, below) and the forward passes
 // (layers 2-4: NHWC bfloat16 maps 60x80x32 -> 30x40x64 -> 15x20x128 ->
 // 8x10x256) on the 5th-generation tensor cores with TMA-fed operands.
 //
@@ -69,10 +70,18 @@ __device__ __forceinline__ uint64_t sw_desc(uint32_t saddr) {
   return (uint64_t)((saddr >> 4) & 0x3FFF) | (1ull << 16) |
          ((uint64_t)(((8 * SW) >> 4) & 0x3FFF) << 32) | (1ull << 46) | (mode << 61);
 }
-// Instruction descriptor of kind::f16: f32 accumulate, bf16 A and B, both
-// K-major, N = n, M = 128.
-__host__ __device__ constexpr uint32_t mma_idesc(int n) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) |
+// Descriptor of an operand that is contiguous along its M / N dimension, in
+// 128-byte rows of 64 elements (a row per k) under the 128-byte swizzle:
+// leading offset mn_step between blocks of 64 elements, stride 1024 bytes
+// between groups of 8 k.
+__device__ __forceinline__ uint64_t mn_desc(uint32_t saddr, uint32_t mn_step) {
+  return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((mn_step >> 4) & 0x3FFF) << 16) |
+         ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+// Instruction descriptor of kind::f16: f32 accumulate, bf16 A and B, A
+// K-major, B K-major or contiguous along N, N = n, M = 128.
+__host__ __device__ constexpr uint32_t mma_idesc(int n, bool b_mn = false) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (b_mn ? 1u << 16 : 0u) | ((uint32_t)(n >> 3) << 17) |
          ((uint32_t)(128 >> 4) << 24);
 }
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c0, int c1,
@@ -81,6 +90,14 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
       "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, "
       "{%2, %3, %4, %5}], [%6];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1,
+                                            int c2, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, "
+      "{%2, %3, %4}], [%5];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
       : "memory");
 }
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1,
@@ -116,6 +133,9 @@ struct ConvTma {
   static constexpr int SMEM = S * STAGE + 1024;   // + slack for 1024-byte alignment
   static constexpr int TMEM_COLS = NB;
   static constexpr int NSPLIT = COUT / NB;        // channel groups (grid.y)
+  static constexpr bool B_MN = false;             // weights K-major
+  static constexpr int B_STEP = 32;               // bytes from one K step of 16 to the next
+  static __device__ __forceinline__ uint64_t b_desc(uint32_t saddr) { return sw_desc<SW>(saddr); }
   static_assert((NI == 1 && TW * TH == 128) || (TX == 1 && TY == 1 && ROWS <= 128),
                 "one 128-row MMA tile: a part of one image, or whole images");
   static_assert(KB == 32 || KB == 64, "64- or 128-byte swizzled rows");
@@ -141,21 +161,21 @@ __device__ __forceinline__ void commit_lane0(uint32_t bar) {
       : "memory");
 }
 
-// K steps 0 .. KS - 1 of one tile into the accumulator at tmem, the stages'
+// K steps 0 .. steps - 1 of one tile into the accumulator at tmem, the stages'
 // running number starting at g0.  False when a wait ran out (the steps before
 // it are issued).
 template <class C, int S, int N>
-__device__ __forceinline__ bool mma_steps(uint32_t tmem, int g0, const uint64_t* s_full,
+__device__ __forceinline__ bool mma_steps(uint32_t tmem, int g0, int steps, const uint64_t* s_full,
                                           const uint64_t* s_empty, uint32_t stages,
                                           volatile int* s_consumed) {
   const uint32_t lane = threadIdx.x & 31;
-  const uint64_t a0 = sw_desc<C::SW>(stages), b0 = sw_desc<C::SW>(stages + C::A_BYTES);
+  const uint64_t a0 = sw_desc<C::SW>(stages), b0 = C::b_desc(stages + C::A_BYTES);
   const uint32_t a_lo = (uint32_t)a0, a_hi = (uint32_t)(a0 >> 32);
   const uint32_t b_lo = (uint32_t)b0, b_hi = (uint32_t)(b0 >> 32);
   int st = g0 % S;
   uint32_t phase = (uint32_t)((g0 / S) & 1);
 #pragma unroll 1
-  for (int s = 0; s < C::KS; ++s) {
+  for (int s = 0; s < steps; ++s) {
     if (!bar_wait(smem_u32(s_full + st), phase)) return false;
     *s_consumed = g0 + s + 1;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -164,13 +184,14 @@ __device__ __forceinline__ bool mma_steps(uint32_t tmem, int g0, const uint64_t*
 #pragma unroll
     for (int j = 0; j < C::MMAS; ++j) {
       // K step j of the stage: 16 channels, 32 bytes into every swizzled row
+      // (or 16 rows of 128 bytes)
       asm volatile(
           "{.reg .pred p, q; .reg .b64 da, db;\n"
           "setp.ne.b32 p, %6, 0; setp.eq.u32 q, %7, 0;\n"
           "mov.b64 da, {%1, %2}; mov.b64 db, {%3, %4};\n"
           "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;}\n" ::"r"(tmem),
-          "r"(a_lo + off + 2 * j), "r"(a_hi), "r"(b_lo + off + 2 * j), "r"(b_hi),
-          "r"(mma_idesc(N)), "r"((s > 0 || j > 0) ? 1u : 0u), "r"(lane));
+          "r"(a_lo + off + 2 * j), "r"(a_hi), "r"(b_lo + off + (C::B_STEP / 16) * j), "r"(b_hi),
+          "r"(mma_idesc(N, C::B_MN)), "r"((s > 0 || j > 0) ? 1u : 0u), "r"(lane));
     }
     commit_lane0(smem_u32(s_empty + st));
     if (++st == S) {
@@ -279,7 +300,7 @@ __global__ void __launch_bounds__(kConvThreads) conv_tma_kernel(
                             n = img;   // images past the batch read as zeros
                           }, nb0);
   if (warp == 0) {
-    const int ok = mma_steps<C, S, NB>(tmem, 0, s_full, s_empty, smem_u32(stages), &s_consumed);
+    const int ok = mma_steps<C, S, NB>(tmem, 0, C::KS, s_full, s_empty, smem_u32(stages), &s_consumed);
     // one last commit tracks every MMA issued (all, or those before a failure)
     commit_lane0(smem_u32(&s_done));
     if (!ok) s_fail = 1;
@@ -411,7 +432,7 @@ __global__ void __launch_bounds__(kPersThreads) conv_tma_pers_kernel(
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      ok = mma_steps<C, S, COUT>(tmem + (uint32_t)(buf * C::TMEM_COLS), k * C::KS, s_full, s_empty,
+      ok = mma_steps<C, S, COUT>(tmem + (uint32_t)(buf * C::TMEM_COLS), k * C::KS, C::KS, s_full, s_empty,
                                  smem_u32(stages), &s_consumed);
       if (ok) commit_lane0(smem_u32(&s_tfull[buf]));
     }
@@ -481,6 +502,197 @@ __global__ void __launch_bounds__(kPersThreads) conv_tma_pers_kernel(
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"(2 * C::TMEM_COLS));
+}
+
+// Data gradient of a layer (3-6): dx = mask * (dz convolved with the
+// transposed weights), by parity class (py, px) of the input pixels (iy, ix)
+// = (2 cy + py, 2 cx + px).  A class sees the taps ky = 1 (py = 0) or 0 and 2
+// (py = 1), likewise in x, and under one tap its pixels read neighbouring
+// pixels of dz at the offset (py && ky == 0, px && kx == 0): a plain box of
+// dz, zeros past the edge.  So the product of a class tile (TH x TW class
+// pixels of one image, or NI whole images) with NB input channels is, per tap
+// and 64 output channels, one A box {64 channels, TW, TH, NI} of dz (K-major,
+// as in the forward pass) and the weights' box {NB input channels, tap, 64
+// output channels} as it lies, contiguous along N.  All four classes go in
+// one launch, the ones of most taps first.  A class's sum over taps, then
+// output channels, is cut where the GEMM it replaces split its K range, a
+// tensor-memory accumulator for each of at most Z pieces, added in order in
+// the epilogue: the results are the same bits at any batch, and those of that
+// GEMM.
+//
+// Against gathers in software (cp.async of 16-byte chunks with their index
+// arithmetic, four launches a layer, FP32 partials and a reduction where a
+// class has few tiles), batch 256: layer 3 146 -> 52 us, layer 4 159 -> 41,
+// layer 5 111 -> 24, layer 6 60 -> 20; the training step 1282 -> 898 us.
+template <int CIN, int COUT, int HI, int WI, int TW, int TH, int S, int NI, int NB, int Z>
+struct DgradTma {
+  static constexpr int HO = (HI + 1) / 2, WO = (WI + 1) / 2;  // dz, and the largest class
+  static constexpr int TX = (WO + TW - 1) / TW, TY = (HO + TH - 1) / TH;
+  static constexpr int SW = 128, CB = COUT / 64, MMAS = 4;
+  static constexpr int ROWS = NI * TW * TH;
+  static constexpr int BOX_BYTES = ROWS * SW;
+  static constexpr int A_BYTES = 128 * SW;
+  static constexpr int B_BYTES = 64 * NB * 2;
+  static constexpr int STAGE = A_BYTES + B_BYTES;
+  static constexpr int TX_BYTES = BOX_BYTES + B_BYTES;
+  static constexpr int SMEM = S * STAGE + 1024;
+  static constexpr int TMEM_COLS = Z * NB, NSPLIT = CIN / NB;  // Z accumulators
+  static constexpr bool B_MN = true;
+  static constexpr int B_STEP = 16 * 128;
+  static __device__ __forceinline__ uint64_t b_desc(uint32_t saddr) { return mn_desc(saddr, NB > 64 ? 64 * 128 : 1024); }
+  static_assert(ROWS <= 128 && (NI == 1 || (TX == 1 && TY == 1)), "one 128-row MMA tile");
+  static_assert(COUT % 64 == 0 && (NB == 64 || NB == 128) && CIN % NB == 0, "channel blocks");
+  static_assert(TMEM_COLS <= 512 && (Z & (Z - 1)) == 0, "tensor-memory columns");
+};
+
+template <int CIN, int COUT, int HI, int WI, int TW, int TH, int S, int NI, int NB, int Z>
+__global__ void __launch_bounds__(kConvThreads) dgrad_tma_kernel(
+    const __grid_constant__ CUtensorMap map_dz, const __grid_constant__ CUtensorMap map_w,
+    const bf16* __restrict__ act, bf16* __restrict__ out, int B, int tiles,
+    const DgradSplits splits, int* __restrict__ err) {
+  using C = DgradTma<CIN, COUT, HI, WI, TW, TH, S, NI, NB, Z>;
+  extern __shared__ unsigned char conv_raw[];
+  __shared__ __align__(8) uint64_t s_full[S], s_empty[S], s_done;
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_fail, s_issued, s_consumed;
+  unsigned char* stages = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(conv_raw) + 1023) & ~(uintptr_t)1023);
+  const int cls = 3 - (int)blockIdx.x / tiles, tile = (int)blockIdx.x % tiles;
+  const int py = cls >> 1, px = cls & 1;
+  const int img = NI == 1 ? tile / (C::TX * C::TY) : tile * NI;
+  const int r = NI == 1 ? tile % (C::TX * C::TY) : 0;
+  const int cy0 = (r / C::TX) * TH, cx0 = (r % C::TX) * TW;
+  const int nb0 = (int)blockIdx.y * NB;
+  const int steps = (1 + py) * (1 + px) * C::CB, per = splits.steps[cls];
+  const int warp = threadIdx.x >> 5;
+
+  if (threadIdx.x == 0) {
+    s_fail = 0;
+    s_issued = 0;
+    s_consumed = 0;
+    for (int i = 0; i < S; ++i) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_full[i])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_empty[i])));
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_done)));
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&s_tmem)),
+                 "r"(C::TMEM_COLS));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = s_tmem;
+
+  if (warp == 1) {
+    const uint32_t lane = threadIdx.x & 31;
+    int st = 0, cb = 0, tx = 0, ty = 0;   // channel block and tap of the class
+    uint32_t phase = 1u;
+#pragma unroll 1
+    for (int g = 0; g < steps; ++g) {
+      if (g >= S && !bar_wait(smem_u32(&s_empty[st]), phase)) {
+        if (lane == 0) atomicExch(&s_fail, 1);
+        break;
+      }
+      const uint32_t base = smem_u32(stages) + (uint32_t)st * C::STAGE;
+      const int ky = py ? 2 * ty : 1, kx = px ? 2 * tx : 1;
+      if (lane == 0) {
+        const uint32_t bar = smem_u32(&s_full[st]);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                     "r"(C::TX_BYTES)
+                     : "memory");
+        tma_load_4d(base, &map_dz, 64 * cb, cx0 + (px && kx == 0), cy0 + (py && ky == 0), img, bar);
+#pragma unroll
+        for (int q = 0; q < NB / 64; ++q)
+          tma_load_3d(base + C::A_BYTES + q * 64 * 128, &map_w, nb0 + 64 * q, 3 * ky + kx, 64 * cb, bar);
+      }
+      *reinterpret_cast<volatile int*>(&s_issued) = g + 1;
+      if (++cb == C::CB) {
+        cb = 0;
+        if (++tx > px) {
+          tx = 0;
+          ++ty;
+        }
+      }
+      if (++st == S) {
+        st = 0;
+        phase ^= 1u;
+      }
+    }
+  }
+  if (warp == 0) {
+    bool ok = true;
+    for (int g = 0, z = 0; g < steps && ok; g += per, ++z)
+      ok = mma_steps<C, S, NB>(tmem + (uint32_t)(z * NB), g, min(per, steps - g), s_full, s_empty,
+                               smem_u32(stages), &s_consumed);
+    // one last commit tracks every MMA issued (all, or those before a failure)
+    commit_lane0(smem_u32(&s_done));
+    if (!ok) s_fail = 1;
+  }
+  if (!bar_wait(smem_u32(&s_done), 0u)) atomicExch(&s_fail, 1);
+  __syncthreads();
+  // loads issued but not consumed (after a failure) land before the CTA exits
+  if (threadIdx.x == 32)
+    for (int s = s_consumed; s < s_issued; ++s)
+      bar_wait(smem_u32(&s_full[s % S]), (uint32_t)((s / S) & 1));
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (!*reinterpret_cast<volatile int*>(&s_fail)) {
+    // TMEM lane = row m: image img + m / (TW TH), class pixel (cy0 + q / TW, cx0 + q % TW)
+    const int m = threadIdx.x;
+    const int g = m / (TW * TH), q = m % (TW * TH);
+    const int iy = 2 * (cy0 + q / TW) + py, ix = 2 * (cx0 + q % TW) + px;
+    const bool ok = g < NI && img + g < B && iy < HI && ix < WI;
+    const size_t off = (((size_t)(img + g) * HI + iy) * WI + ix) * CIN + nb0;
+#pragma unroll 1
+    for (int c0 = 0; c0 < NB; c0 += 16) {
+      uint4 mk[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
+      if (ok) {
+        mk[0] = *reinterpret_cast<const uint4*>(act + off + c0);
+        mk[1] = *reinterpret_cast<const uint4*>(act + off + c0 + 8);
+      }
+      float x[16];
+      for (int z = 0; z * per < steps; ++z) {
+        uint32_t v[16];
+        const uint32_t taddr = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(z * NB + c0);
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, "
+            "%10, %11, %12, %13, %14, %15}, [%16];\n"
+            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+              "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
+              "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+            : "r"(taddr));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int j = 0; j < 16; ++j) x[j] = z ? x[j] + __uint_as_float(v[j]) : __uint_as_float(v[j]);
+      }
+      if (ok) {
+        const uint32_t mw[8] = {mk[0].x, mk[0].y, mk[0].z, mk[0].w, mk[1].x, mk[1].y, mk[1].z, mk[1].w};
+        uint32_t packed[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&mw[j]);
+          const float x0 = __bfloat162float(a.x) > 0.f ? x[2 * j] : 0.f;
+          const float x1 = __bfloat162float(a.y) > 0.f ? x[2 * j + 1] : 0.f;
+          const __nv_bfloat162 b2 = __floats2bfloat162_rn(x0, x1);
+          packed[j] = *reinterpret_cast<const uint32_t*>(&b2);
+        }
+        uint4* d = reinterpret_cast<uint4*>(out + off + c0);
+        d[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+        d[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
+      }
+    }
+  } else if (threadIdx.x == 0 && err) {
+    atomicExch(err, 1);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"(C::TMEM_COLS));
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
@@ -609,9 +821,50 @@ int run_pers(const bf16* x, int B, const bf16* w, const float* bias, bf16* out, 
   return GS2D_OK;
 }
 
-}  // namespace
+// dz map: NHWC bfloat16 {C_out, WO, HO, N}, box {64, TW, TH, NI}; weight map:
+// [C_out][9][C_in] as {C_in, 9, C_out}, box {64, 1, 64}; 128-byte swizzle.
+template <int CIN, int COUT, int HI, int WI, int TW, int TH, int S, int NI, int NB, int Z>
+int run_dgrad(const bf16* dz, int B, const bf16* w, const bf16* act, bf16* out,
+              const DgradSplits& splits, int* err, cudaStream_t st) {
+  using C = DgradTma<CIN, COUT, HI, WI, TW, TH, S, NI, NB, Z>;
+  for (int c = 0; c < 4; ++c)
+    if (splits.steps[c] <= 0 || splits.steps[c] * Z < (1 + (c >> 1)) * (1 + (c & 1)) * C::CB)
+      return GS2D_ERR_INVALID_ARG;
+  EncodeTiledFn enc = encode_tiled();
+  if (!enc) return GS2D_ERR_CUDA;
+  if ((reinterpret_cast<uintptr_t>(dz) | reinterpret_cast<uintptr_t>(w) |
+       reinterpret_cast<uintptr_t>(act) | reinterpret_cast<uintptr_t>(out)) & 15)
+    return GS2D_ERR_INVALID_ARG;
+  CUtensorMap mz, mw;
+  const cuuint64_t zdim[4] = {(cuuint64_t)COUT, (cuuint64_t)C::WO, (cuuint64_t)C::HO, (cuuint64_t)B};
+  const cuuint64_t zstr[3] = {(cuuint64_t)COUT * 2, (cuuint64_t)C::WO * COUT * 2,
+                              (cuuint64_t)C::HO * C::WO * COUT * 2};
+  const cuuint32_t zbox[4] = {64, TW, TH, NI}, zes[4] = {1, 1, 1, 1};
+  const cuuint64_t wdim[3] = {(cuuint64_t)CIN, 9, (cuuint64_t)COUT};
+  const cuuint64_t wstr[2] = {(cuuint64_t)CIN * 2, (cuuint64_t)9 * CIN * 2};
+  const cuuint32_t wbox[3] = {64, 1, 64}, wes[3] = {1, 1, 1};
+  if (enc(&mz, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16*>(dz), zdim, zstr, zbox, zes,
+          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+          CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
+      enc(&mw, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<bf16*>(w), wdim, wstr, wbox, wes,
+          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+          CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return GS2D_ERR_CUDA;
+  static std::once_flag smem_once;
+  static cudaError_t smem_err = cudaSuccess;
+  std::call_once(smem_once, [] {
+    smem_err = cudaFuncSetAttribute(dgrad_tma_kernel<CIN, COUT, HI, WI, TW, TH, S, NI, NB, Z>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+  });
+  if (smem_err != cudaSuccess) return GS2D_ERR_CUDA;
+  const int tiles = NI == 1 ? B * C::TX * C::TY : (B + NI - 1) / NI;
+  dgrad_tma_kernel<CIN, COUT, HI, WI, TW, TH, S, NI, NB, Z>
+      <<<dim3(4 * tiles, C::NSPLIT), kConvThreads, C::SMEM, st>>>(mz, mw, act, out, B, tiles, splits, err);
+  GS2D_LAUNCH_CHECK();
+  return GS2D_OK;
+}
 
-bool conv_tma_layer(int layer) { return layer >= 1 && layer <= 5; }
+}  // namespace
 
 // Which form a layer runs in at a batch.  None changes a result: every tile
 // sums its K steps in the same order.  A CTA's time is its chain of K steps
@@ -659,6 +912,19 @@ int conv_tma_forward(int layer, const bf16* x, int B, const bf16* w, const float
     case 5:
       return (B + 20) / 21 * 8 <= kSms ? run<256, 256, 4, 5, 3, 2, 11, 21, 32>(x, B, w, bias, out, err, st)
                                        : run<256, 256, 4, 5, 3, 2, 5, 21, 32>(x, B, w, bias, out, err, st);
+    default: return GS2D_ERR_INVALID_ARG;
+  }
+}
+
+// Tiles: layer 3's 15 x 20 class pixels in three parts of 6 rows, layer 4's 8
+// x 10 whole, 6 images' 4 x 5 of layer 5, 21 images' 2 x 3 of layer 6.
+int dgrad_tma(int layer, const bf16* dz, int B, const bf16* w, const bf16* act, bf16* out,
+              const DgradSplits& splits, int* err, cudaStream_t st) {
+  switch (layer) {
+    case 2: return run_dgrad<64, 128, 30, 40, 20, 6, 3, 1, 64, 1>(dz, B, w, act, out, splits, err, st);
+    case 3: return run_dgrad<128, 256, 15, 20, 10, 8, 3, 1, 128, 2>(dz, B, w, act, out, splits, err, st);
+    case 4: return run_dgrad<256, 256, 8, 10, 5, 4, 4, 6, 64, 2>(dz, B, w, act, out, splits, err, st);
+    case 5: return run_dgrad<256, 256, 4, 5, 3, 2, 8, 21, 64, 8>(dz, B, w, act, out, splits, err, st);
     default: return GS2D_ERR_INVALID_ARG;
   }
 }

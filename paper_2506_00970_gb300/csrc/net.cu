@@ -2,26 +2,19 @@
 // starting pose of the tracking loop of Sec. III-D): forward, loss,
 // backward and AdamW on BF16 tensor cores with FP32 accumulation.
 //
-// Every contraction of the network but the first layer's forward (a direct
-// convolution kernel, conv_s2_kernel below) -- each convolution's forward
-// (implicit im2col GEMM), data gradient (stride-2 transposed gather) and
-// weight gradient (split-K GEMM over the pixels), and each fully connected
-// layer's three products -- runs through one tiled GEMM kernel
+// The convolutions' forward and data gradients have kernels of their own (the
+// first layer's forward and the first two layers' gradients are direct
+// kernels below, the others' are in conv_tma.cu).  The weight gradients of
+// layers 3-6 (split-K GEMM over the pixels) and each fully connected layer's
+// three products run through one tiled GEMM kernel
 //     C[M, N] = sum_k A[m, k] B[n, k]
 // whose operand tiles are gathered straight from the NHWC activations and
 // the weights by an address mode (no im2col buffer is materialised):
 //   K-major modes (8 consecutive k of one row are contiguous):
 //     K_DENSE   row-major [rows][ld] matrix
-//     K_IM2COL  conv forward: row = (b, oy, ox), k = tap * C + c
-//     K_DGRADP  conv data gradient of one parity class (py, px) of the input
-//               pixels: row = (b, cy, cx) -> pixel (2 cy + py, 2 cx + px),
-//               k = t * C_out + co over the class's taps t, reading dZ at
-//               ((iy + 1 - ky) / 2, (ix + 1 - kx) / 2)
 //   row-major modes (8 consecutive rows of one k are contiguous):
 //     R_DENSE   element (row, k) at p[k * ld + row]
 //     R_IM2COL  conv weight gradient: row = tap * C + c, k = (b, oy, ox)
-//     R_WTP     conv weights read transposed for a parity class:
-//               row = c_in, k = t * C_out + co
 // Pixel and tap indices come from shifts (channel counts are powers of two)
 // and precomputed reciprocal multiplies (no integer division in the loop).
 // Tiles of 128 x 64 x 32 move global -> shared memory with 16-byte cp.async
@@ -46,8 +39,8 @@ namespace net {
 typedef __nv_bfloat16 bf16;
 
 enum Mode {
-  K_DENSE = 0, K_IM2COL = 1, K_DGRADP = 3,  // K-major
-  R_DENSE = 4, R_IM2COL = 5, R_WTP = 7      // row-major
+  K_DENSE = 0,                // K-major
+  R_DENSE = 4, R_IM2COL = 5   // row-major
 };
 enum Epi { E_BIAS_RELU = 0, E_BIAS_F32 = 1, E_MASK = 2, E_PARTIAL = 3 };
 
@@ -81,25 +74,12 @@ __device__ __forceinline__ int fdiv(int n, FastDiv f) {
 
 struct Operand {
   const bf16* p;
-  int ld;                // dense modes: leading dimension; R_WTP: C_out
+  int ld;                // dense modes: leading dimension
   int rows;              // valid rows (M or N); multiple of 8 for row-major modes
   int H, W, C, Ho, Wo;   // conv geometry (input H x W x C, output Ho x Wo)
-  int py, px, Hc, Wc;    // parity class of the data gradient (K_DGRADP, R_WTP)
   int c_shift;           // log2 C (channel counts are powers of two)
-  int ld_shift;          // log2 ld (R_WTP)
   FastDiv f_hw, f_w;     // pixels per image and per row of the indexed pixel grid
 };
-
-// Taps of a parity class of the stride-2 data gradient: input row iy gets
-// contributions from ky = 1 when iy is even and ky in {0, 2} when it is odd
-// (iy + 1 - ky must be even); likewise for columns.  Tap t of the class is
-// (t / nx, t % nx) over its ny x nx taps.
-__device__ __forceinline__ void class_tap(int py, int px, int t, int& ky, int& kx) {
-  const int nx = px ? 2 : 1;
-  const int tyi = t / nx, txi = t - tyi * nx;
-  ky = py ? 2 * tyi : 1;
-  kx = px ? 2 * txi : 1;
-}
 
 struct Gemm {
   int M, N, K, k_split;
@@ -110,9 +90,6 @@ struct Gemm {
   const bf16* mask;
   int n_valid;
   void* part;            // split-K partials [S][M][N] (FP32)
-  // output row remap of a parity-class data gradient: GEMM row (b, cy, cx)
-  // -> pixel (b, 2 cy + py, 2 cx + px) of an H x W map
-  int remap, rH, rW, rHc, rWc, rpy, rpx;
   int* err;              // set to 1 by a tensor-core kernel whose wait timed out
 };
 
@@ -164,8 +141,7 @@ template <int MODE, int ROWS, int NT = THREADS, int KB = BK>
 struct Loader {
   static constexpr int kVec = ROWS * KB / 8;
   static constexpr int kPer = kVec / NT;  // 16-byte vectors per thread and stage
-  const bf16* base[kPer];  // K-major: row start (dense) or image start (gathers)
-  int iy0[kPer], ix0[kPer];
+  const bf16* base[kPer];  // K-major: row start
   bool ok[kPer];
   int ky, kx, c;            // R_IM2COL: the row group's tap and channel
 
@@ -176,27 +152,11 @@ struct Loader {
       if (is_kmajor<MODE>()) {
         const int row = r0 + v / (KB / 8);
         ok[i] = row < o.rows;
-        iy0[i] = ix0[i] = 0;
-        if (MODE == K_DENSE) {
-          base[i] = o.p + (size_t)row * o.ld;
-        } else if (MODE == K_IM2COL) {
-          const int b = fdiv(row, o.f_hw), r = row - b * o.Ho * o.Wo;
-          const int oy = fdiv(r, o.f_w), ox = r - oy * o.Wo;
-          base[i] = o.p + (size_t)b * o.H * o.W * o.C;
-          iy0[i] = 2 * oy - 1;
-          ix0[i] = 2 * ox - 1;
-        } else {  // K_DGRADP
-          const int b = fdiv(row, o.f_hw), r = row - b * o.Hc * o.Wc;
-          const int cy = fdiv(r, o.f_w), cx = r - cy * o.Wc;
-          base[i] = o.p + (size_t)b * o.Ho * o.Wo * o.C;
-          iy0[i] = 2 * cy + o.py;
-          ix0[i] = 2 * cx + o.px;
-        }
+        base[i] = o.p + (size_t)row * o.ld;
       } else {
         const int row0 = r0 + (v % (ROWS / 8)) * 8;
         ok[i] = row0 < o.rows;
         base[i] = o.p;
-        iy0[i] = ix0[i] = 0;
       }
     }
     ky = kx = c = 0;
@@ -211,36 +171,18 @@ struct Loader {
 
   __device__ __forceinline__ const bf16* kaddr(const Operand& o, int i, int k, int kend) const {
     if (!ok[i] || k >= kend) return nullptr;
-    if (MODE == K_DENSE) return base[i] + k;
-    const int tap = k >> o.c_shift, ch = k & ((1 << o.c_shift) - 1);
-    if (MODE == K_IM2COL) {
-      const int tky = tap / 3, tkx = tap - tky * 3;
-      const int iy = iy0[i] + tky, ix = ix0[i] + tkx;
-      if (iy < 0 || iy >= o.H || ix < 0 || ix >= o.W) return nullptr;
-      return base[i] + ((size_t)iy * o.W + ix) * o.C + ch;
-    }
-    int tky, tkx;  // K_DGRADP
-    class_tap(o.py, o.px, tap, tky, tkx);
-    const int oy = (iy0[i] + 1 - tky) >> 1, ox = (ix0[i] + 1 - tkx) >> 1;
-    if (oy < 0 || oy >= o.Ho || ox < 0 || ox >= o.Wo) return nullptr;
-    return base[i] + ((size_t)oy * o.Wo + ox) * o.C + ch;
+    return base[i] + k;
   }
 
   __device__ __forceinline__ const bf16* raddr(const Operand& o, int i, int row0, int k,
                                                int kend) const {
     if (!ok[i] || k >= kend) return nullptr;
     if (MODE == R_DENSE) return o.p + (size_t)k * o.ld + row0;
-    if (MODE == R_IM2COL) {
-      const int b = fdiv(k, o.f_hw), r = k - b * o.Ho * o.Wo;
-      const int oy = fdiv(r, o.f_w), ox = r - oy * o.Wo;
-      const int iy = 2 * oy - 1 + ky, ix = 2 * ox - 1 + kx;
-      if (iy < 0 || iy >= o.H || ix < 0 || ix >= o.W) return nullptr;
-      return o.p + (((size_t)b * o.H + iy) * o.W + ix) * o.C + c;
-    }
-    const int t = k >> o.ld_shift, co = k & ((1 << o.ld_shift) - 1);  // R_WTP
-    int tky, tkx;
-    class_tap(o.py, o.px, t, tky, tkx);
-    return o.p + ((size_t)co * 9 + tky * 3 + tkx) * o.C + row0;
+    const int b = fdiv(k, o.f_hw), r = k - b * o.Ho * o.Wo;  // R_IM2COL
+    const int oy = fdiv(r, o.f_w), ox = r - oy * o.Wo;
+    const int iy = 2 * oy - 1 + ky, ix = 2 * ox - 1 + kx;
+    if (iy < 0 || iy >= o.H || ix < 0 || ix >= o.W) return nullptr;
+    return o.p + (((size_t)b * o.H + iy) * o.W + ix) * o.C + c;
   }
 
   // One stage in the tcgen05 operand layout: 8 x 8 core matrices of 128
@@ -304,29 +246,21 @@ __device__ __forceinline__ void frag_b(uint32_t b[4], const bf16* s, int n0, int
     ldsm_x4_t(b, s + (k0 + 8 * (i & 1) + rr) * (ROWS + PAD) + n0 + 8 * (i >> 1));
 }
 
-// Output offset of GEMM row `row` (times the row stride ldc).
-__device__ __forceinline__ size_t out_row(const Gemm& g, int row) {
-  if (!g.remap) return (size_t)row;
-  const int hw = g.rHc * g.rWc;
-  const int b = row / hw, r = row - b * hw, cy = r / g.rWc, cx = r - cy * g.rWc;
-  return ((size_t)b * g.rH + 2 * cy + g.rpy) * g.rW + 2 * cx + g.rpx;
-}
-
 template <int EPI>
 __device__ __forceinline__ void apply_epi(const Gemm& g, int row, int col, float v0, float v1) {
   if (row >= g.M) return;
   if (EPI == E_BIAS_RELU) {
     if (col >= g.N) return;
     const float x0 = fmaxf(v0 + g.bias[col], 0.f), x1 = fmaxf(v1 + g.bias[col + 1], 0.f);
-    *reinterpret_cast<__nv_bfloat162*>(static_cast<bf16*>(g.out) + out_row(g, row) * g.ldc + col) =
+    *reinterpret_cast<__nv_bfloat162*>(static_cast<bf16*>(g.out) + (size_t)row * g.ldc + col) =
         __floats2bfloat162_rn(x0, x1);
   } else if (EPI == E_BIAS_F32) {
-    float* o = static_cast<float*>(g.out) + out_row(g, row) * g.ldc;
+    float* o = static_cast<float*>(g.out) + (size_t)row * g.ldc;
     if (col < g.n_valid) o[col] = v0 + g.bias[col];
     if (col + 1 < g.n_valid) o[col + 1] = v1 + g.bias[col + 1];
   } else if (EPI == E_MASK) {
     if (col >= g.N) return;
-    const size_t off = out_row(g, row) * g.ldc + col;
+    const size_t off = (size_t)row * g.ldc + col;
     const __nv_bfloat162 m = *reinterpret_cast<const __nv_bfloat162*>(g.mask + off);
     const float x0 = __bfloat162float(m.x) > 0.f ? v0 : 0.f;
     const float x1 = __bfloat162float(m.y) > 0.f ? v1 : 0.f;
@@ -1612,7 +1546,6 @@ int splits_count(int K, int s) {
   const int ks = s > 1 ? k_split_for(K, s) : (int)align_up((size_t)K, 64);
   return max((K + ks - 1) / ks, 1);
 }
-int class_hc(int H, int py) { return (H + 1 - py) / 2; }
 
 // Rows per block of the bias-gradient column sums: about 304 blocks, a
 // multiple of the rows one pass of the block covers (256 / (C / 8)).
@@ -1639,11 +1572,6 @@ size_t max_partials(int B) {
     const int rows = B * kHin[l + 1] * kWin[l + 1];
     const int rpb = colsum_rows_per_block(rows, kCout[l]);
     mx = max(mx, (size_t)((rows + rpb - 1) / rpb) * kCout[l]);
-    nom(kHin[l + 1] * kWin[l + 1], kCout[l], 9 * kCin[l]);
-    for (int py = 0; py < 2; ++py)
-      for (int px = 0; px < 2; ++px)
-        nom(class_hc(kHin[l], py) * class_hc(kWin[l], px), kCin[l],
-            (py ? 2 : 1) * (px ? 2 : 1) * kCout[l]);
   }
   upd(kHidden, kFlat, B);
   upd(kOutPad, kHidden, B);
@@ -1694,7 +1622,7 @@ int log2_exact(int v) {
   while ((1 << s) < v) ++s;
   return s;
 }
-// Gathers over the output grid of conv layer l (K_IM2COL, R_IM2COL) with C
+// Gathers over the output grid of conv layer l (R_IM2COL) with C
 // channels of the gathered tensor (a power of two).
 Operand conv_op(const bf16* p, int rows, int l, int C) {
   Operand o{};
@@ -1711,12 +1639,10 @@ Operand conv_op(const bf16* p, int rows, int l, int C) {
   return o;
 }
 
-// Launches one GEMM.  Split-K partial products (the deep-K weight
-// gradients and the split deep layers) run on the tcgen05 kernel; GEMMs with
-// a direct epilogue (large M, the gather-bound convolutions) on the mma.sync
-// kernel, whose smaller blocks keep more warps resident to hide the gathers
-// (measured on the batch-256 training step: all mma.sync 2.38 ms, this split
-// 2.46 ms, all tcgen05 3.19 ms).
+// Launches one GEMM.  Split-K partial products (the deep-K weight gradients
+// and the fully connected layers) run on the tcgen05 kernel; GEMMs with a
+// direct epilogue (the few-row fully connected data gradient that is not
+// split) on the mma.sync kernel.
 template <int AM, int BMODE, int EPI>
 int run(Gemm g, int splits, cudaStream_t st, int* n_splits = nullptr) {
   constexpr bool tc = EPI == E_PARTIAL;
@@ -1744,7 +1670,7 @@ int run(Gemm g, int splits, cudaStream_t st, int* n_splits = nullptr) {
   return GS2D_OK;
 }
 
-// A forward or data-gradient GEMM with its epilogue: split-K (at the
+// A fully connected forward or data-gradient GEMM with its epilogue: split-K (at the
 // nominal-batch count for rows_per_sample) through FP32 partials and a
 // fixed-order reduction when the tile grid is small.
 template <int AM, int BMODE, int EPI>
@@ -1884,25 +1810,8 @@ int forward(const float* params, const bf16* x, int B, const Ws& w, float* y, cu
   if (r) return r;
   const bf16* in = w.act[1];
   for (int l = 1; l < kConv; ++l) {
-    if (conv_tma_layer(l)) {
-      // layers 2-4: tcgen05 with TMA-fed operands
-      r = conv_tma_forward(l, in, B, w.wbf + L.wbf_off[l], params + L.b_off[l], w.act[l + 1],
-                           w.err, st);
-      if (r) return r;
-      in = w.act[l + 1];
-      continue;
-    }
-    Gemm g{};
-    g.err = w.err;
-    g.M = B * kHin[l + 1] * kWin[l + 1];
-    g.N = kCout[l];
-    g.K = 9 * kCin[l];
-    g.a = conv_op(in, g.M, l, kCin[l]);
-    g.b = op(w.wbf + L.wbf_off[l], g.K, g.N);
-    g.out = w.act[l + 1];
-    g.ldc = g.N;
-    g.bias = params + L.b_off[l];
-    r = fused<K_IM2COL, K_DENSE, E_BIAS_RELU>(g, kHin[l + 1] * kWin[l + 1], w.part, st);
+    // layers 2-6: tcgen05 with TMA-fed operands
+    r = conv_tma_forward(l, in, B, w.wbf + L.wbf_off[l], params + L.b_off[l], w.act[l + 1], w.err, st);
     if (r) return r;
     in = w.act[l + 1];
   }
@@ -2020,50 +1929,18 @@ int backward(const float* params, const bf16* x, int B, const Ws& w, float* grad
       r = bias_grad(cur, P, kCout[l], kCout[l], w.part, grad + L.b_off[l], st);
       if (r) return r;
     }
-    // data gradient: layer 2's by its direct kernel; the others by one GEMM
-    // per parity class of the input pixels, each with only the taps that
-    // reach it (9 taps over the 4 classes)
-    if (l == 1) {
-      r = dgrad2(cur, B, w.wbf + L.wbf_off[1], w.act[1], nxt, st);
-      if (r) return r;
+    // data gradient: layer 2's by its direct kernel, the others' on TMA-fed
+    // tensor-core tiles
+    DgradSplits sp;
+    for (int c = 0; c < 4; ++c) {
+      const int hc = (kHin[l] + 1 - (c >> 1)) / 2, wc = (kWin[l] + 1 - (c & 1)) / 2;
+      const int K = (1 + (c >> 1)) * (1 + (c & 1)) * kCout[l];
+      const int s = splits_nominal(hc * wc, kCin[l], K);
+      sp.steps[c] = (s > 1 ? k_split_for(K, s) : K) / 64;
     }
-    for (int py = 0; py < 2 && l != 1; ++py)
-      for (int px = 0; px < 2; ++px) {
-        const int Hc = class_hc(kHin[l], py), Wc = class_hc(kWin[l], px);
-        Gemm d{};
-        d.err = w.err;
-        d.M = B * Hc * Wc;
-        d.N = kCin[l];
-        d.K = (py ? 2 : 1) * (px ? 2 : 1) * kCout[l];
-        d.a = conv_op(cur, d.M, l, kCout[l]);
-        d.a.py = py;
-        d.a.px = px;
-        d.a.Hc = Hc;
-        d.a.Wc = Wc;
-        d.a.f_hw = make_fastdiv((uint32_t)(Hc * Wc));
-        d.a.f_w = make_fastdiv((uint32_t)Wc);
-        Operand wt{};
-        wt.p = w.wbf + L.wbf_off[l];
-        wt.ld = kCout[l];
-        wt.ld_shift = log2_exact(kCout[l]);
-        wt.rows = kCin[l];
-        wt.C = kCin[l];
-        wt.py = py;
-        wt.px = px;
-        d.b = wt;
-        d.out = nxt;
-        d.ldc = kCin[l];
-        d.mask = w.act[l];
-        d.remap = 1;
-        d.rH = kHin[l];
-        d.rW = kWin[l];
-        d.rHc = Hc;
-        d.rWc = Wc;
-        d.rpy = py;
-        d.rpx = px;
-        r = fused<K_DGRADP, R_WTP, E_MASK>(d, Hc * Wc, w.part, st);
-        if (r) return r;
-      }
+    r = l == 1 ? dgrad2(cur, B, w.wbf + L.wbf_off[1], w.act[1], nxt, st)
+               : dgrad_tma(l, cur, B, w.wbf + L.wbf_off[l], w.act[l], nxt, sp, w.err, st);
+    if (r) return r;
     bf16* t = cur;
     cur = nxt;
     nxt = t;

@@ -389,3 +389,11 @@ def test_forward_does_not_depend_on_the_batch(torch_cuda):
     for b in (1, 12, 13, 15, 16, 19, 20, 33, 34, 38, 39, 76, 77, 95, 96, 101, 102, 152, 153, 190,
               191, 380, 381, 399):
         assert torch.equal(forward(b), ref[:b]), b
+
+
+@pytest.mark.parametrize("B", [1, 2, 16, 64])
+def test_data_gradients_of_ragged_image_tiles(torch_cuda, B):
+    """The data gradients of layers 5 and 6 put 6 and 21 images in a tile: a
+    part of one, a whole one and a remainder, and two remainders of the same
+    batch.  On exactly representable inputs every gradient is exact."""
+    test_net_is_bit_exact_on_exactly_representable_inputs(torch_cuda, B)
