@@ -5,10 +5,11 @@
 // depth mu_c.z (positive floats order like their bits), then by surfel id.
 // A tile's list is short (hundreds of entries), so instead of a global depth
 // sort the pairs are binned first and every tile sorts its own segment:
-//   1. scan: per surfel (id order) its tile count k_i -> emission offset
+//   1. count and scan: per surfel (id order) its tile count k_i -> emission offset
 //      (exclusive scan with decoupled look-back) and the total K; every
 //      covered tile's counter is incremented;
-//   2. tile scan: one block turns the tile counts into tile ranges;
+//   2. tile scan: the last block of that launch turns the tile counts into
+//      tile ranges (in a batch of many views, one block a view);
 //   3. scatter: every pair writes the 64-bit key (depth bits << 32 | id)
 //      into its tile's segment at an atomically claimed slot (the order
 //      inside a segment is arbitrary at this point);
@@ -130,15 +131,6 @@ __device__ __forceinline__ void count_body(const float4* __restrict__ proj,
     if (s_hist[t]) atomicAdd(tile_count + t, s_hist[t]);
 }
 
-__global__ void __launch_bounds__(kScanThreads) count_kernel(
-    const float4* __restrict__ proj, const int32_t* __restrict__ tiles, int n, int tiles_x,
-    int n_tiles, uint32_t* __restrict__ tile_count, const int32_t* __restrict__ gate) {
-  extern __shared__ uint32_t s_hist[];
-  __shared__ WalkScratch s_walk[kScanThreads / 32];
-  if (*gate) return;
-  count_body(proj, tiles, n, tiles_x, n_tiles, tile_count, blockIdx.x, gridDim.x, s_hist, s_walk);
-}
-
 // 1b. Exclusive scan of k_i over surfel ids with decoupled look-back (64-bit
 // chunk words: flag in bits 62-63; a warp examines 32 predecessors at a
 // time; the spin is bounded by spin_limit polls and past it records
@@ -231,31 +223,55 @@ __device__ __forceinline__ void emit_scan_body(const int32_t* __restrict__ tiles
   }
 }
 
-__global__ void __launch_bounds__(kScanThreads) emit_scan_kernel(
-    const int32_t* __restrict__ tiles, int n, uint32_t* __restrict__ surfel_off,
-    unsigned long long* __restrict__ chunk_status, uint32_t* __restrict__ ticket,
-    int32_t* __restrict__ gate, int spin_limit, int withheld) {
-  __shared__ ScanSmem sm;
-  __shared__ int s_chunk;
-  if (*gate) return;
-  if (threadIdx.x == 0) s_chunk = (int)atomicAdd(ticket, 1u);
+// 1 and 2 in one launch: `chunks` blocks scan the emission offsets while the
+// others count, and the last block to finish turns the counts into tile ranges
+// (2.: K and the capacity check too).  As three launches of a few us each,
+// mostly start, drain and latency, they took 15 us for 4,000 surfels and 22.6
+// us for 200,000; together 10.7 and 16.1.
+constexpr int kScanSmallTiles = 4096;
+__global__ void __launch_bounds__(kScanThreads) count_scan_kernel(
+    const float4* __restrict__ proj, const int32_t* __restrict__ tiles, int n, int tiles_x,
+    int n_tiles, uint32_t* __restrict__ tile_count, int chunks, uint32_t* __restrict__ surfel_off,
+    unsigned long long* __restrict__ chunk_status, uint32_t* __restrict__ ticket, int spin_limit,
+    int withheld, uint32_t* __restrict__ done, int32_t* __restrict__ ranges,
+    int32_t* __restrict__ n_isect, long long capacity, uint32_t* __restrict__ long_list,
+    uint32_t* __restrict__ n_long, int32_t* __restrict__ gate) {
+  extern __shared__ uint32_t s_hist[];
+  __shared__ union {
+    ScanSmem scan;
+    WalkScratch walk[kScanThreads / 32];
+    uint32_t w[33];
+  } sm;
+  __shared__ int s_chunk, s_gate;
+  __shared__ bool s_last;
+  // one read for the block: a scan that times out sets the gate meanwhile
+  if (threadIdx.x == 0) s_gate = *reinterpret_cast<const volatile int32_t*>(gate);
   __syncthreads();
-  emit_scan_body(tiles, n, surfel_off, chunk_status, s_chunk, gate, spin_limit, withheld, sm);
-}
-
-// 2. Tile ranges from the tile counts (one block), K and the capacity check.
-__global__ void __launch_bounds__(1024) tile_scan_kernel(const uint32_t* __restrict__ tile_count,
-                                                        int n_tiles, int32_t* __restrict__ ranges,
-                                                        int32_t* __restrict__ n_isect,
-                                                        long long capacity,
-                                                        uint32_t* __restrict__ long_list,
-                                                        uint32_t* __restrict__ n_long,
-                                                        int32_t* __restrict__ gate) {
-  __shared__ uint32_t s_w[32];
-  __shared__ uint32_t s_carry;
-  if (*gate) return;
-  tile_scan_block(tile_count, n_tiles, ranges, n_isect, capacity, long_list, n_long, kSegSmem, gate,
-                  s_w, &s_carry);
+  if (s_gate) return;
+  if ((int)blockIdx.x < chunks) {
+    if (threadIdx.x == 0) s_chunk = (int)atomicAdd(ticket, 1u);
+    __syncthreads();
+    emit_scan_body(tiles, n, surfel_off, chunk_status, s_chunk, gate, spin_limit, withheld, sm.scan);
+  } else {
+    count_body(proj, tiles, n, tiles_x, n_tiles, tile_count, (int)blockIdx.x - chunks,
+               (int)gridDim.x - chunks, s_hist, sm.walk);
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __threadfence();
+    s_gate = *reinterpret_cast<const volatile int32_t*>(gate);
+  }
+  __syncthreads();
+  if (!s_last || s_gate) return;
+  if (n_tiles <= kScanSmallTiles)
+    tile_scan_order_small<kScanSmallTiles / 256>(tile_count, n_tiles, ranges, n_isect, capacity,
+                                                 long_list, n_long, kSegSmem, gate, nullptr, nullptr,
+                                                 sm.w);
+  else
+    tile_scan_block(tile_count, n_tiles, ranges, n_isect, capacity, long_list, n_long, kSegSmem,
+                    gate, sm.w, sm.w + 32);
 }
 
 // 3. Scatter of the keys into the tile segments: depth bits << 32 | id, or,
@@ -529,7 +545,7 @@ struct SortWs {
   unsigned long long* seg_tmp;   // [cap] merge buffer of long segments
   uint32_t* long_list;           // [n_tiles] tiles with segments over kSegSmem
   uint32_t* n_long;              // [1] (zeroed per call)
-  uint32_t* proj_done;           // [1] blocks of a fused projection finished (zeroed per call)
+  uint32_t* proj_done;           // [1] blocks of the count, or of a fused projection, finished (zeroed)
   uint32_t* grid_bar;            // [1] grid barrier of a projection with fused scatter (zeroed)
   uint32_t* zero_begin;          // start of the zeroed region
   uint32_t* tile_count;          // [n_tiles]
@@ -665,21 +681,14 @@ int bin_sort_launch(const float* proj, const int32_t* tiles_per_surfel, int n,
     GS2D_LAUNCH_CHECK();
   }
   const bool scanned = (flags & kSortPreScanned) != 0;
-  if (n > 0 && !scanned) {
-    const int blocks = min((n + kScanThreads - 1) / kScanThreads, 152 * 4);
-    count_kernel<<<blocks, kScanThreads, hist_smem, st>>>(p4, tiles_per_surfel, n, tx, n_tiles,
-                                                          w.tile_count, gate);
-    GS2D_LAUNCH_CHECK();
-    if (need_emit) {
-      emit_scan_kernel<<<w.chunks_n, kScanThreads, 0, st>>>(
-          tiles_per_surfel, n, bins->surfel_off, w.estatus, w.ticket, gate,
-          g_lookback_spins > 0 ? g_lookback_spins : kSpinLimit, g_lookback_withheld);
-      GS2D_LAUNCH_CHECK();
-    }
-  }
   if (!scanned) {
-    tile_scan_kernel<<<1, 1024, 0, st>>>(w.tile_count, n_tiles, bins->tile_ranges, bins->n_isect,
-                                         cap, w.long_list, w.n_long, gate);
+    // (a grid of no surfels still writes the empty ranges)
+    const int chunks = n > 0 && need_emit ? w.chunks_n : 0;
+    const int blocks = max(1, min((n + kScanThreads - 1) / kScanThreads, 152 * 4));
+    count_scan_kernel<<<chunks + blocks, kScanThreads, hist_smem, st>>>(
+        p4, tiles_per_surfel, n, tx, n_tiles, w.tile_count, chunks, bins->surfel_off, w.estatus,
+        w.ticket, g_lookback_spins > 0 ? g_lookback_spins : kSpinLimit, g_lookback_withheld,
+        w.proj_done, bins->tile_ranges, bins->n_isect, cap, w.long_list, w.n_long, gate);
     GS2D_LAUNCH_CHECK();
   }
   if (n == 0) return GS2D_OK;
