@@ -27,19 +27,34 @@
 
 namespace gs2d {
 
-// 8 x 4 blocks per region (pixels per lane): a whole 256-pixel tile per warp
-// when the view has tiles enough to fill the GPU (one partial per (tile,
-// surfel)), half a tile for small views (twice the work units).
-constexpr int kBwdRegion = 8;
-constexpr int kBwdRegionSmall = 4;
+constexpr int kBwdRegion = 8;      // 8 x 4 blocks per region of a batch of views
 constexpr int kBwdWarps = 4;       // warps (independent work items) per block
 constexpr int kBwdWarpBlocks = 4;  // resident blocks per SM the registers are sized for
-// Regions per tile of a tile shape with R blocks per region, and the most
-// any shape (up to 1024 pixels) and region size can have.
+constexpr int kBwdMaxRegions = 8;  // regions per tile that the partials have room for
+// Regions per tile of a tile shape (up to 1024 pixels) with R blocks per region.
 __host__ __device__ inline int bwd_regions(const gs2d_config& c, int R = kBwdRegion) {
   return c.tile_w * c.tile_h / (32 * R);
 }
-constexpr int kBwdMaxRegions = 1024 / (32 * kBwdRegionSmall);
+// Blocks per region of a single view: the fewest of 1, 2, 4 whose regions fit
+// one wave of resident warps (152 SMs x 16), else 8.  Few regions leave SMs
+// idle and make each warp's walk long; past one wave, more regions only repeat
+// the staging and the warp sums.  Regions of one block need a little more
+// room: their sums outweigh their pixels.  Whole backward pass, us, regions of
+// 1 / 2 / 4 / 8 blocks, 300,000-surfel room (and 4,000-surfel slab); in
+// brackets what the line takes:
+//   160x120    80 tiles  [100] 137  225  477   ([42]  47   65  114)
+//   280x200   234 tiles    86  [96] 148  277   ( 52  [45]  51   80)
+//   480x360   690 tiles   119  107 [111] 190   ( 85   60  [55]  72)
+//   640x480  1200 tiles   169  127 [119] 170   (123   82  [65]  75)
+//   800x600  1900 tiles   232  168  149 [165]  (169  109   84  [78])
+// (before: 4 blocks below 304 tiles, else 8).
+inline int bwd_region_for(const gs2d_config& c, int n_tiles) {
+  constexpr long long kWave = 152LL * kBwdWarpBlocks * kBwdWarps;
+  const long long blocks = (long long)n_tiles * bwd_regions(c, 1);
+  for (int R = 1; R < kBwdRegion; R *= 2)
+    if (bwd_regions(c, R) <= kBwdMaxRegions && blocks <= R * (R == 1 ? kWave * 3 / 4 : kWave)) return R;
+  return kBwdRegion;
+}
 
 // Per-warp shared memory: the staged records of 32 list entries and the
 // region's per-pixel upstream gradients, [k][0] = (dC, dD), [k][1] = (dN,

@@ -38,6 +38,8 @@
 // chains to world space, scales and the quaternion, and forms the pose term.
 // Tracking mode: pixels accumulate the 6-vector pose gradient directly; one
 // partial per tile, reduced in a fixed order.
+#include <type_traits>
+
 #include "bwd_warp.cuh"
 #include "gs2d_common.cuh"
 #include "gs2d_internal.h"
@@ -1024,19 +1026,24 @@ int render_bwd_launch(const float* proj, const gs2d_bins* bins, const int32_t* t
   const BwdWs w = carve_bwd_ws(workspace, s->n, bins->capacity, n_tiles, full, kBwdMaxRegions);
   const float4* p4 = reinterpret_cast<const float4*>(proj);
   if (full) {
-    // a view of few tiles (fewer than two per SM) replays half tiles
-    const bool small = n_tiles < 2 * 152;
-    const int Q = bwd_regions(*cfg, small ? kBwdRegionSmall : kBwdRegion);
+    // regions as small as fill the GPU: see bwd_region_for
+    const int R = bwd_region_for(*cfg, n_tiles);
+    const int Q = bwd_regions(*cfg, R);
     const int units = n_tiles * Q;
     const int blocks = (units + kBwdWarps - 1) / kBwdWarps;
-    if (small)
-      render_bwd_warp_kernel<kBwdRegionSmall><<<blocks, kBwdWarps * 32, 0, st>>>(
+    auto launch = [&](auto r) {
+      render_bwd_warp_kernel<decltype(r)::value><<<blocks, kBwdWarps * 32, 0, st>>>(
           p4, bins->vals, bins->isect_emit, bins->tile_ranges, *cam, *cfg, tx, Q, units, t_final,
           n_last, d_rgb, d_depth, d_normal, d_opacity, w.partials, gate);
+    };
+    if (R == 1)
+      launch(std::integral_constant<int, 1>());
+    else if (R == 2)
+      launch(std::integral_constant<int, 2>());
+    else if (R == 4)
+      launch(std::integral_constant<int, 4>());
     else
-      render_bwd_warp_kernel<kBwdRegion><<<blocks, kBwdWarps * 32, 0, st>>>(
-          p4, bins->vals, bins->isect_emit, bins->tile_ranges, *cam, *cfg, tx, Q, units, t_final,
-          n_last, d_rgb, d_depth, d_normal, d_opacity, w.partials, gate);
+      launch(std::integral_constant<int, kBwdRegion>());
     GS2D_LAUNCH_CHECK();
     if (s->n > 0) {
       const int nb = (s->n + 255) / 256;

@@ -339,3 +339,39 @@ def test_forward_only_binning_matches(torch_cuda):
     assert int(r.status.item()) == 0 and int(r.n_isect.item()) == K
     assert torch.equal(r.vals[:K], vals) and torch.equal(r.ranges, ranges)
     assert torch.equal(r.rgb, rgb)
+
+
+@pytest.mark.parametrize("tile,px,grid", [((16, 16), 1, (3, 2)), ((16, 16), 1, (19, 12)), ((16, 16), 1, (23, 10)),
+                                          ((16, 16), 1, (32, 19)), ((16, 16), 1, (29, 21)),
+                                          ((16, 16), 1, (38, 32)), ((16, 16), 1, (42, 29)),
+                                          ((32, 16), 2, (19, 16)), ((32, 16), 2, (61, 5)),
+                                          ((32, 24), 3, (21, 19)), ((32, 24), 3, (37, 11)),
+                                          ((32, 32), 4, (19, 16)), ((32, 32), 4, (61, 5))])
+def test_backward_regions_of_every_size_sum_alike(torch_cuda, tile, px, grid):
+    """A single view's backward cuts its tiles into regions of 1, 2, 4 or 8
+    blocks by the size of the tile grid (both sides of each line, every tile
+    shape); a batch of one view always takes 8.  The same pair terms are
+    summed in another order: 2e-6 of the largest, 16 FP32 roundings."""
+    torch = torch_cuda
+    from paper_2506_00970_gb300 import gs2d
+    w, h = grid[0] * tile[0] - 3, grid[1] * tile[1] - 2
+    cam = scenes.Camera(0.9 * w, 0.9 * w, w / 2, h / 2, w, h)
+    s = scenes.slab_scene(7, 3000)
+    ds, pose = gs2d.DeviceSurfels(s), scenes.identity_pose()
+    r = gs2d.Rasterizer(cam, s.n, capacity=2_000_000, tile=tile, px=px)
+    assert r.n_tiles == grid[0] * grid[1]
+    r.forward(ds, gs2d.pose_tensor(pose))
+    up = scenes.random_upstream(3, h, w)
+    d_rgb, d_depth = (torch.tensor(u, dtype=torch.float32, device="cuda") for u in up[:2])
+    g = r.backward(ds, gs2d.pose_tensor(pose), d_rgb, d_depth)
+    br = gs2d.BatchRasterizer([cam], s.n, tiles=[tile], px=px, capacities=[2_000_000])
+    br.set_poses([pose])
+    br.forward(ds)
+    br.keep[0]["d_rgb"].copy_(d_rgb)
+    br.keep[0]["d_depth"].copy_(d_depth)
+    gb = br.backward(ds)
+    torch.cuda.synchronize()
+    for k in ("mu", "quat", "scale", "opacity", "rgb"):
+        ref = gb[k].reshape(g[k].shape)
+        assert float(ref.abs().max()) > 0
+        assert float((g[k] - ref).abs().max()) <= 2e-6 * float(ref.abs().max()), k
