@@ -365,8 +365,9 @@ size_t gs2d_mapping_loss_batch_workspace(const gs2d_loss_view* views, int n_view
   for (int v = 0; v < n_views; ++v) {
     const gs2d_camera& c = views[v].cam;
     if (c.width <= 0 || c.height <= 0) return 0;
-    // sized for the smaller strips
-    items += (size_t)strips_along(c.width, kStripW) * strips_along(c.height, kStripRowsSmall);
+    // eight partials per 32 x 8 pixels: room for the smaller strips (28 x 2) of
+    // any size, ceil(w / 28) <= 2 ceil(w / 32) and ceil(h / 2) <= 4 ceil(h / 8)
+    items += (size_t)strips_along(c.width, 32) * strips_along(c.height, 8) * 8;
   }
   return align_up(items * sizeof(float), 256);
 }
