@@ -46,7 +46,7 @@ TIMED_EVERY = 10          # fused-kernel launches bracketed by events: every 10t
 # DRAM bytes per launch of the roofline kernel (dram__bytes_read.sum +
 # dram__bytes_write.sum of one ncu capture of the fused tracking kernel on
 # this workload); None while the kernel has changed since the capture.
-TRAFFIC_BYTES = {"track_tile": 6610432}
+TRAFFIC_BYTES = {"track_tile": None}
 # batched workloads reported beside the tracking line
 MAP_SURFELS, MAP_VIEWS = 1_000_000, 8
 UNEVEN_SURFELS, UNEVEN_VIEWS = 2_000_000, 32
@@ -454,7 +454,7 @@ def roofline(r, ds, frames, cam, cfg, stream, ms_iter, fused_ms):
     work_fused = np.mean(work_f) + np.mean(work_b) + FLOPS_LOSS_PIXEL * P
     tfu = fused_ms / 1e3
     afu = work_fused / tfu / 1e12
-    fused = {"kernel": "track_tile_kernel (render + tracking loss + pose backward)", "bound": "alu",
+    fused = {"kernel": "track_quad_kernel (render + tracking loss + pose backward)", "bound": "alu",
              "achieved": afu, "peak": peak, "unit": "TFLOP/s", "frac": afu / peak,
              "traffic": TRAFFIC_BYTES["track_tile"],
              "traffic_note": "ncu capture of one launch on the first of the timed frames "

@@ -158,8 +158,8 @@ int gs2d_project(const gs2d_surfels* s, const gs2d_camera* cam, const float* pos
  * intersections are ordered by (tile, mu_c.z bits, surfel id) -- the order
  * of a stable sort by tile of the depth-ordered emission -- by binning the
  * pairs into per-tile segments and sorting every segment by (depth bits, id)
- * in shared memory (hand-written bitonic networks; long segments in chunks
- * merged in global memory), so the result is unique and deterministic.
+ * in shared memory (runs sorted in registers, then merged; long segments in
+ * chunks merged in global memory), so the result is unique and deterministic.
  * This replaces the global LSD radix sort on (tile, depth) keys of the first
  * design (four 8-bit passes over the depth keys, then one or two over the
  * tile keys): the per-tile sort gives the identical order in fewer passes

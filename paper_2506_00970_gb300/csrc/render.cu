@@ -30,12 +30,11 @@
 // normal image -- the Jacobians [I, -mu_c^x] and [0, -R_c,:,i^x] of Sec. III-B
 // contracted with these rank-one gradients.
 //
-// Full mode: per batch each warp sums its 32 pixels' 16 per-pair values with
-// a butterfly reduce-scatter (16 shuffles per surfel instead of 80), the 8
-// warps are summed through shared memory, and one 64-byte partial per
-// (tile, surfel) pair is written at the pair's emission index.  A second
-// kernel adds each surfel's partials in emission order (deterministic),
-// chains to world space, scales and the quaternion, and forms the pose term.
+// Full mode: one warp replays one region of a tile (bwd_warp.cuh) and writes a
+// 64-byte partial per (tile, region, surfel) at the pair's emission index.  A
+// second kernel adds each surfel's partials in emission order
+// (deterministic), chains to world space, scales and the quaternion, and
+// forms the pose term.
 // Tracking mode: pixels accumulate the 6-vector pose gradient directly; one
 // partial per tile, reduced in a fixed order.
 #include <type_traits>
