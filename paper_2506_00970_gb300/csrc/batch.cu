@@ -244,7 +244,7 @@ BatchWs carve_batch_ws(void* base, const gs2d_view* views, int n_views, int n) {
     const size_t cap = views[v].bins.capacity > 0 ? views[v].bins.capacity : 1;
     w.partials[v] = c.take<float>(cap * bwd_regions(views[v].cfg) * 16);
     const int m = views[v].active ? views[v].n_active : n;
-    w.pose_part[v] = c.take<float>((size_t)max(1, (m + 255) / 256) * 6);
+    w.pose_part[v] = c.take<float>((size_t)max(1, grad_blocks(m)) * 6);
   }
   w.bytes = align_up(c.off, 256);
   return w;
@@ -463,7 +463,7 @@ int gs2d_render_bwd_batch(const gs2d_view* views, int n_views, const gs2d_surfel
       t.v[t.n++] = GradView{x.pose, x.tiles_per_surfel, x.bins.surfel_off, x.proj, w.partials[v],
                             w.pose_part[v], x.bins.status};
       if (x.d_pose6)
-        pt.v[pt.n++] = PoseReduceView{w.pose_part[v], (m + 255) / 256, x.d_pose6, x.bins.status};
+        pt.v[pt.n++] = PoseReduceView{w.pose_part[v], grad_blocks(m), x.d_pose6, x.bins.status};
       ++v;
     } while (!active && v < n_views && !views[v].active);
     r = surfel_grad_launch(s, active, m, first == 0 && !active ? kGradSum : kGradAdd, Q, t, d_mu,

@@ -134,7 +134,7 @@ int tracking_loss_launch(const float* rgb, const float* depth, const float* norm
 // Per-surfel reduction of the (tile, region, surfel) partials, Q region slots
 // per tile, of one or several views of the same m records (record i is surfel
 // active[i] or i), and the block partials of each view's pose gradient
-// ([ceil(m / 256)][6]).  mode: kGradWrite writes the sum of the views'
+// ([grad_blocks(m)][6]).  mode: kGradWrite writes the sum of the views'
 // gradients, or nothing if the gate keeps the (one) view out; kGradSum writes
 // the sum over the views that their gates let in; kGradAdd adds that sum.
 enum GradMode { kGradWrite = 0, kGradAdd = 1, kGradSum = 2 };
@@ -151,6 +151,14 @@ struct GradTable {
   int n;
   GradView v[GS2D_MAX_VIEWS];
 };
+// Surfels per warp: eight, whose partials a warp sums in one pass, while all
+// their warps fit one resident wave (152 SMs x 24); else 32, in up to four
+// passes.  4,096 surfels with eight regions a tile: 19.8 -> 11.6 us.
+inline int grad_surfels_per_warp(int m) { return m <= 152 * 24 * 8 ? 8 : 32; }
+inline int grad_blocks(int m) {
+  const int per = 8 * grad_surfels_per_warp(m);
+  return (m + per - 1) / per;
+}
 int surfel_grad_launch(const gs2d_surfels* s, const int32_t* active, int m, int mode, int Q,
                        const GradTable& t, float* d_mu, float* d_quat, float* d_scale,
                        float* d_opac, float* d_rgb, cudaStream_t st);

@@ -660,7 +660,9 @@ __global__ void __launch_bounds__(kTileThreads, 4) track_quad_kernel(
 // chain rule.  1M surfels x 8 views of 1200 x 680: 684 -> 311 us (all
 // views in one launch); 32 views of subsets, each in a launch of its own that
 // mostly moves the scattered outputs and parameters, 1389 -> 1370 us.
+// SPW: surfels per warp (grad_surfels_per_warp).
 constexpr int kGradThreads = 256, kGradWarps = kGradThreads / 32;
+template <int SPW>
 __global__ void __launch_bounds__(kGradThreads, 3) surfel_grad_kernel(
     const GradTable t, const float* __restrict__ mu, const float* __restrict__ quat,
     const float* __restrict__ scale, int m, const int32_t* __restrict__ active, int n_all, int mode,
@@ -675,8 +677,8 @@ __global__ void __launch_bounds__(kGradThreads, 3) surfel_grad_kernel(
   for (int e = threadIdx.x; e < t.n * 12; e += kGradThreads) s_in[e / 12][e % 12] = t.v[e / 12].pose[e % 12];
   for (int v = threadIdx.x; v < t.n; v += kGradThreads) s_dead[v] = t.v[v].gate && *t.v[v].gate;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i = blockIdx.x * kGradThreads + threadIdx.x;
-  const bool in = i < m;
+  const int i = ((int)blockIdx.x * kGradWarps + warp) * SPW + lane;
+  const bool in = lane < SPW && i < m;
   const int sid = !in ? 0 : (active ? min(max(active[i], 0), n_all - 1) : i);
   float4 q4 = make_float4(1.f, 0.f, 0.f, 0.f);
   F3 mw = f3(0.f, 0.f, 0.f);
@@ -869,7 +871,7 @@ BwdWs carve_bwd_ws(void* base, int n, size_t cap, int n_tiles, bool full, int Q)
   Carver c(base);
   BwdWs w;
   w.partials = c.take<float>(full ? (cap > 0 ? cap : 1) * Q * kRedVals : 1);
-  const int nb = max(n_tiles, (n + 255) / 256);
+  const int nb = max(n_tiles, grad_blocks(n));
   w.pose_part = c.take<float>((size_t)max(nb, 1) * 6);
   w.bytes = align_up(c.off, 256);
   return w;
@@ -971,8 +973,9 @@ int surfel_grad_launch(const gs2d_surfels* s, const int32_t* active, int m, int 
                        const GradTable& t, float* d_mu, float* d_quat, float* d_scale,
                        float* d_opac, float* d_rgb, cudaStream_t st) {
   if (m <= 0) return GS2D_OK;
-  surfel_grad_kernel<<<(m + kGradThreads - 1) / kGradThreads, kGradThreads, 0, st>>>(
-      t, s->mu, s->quat, s->scale, m, active, s->n, mode, Q, d_mu, d_quat, d_scale, d_opac, d_rgb);
+  auto kern = grad_surfels_per_warp(m) == 8 ? surfel_grad_kernel<8> : surfel_grad_kernel<32>;
+  kern<<<grad_blocks(m), kGradThreads, 0, st>>>(t, s->mu, s->quat, s->scale, m, active, s->n, mode, Q,
+                                                d_mu, d_quat, d_scale, d_opac, d_rgb);
   GS2D_LAUNCH_CHECK();
   return GS2D_OK;
 }
@@ -1045,7 +1048,6 @@ int render_bwd_launch(const float* proj, const gs2d_bins* bins, const int32_t* t
       launch(std::integral_constant<int, kBwdRegion>());
     GS2D_LAUNCH_CHECK();
     if (s->n > 0) {
-      const int nb = (s->n + 255) / 256;
       GradTable t;
       t.n = 1;
       t.v[0] = GradView{pose, tiles_per_surfel, bins->surfel_off, proj, w.partials, w.pose_part, gate};
@@ -1053,7 +1055,7 @@ int render_bwd_launch(const float* proj, const gs2d_bins* bins, const int32_t* t
                                         d_opac, d_rgb_out, st);
       if (gr) return gr;
       if (d_pose6) {
-        const int pr = pose_reduce_one(w.pose_part, nb, d_pose6, gate, st);
+        const int pr = pose_reduce_one(w.pose_part, grad_blocks(s->n), d_pose6, gate, st);
         if (pr) return pr;
       }
     } else if (d_pose6) {

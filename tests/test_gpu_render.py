@@ -375,3 +375,36 @@ def test_backward_regions_of_every_size_sum_alike(torch_cuda, tile, px, grid):
         ref = gb[k].reshape(g[k].shape)
         assert float(ref.abs().max()) > 0
         assert float((g[k] - ref).abs().max()) <= 2e-6 * float(ref.abs().max()), k
+
+
+@pytest.mark.parametrize("n", [7, 8, 63, 65, 29184, 29185])
+def test_surfel_gradients_of_warps_of_8_and_of_32(torch_cuda, n):
+    """Both sides of the line between warps of 8 and of 32 surfels, and
+    remainders of a warp and a block: a map padded with surfels behind the
+    camera past the line has the same gradients, its sums over the same
+    partials in the same order; the pose sum adds block partials in another
+    grouping: 1e-5 of its largest component (30,000 FP32 terms, pairwise)."""
+    torch = torch_cuda
+    from paper_2506_00970_gb300 import gs2d
+    cam = scenes.Camera(150.0, 150.0, 80.0, 60.0, 160, 120)
+    s = scenes.slab_scene(3, n)
+    pad = scenes.slab_scene(4, 40000)
+    pad.mu[:, 2] = -5.0
+    big = scenes.Surfels(*(np.concatenate([getattr(s, k), getattr(pad, k)])
+                           for k in ("mu", "quat", "scale", "opacity", "rgb")))
+    up = scenes.random_upstream(3, 120, 160)
+    d_rgb, d_depth = (torch.tensor(u, dtype=torch.float32, device="cuda") for u in up[:2])
+    pose = gs2d.pose_tensor(scenes.identity_pose())
+    out = []
+    for m in (s, big):
+        ds = gs2d.DeviceSurfels(m)
+        r = gs2d.Rasterizer(cam, m.n, capacity=40 * n + 1000)
+        r.forward(ds, pose)
+        out.append(r.backward(ds, pose, d_rgb, d_depth))
+    torch.cuda.synchronize()
+    a, b = out
+    for k in ("mu", "quat", "scale", "opacity", "rgb"):
+        assert float(a[k].abs().max()) > 0
+        assert torch.equal(a[k], b[k][:n]), k
+        assert not b[k][n:].any(), k
+    assert float((a["pose6"] - b["pose6"]).abs().max()) <= 1e-5 * float(b["pose6"].abs().max())
