@@ -4,8 +4,8 @@
 // bound (160x120 has 80 tiles of 16x16; one thread per pixel leaves 1 warp
 // per scheduler).
 //
-// A 256-pixel tile is cut into its four 8 x 8 quadrants, one block each.  The
-// block keeps only the entries whose footprint touches its quadrant (about
+// A 256-pixel tile is cut into its four 8 x 8 quadrants, one block each (a tile
+// of 64 x 4 pixels into four of 16 x 4).  The block keeps only the entries whose footprint touches its quadrant (about
 // half of a small image's list), and each warp owns 4 x 2 pixels with four
 // lanes per pixel (lane = 4 * pixel + e): the lanes evaluate four successive
 // hits of their pixel at once, then all four replay the pixel's transmittance
@@ -29,20 +29,26 @@ namespace gs2d {
 constexpr int kQuads = 4;        // 8 x 8 quadrants of a 256-pixel tile
 constexpr int kQuadBatch = 256;  // entries staged at a time
 
+// Tiles 4 pixels high have quadrants of 16 x 4 pixels.
+__device__ __forceinline__ bool quad_flat(const gs2d_config& cfg) { return cfg.tile_h < 8; }
+
 // The block's quadrant and the lane's pixel: quadrant q at tile offset
 // (8 (q % (tile_w / 8)), 8 (q / (tile_w / 8))), warp w the 4 x 2 pixels at
-// (4 (w & 1), 2 (w >> 1)) of it.
+// (4 (w & 1), 2 (w >> 1)) of it; in a flat tile at (16 q, 0) and
+// (4 (w & 3), 2 (w >> 2)).
 struct QuadPix {
   int x0, y0;      // the quadrant's first pixel
   int px, py;      // the lane's pixel
   float lx, ly;    // its centre relative to the tile's first pixel centre
-  int slot;        // its index 8 (py - y0) + (px - x0) in the quadrant
+  int slot;        // its index in the quadrant, whose two 8 x 4 blocks follow each other
+  bool flat;
 };
-__device__ __forceinline__ QuadPix quad_pixel(int q, int tile_x0, int tile_y0, int tile_w) {
+__device__ __forceinline__ QuadPix quad_pixel(int q, int tile_x0, int tile_y0, int tile_w,
+                                              bool flat) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, p = lane >> 2;
   const int per_row = tile_w >> 3;
-  const int ox = (q % per_row) * 8, oy = (q / per_row) * 8;
-  const int cx = (w & 1) * 4 + (p & 3), cy = (w >> 1) * 2 + (p >> 2);
+  const int ox = flat ? q * 16 : (q % per_row) * 8, oy = flat ? 0 : (q / per_row) * 8;
+  const int cx = (flat ? w & 3 : w & 1) * 4 + (p & 3), cy = (flat ? w >> 2 : w >> 1) * 2 + (p >> 2);
   QuadPix t;
   t.x0 = tile_x0 + ox;
   t.y0 = tile_y0 + oy;
@@ -50,17 +56,31 @@ __device__ __forceinline__ QuadPix quad_pixel(int q, int tile_x0, int tile_y0, i
   t.py = t.y0 + cy;
   t.lx = (float)(ox + cx);
   t.ly = (float)(oy + cy);
-  t.slot = 8 * cy + cx;
+  t.slot = flat ? 32 * (cx >> 3) + 8 * cy + (cx & 7) : 8 * cy + cx;
+  t.flat = flat;
   return t;
+}
+
+// Which of the tile's 8 x 4 pixel blocks is block `half` of quadrant q.
+__device__ __forceinline__ int quad_block(int q, int half, int tile_w, bool flat) {
+  if (flat) return 2 * q + half;
+  const int per_row = tile_w >> 3;
+  return (2 * (q / per_row) + half) * per_row + q % per_row;
 }
 
 // Mask of the quadrant's eight warps whose 4 x 2 pixels a footprint (packed
 // pixel ranges) touches; 0 when it misses the quadrant.
-__device__ __forceinline__ uint32_t quad_mask(float bi, float bj, int x0, int y0) {
+__device__ __forceinline__ uint32_t quad_mask(float bi, float bj, const QuadPix& tp) {
   const uint32_t I = __float_as_uint(bi), J = __float_as_uint(bj);
-  const int i0 = max((int)(I & 0xFFFF) - x0, 0), i1 = min((int)(I >> 16) - x0, 7);
-  const int j0 = max((int)(J & 0xFFFF) - y0, 0), j1 = min((int)(J >> 16) - y0, 7);
+  const int i0 = max((int)(I & 0xFFFF) - tp.x0, 0);
+  const int i1 = min((int)(I >> 16) - tp.x0, tp.flat ? 15 : 7);
+  const int j0 = max((int)(J & 0xFFFF) - tp.y0, 0);
+  const int j1 = min((int)(J >> 16) - tp.y0, tp.flat ? 3 : 7);
   if (i0 > i1 || j0 > j1) return 0u;
+  if (tp.flat) {
+    const uint32_t cols = (2u << (i1 >> 2)) - (1u << (i0 >> 2));
+    return (j0 < 2 ? cols : 0u) | (j1 >= 2 ? cols << 4 : 0u);
+  }
   const uint32_t cols = (i0 < 4 ? 1u : 0u) | (i1 >= 4 ? 2u : 0u);
   uint32_t m = 0u;
 #pragma unroll

@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) render_fwd_quad_kernel(
   if (gate && *gate) return;
   const int tile = blockIdx.x / kQuads, q = blockIdx.x % kQuads;
   const int tile_x0 = (tile % tiles_x) * cfg.tile_w, tile_y0 = (tile / tiles_x) * cfg.tile_h;
-  const QuadPix tp = quad_pixel(q, tile_x0, tile_y0, cfg.tile_w);
+  const QuadPix tp = quad_pixel(q, tile_x0, tile_y0, cfg.tile_w, quad_flat(cfg));
   const bool inside = tp.px < cam.width && tp.py < cam.height;
   const float xt = (float)tile_x0 + 0.5f - cam.cx;
   const float yt = (float)tile_y0 + 0.5f - cam.cy;
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) render_fwd_quad_kernel(
     uint32_t m = 0u;
     if (idx < end) {
       const float4 r7 = proj[(size_t)id * (kProjFloats / 4) + 7];
-      m = quad_mask(r7.z, r7.w, tp.x0, tp.y0);
+      m = quad_mask(r7.z, r7.w, tp);
     }
     const uint32_t bal = __ballot_sync(0xffffffffu, m != 0u);
     if (lane == 0) s_cnt[turn][warp] = __popc(bal);
@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) track_quad_kernel(
   } else {
     QuadTrackSmem& s = sh.q;
     const int tile_x0 = (tile % tiles_x) * cfg.tile_w, tile_y0 = (tile / tiles_x) * cfg.tile_h;
-    const QuadPix tp = quad_pixel(quad, tile_x0, tile_y0, cfg.tile_w);
+    const QuadPix tp = quad_pixel(quad, tile_x0, tile_y0, cfg.tile_w, quad_flat(cfg));
     const bool inside = tp.px < cam.width && tp.py < cam.height;
     const float xt = (float)tile_x0 + 0.5f - cam.cx;
     const float yt = (float)tile_y0 + 0.5f - cam.cy;
@@ -537,7 +537,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) track_quad_kernel(
         key = ts.seg_keys[start + i];
         const uint32_t id = min((uint32_t)(key & 0xFFFFFFFFull), (uint32_t)(ts.n - 1));
         const float4 r7 = proj[(size_t)id * (kProjFloats / 4) + 7];
-        hit = quad_mask(r7.z, r7.w, tp.x0, tp.y0) != 0u;
+        hit = quad_mask(r7.z, r7.w, tp) != 0u;
       }
       const uint32_t b = __ballot_sync(0xffffffffu, hit);
       int o = 0;
@@ -557,7 +557,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) track_quad_kernel(
       if ((int)threadIdx.x < cnt) {
         stage_record_to<kBwdVec4>(proj, s.ids[b + threadIdx.x], xt, yt, s.st.rec[threadIdx.x]);
         const float4 r6 = s.st.rec[threadIdx.x][6];
-        s.st.mask[threadIdx.x] = (uint8_t)quad_mask(r6.z, r6.w, tp.x0, tp.y0);
+        s.st.mask[threadIdx.x] = (uint8_t)quad_mask(r6.z, r6.w, tp);
       }
       __syncthreads();
       return quad_hits(s.st, cnt);
@@ -618,10 +618,8 @@ __global__ void __launch_bounds__(kTileThreads, 4) track_quad_kernel(
       float x = s.out[c][32 * half + lane];
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-      // block (8 x 4) of the tile: row 2 (quadrant row) + half
-      const int per_row = cfg.tile_w >> 3;
-      const size_t part = (size_t)rank * kTileParts +
-                          (2 * (quad / per_row) + half) * per_row + quad % per_row;
+      const size_t part =
+          (size_t)rank * kTileParts + quad_block(quad, half, cfg.tile_w, tp.flat);
       if (lane == 0) ts.quad_part[part * 7 + c] = x;
     }
     __threadfence();

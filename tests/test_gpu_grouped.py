@@ -134,3 +134,25 @@ def test_grouped_forms_agree_over_list_lengths_and_shapes(torch_cuda, w, h, f, t
     for other in res[1:]:
         for k in res[0]:
             assert torch.equal(res[0][k], other[k]), k
+
+
+@pytest.mark.parametrize("w,h,f", [
+    (160, 120, 150.0),     # every tile may split
+    (101, 77, 95.0),       # ragged image, the last row of tiles one pixel high
+    (333, 251, 275.0),     # more tiles than may split
+])
+def test_tiles_four_pixels_high_have_quadrants_of_their_own(torch_cuda, w, h, f):
+    """A 64x4 tile has no 8 x 8 quadrants: its quadrants are 16 x 4.  The forms
+    agree bit for bit, and the images equal the 16x16 tiles' but for the point
+    at which intersections are re-based."""
+    from gpu_helpers import assert_images_close
+    from paper_2506_00970_gb300 import gs2d
+    test_grouped_forms_agree_over_list_lengths_and_shapes(torch_cuda, w, h, f, (64, 4))
+    s, pose = scenes.room_scene(3, 30_000), gs2d.pose_tensor(scenes.room_pose(11))
+    ds, cam, out = gs2d.DeviceSurfels(s), scenes.Camera(f, f, w / 2, h / 2, w, h), []
+    for tile in ((16, 16), (64, 4)):
+        img = gs2d.Rasterizer(cam, s.n, tile=tile).forward(ds, pose)
+        out.append({k: v.cpu().numpy() for k, v in img.items()})
+    assert out[0]["opacity"].max() > 0.9
+    assert_images_close(out[1], {k: out[0][k].astype(np.float64)
+                                 for k in ("rgb", "depth", "normal", "opacity")})
