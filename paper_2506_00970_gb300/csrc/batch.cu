@@ -63,13 +63,13 @@ __global__ void __launch_bounds__(kOrderThreads) order_items_kernel(ViewTable ta
                                                                   int32_t* __restrict__ order) {
   __shared__ uint32_t hist[kOrderBuckets];
   __shared__ int s_first[GS2D_MAX_VIEWS + 1];
-  __shared__ const int2* s_ranges[GS2D_MAX_VIEWS];
+  __shared__ const int32_t* s_ranges[GS2D_MAX_VIEWS];
   __shared__ bool s_dead[GS2D_MAX_VIEWS];
   for (int b = threadIdx.x; b < kOrderBuckets; b += blockDim.x) hist[b] = 0u;
   for (int v = threadIdx.x; v <= tab.n_views; v += blockDim.x) {
     s_first[v] = v < tab.n_views ? tab.v[v].item0 : tab.n_items;
     if (v < tab.n_views) {
-      s_ranges[v] = reinterpret_cast<const int2*>(tab.v[v].ranges);
+      s_ranges[v] = tab.v[v].ranges;
       s_dead[v] = tab.v[v].status && *tab.v[v].status;
     }
   }
@@ -84,7 +84,9 @@ __global__ void __launch_bounds__(kOrderThreads) order_items_kernel(ViewTable ta
       bk[k] = i < tab.n_items ? 0 : -1;
       if (i < tab.n_items) {
         while (i >= s_first[v + 1]) ++v;
-        if (!s_dead[v]) r[k] = s_ranges[v][i - s_first[v]];
+        // (word by word: the caller's ranges need only the alignment of an int)
+        const int32_t* p = s_ranges[v] + 2 * (i - s_first[v]);
+        if (!s_dead[v]) r[k] = make_int2(p[0], p[1]);
       }
     }
 #pragma unroll

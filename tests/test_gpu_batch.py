@@ -363,3 +363,31 @@ def test_batch_backward_in_any_order_of_views(torch_cuda, order, overflow):
         assert np.nanmax(np.abs(a - total[k])) <= lim, k
         rest = np.delete(a, 20, axis=0)
         assert np.all(rest[:39] == 0), k
+
+
+def test_batch_reads_tile_ranges_at_any_word(torch_cuda):
+    """tile_ranges is an array of ints: ranges that start at an odd word give
+    the aligned ones' images and gradients."""
+    torch = torch_cuda
+    from paper_2506_00970_gb300 import gs2d
+    s, cams, poses, actives, tiles = _setup()
+    ds, out = gs2d.DeviceSurfels(s), []
+    for shift in (0, 1):
+        br = gs2d.BatchRasterizer(cams, s.n, actives=actives, tiles=tiles,
+                                  capacities=[200000] * len(cams))
+        for b in br.keep:
+            b["ranges"] = torch.empty(2 * b["n_tiles"] + shift, dtype=torch.int32, device="cuda")[shift:]
+            assert b["ranges"].data_ptr() % 8 == 4 * shift
+        br._rebuild()
+        br.set_poses(poses)
+        br.forward(ds)
+        for v, b in enumerate(br.keep):
+            up = scenes.random_upstream(30 + v, cams[v].height, cams[v].width)
+            b["d_rgb"].copy_(torch.tensor(up[0], dtype=torch.float32))
+            b["d_depth"].copy_(torch.tensor(up[1], dtype=torch.float32))
+        g = br.backward(ds)
+        out.append([b[k].clone() for b in br.keep for k in ("rgb", "depth", "n_last", "d_pose6")]
+                   + [g[k].clone() for k in sorted(g)])
+    assert float(out[0][-1].abs().max()) > 0
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
