@@ -57,11 +57,12 @@ __device__ inline void bitonic_sort(unsigned long long* a, int len) {
   }
 }
 
-// Ascending sort of n distinct keys of shared memory by the whole block, a
-// and b two buffers of n keys; returns the one that holds the result (visible
-// to the block).  Warps sort runs of 32 keys in registers (a bitonic network
+// Ascending sort of n keys of shared memory by the whole block, a and b two
+// buffers of n keys; returns the one that holds the result (visible to the
+// block).  (Keys are distinct but for rectangles that reach past the tile
+// grid, whose pairs fall into the tiles that are there.)  Warps sort runs of 32 keys in registers (a bitonic network
 // by shuffles); then runs are merged two by two, every key finding its place
-// as its index in its own run plus the number of smaller keys in the other
+// as its index in its own run plus the number of keys before it in the other
 // (a binary search), from one buffer into the other.  log2(n / 32) barriers
 // instead of the log2(n)^2 / 2 of a bitonic network in shared memory, which
 // spent its time on them (80 tiles of ~300 to 1300 keys at 160x120, 27 -> 19
@@ -90,10 +91,11 @@ static __device__ __noinline__ unsigned long long* merge_sort(unsigned long long
       const int other = (i & ~(w - 1)) ^ w;          // the sibling run
       const int len = min(w, n - other);
       const unsigned long long* q = a + other - 1;   // q[m]: its m-th key
-      int m = 0;                                     // keys below k
+      const unsigned long long lim = k + ((i & w) ? 1u : 0u);   // equal keys: the first run's first
+      int m = 0;                                     // keys below lim
       if (len > 0)
         for (int step = w; step > 0; step >>= 1)
-          if (m + step <= len && q[m + step] < k) m += step;
+          if (m + step <= len && q[m + step] < lim) m += step;
       b[(i & ~(2 * w - 1)) + (i & (w - 1)) + m] = k;
     }
     __syncthreads();

@@ -408,3 +408,40 @@ def test_surfel_gradients_of_warps_of_8_and_of_32(torch_cuda, n):
         assert torch.equal(a[k], b[k][:n]), k
         assert not b[k][n:].any(), k
     assert float((a["pose6"] - b["pose6"]).abs().max()) <= 1e-5 * float(b["pose6"].abs().max())
+
+
+@pytest.mark.parametrize("n,grid,onto", [(300, (14, 9), (10, 6)), (4000, (14, 9), (10, 6)),
+                                         (3500, (5, 4), (2, 2))])
+def test_bins_of_rectangles_that_reach_past_the_grid(torch_cuda, n, grid, onto):
+    """Records of a larger tile grid: a pair's tile is y tiles_x + x, at most
+    the last one, so a tile can hold a surfel several times.  The forward-only
+    bins, whose keys are then equal, keep every pair, in the order of (tile,
+    depth, id), and hold what the bins with emission arrays hold."""
+    torch = torch_cuda
+    from paper_2506_00970_gb300 import gs2d
+    rect, depth, count = scenes.random_tile_records(8, n, *grid)
+    proj, tiles = records_to_proj(torch, rect, depth, count)
+    cam = scenes.Camera(100.0, 100.0, 8.0, 8.0, onto[0] * 16, onto[1] * 16)
+    pairs = []
+    for i, (x0, y0, x1, y1) in enumerate(rect):
+        if count[i] > 0:
+            y, x = np.mgrid[y0:y1 + 1, x0:x1 + 1]
+            pairs.append(np.stack([np.minimum(y * onto[0] + x, onto[0] * onto[1] - 1).ravel(),
+                                   np.full(y.size, i)]))
+    t, ids = np.concatenate(pairs, 1)
+    order = np.lexsort((ids, np.asarray(depth, np.float32).view(np.uint32)[ids], t))
+    assert (np.diff(ids[order]) == 0).any() and len(t) == count.sum()
+    r = gs2d.Rasterizer(cam, n, capacity=len(t) + 5)
+    r.proj.copy_(proj)
+    r.tiles.copy_(tiles)
+    whole = r.bins
+    forward = gs2d.Bins(None, whole.vals, None, None, whole.tile_ranges, whole.n_isect, whole.status,
+                        whole.capacity)
+    for bins in (forward, whole):
+        r.vals.fill_(-1)
+        r.status.zero_()
+        gs2d.gs2d_bin_sort(r.proj, r.tiles, n, r.cam, r.cfg, r.sort_ws, bins)
+        torch.cuda.synchronize()
+        assert int(r.status.item()) == 0 and int(r.n_isect.item()) == len(t)
+        np.testing.assert_array_equal(r.vals[: len(t)].cpu().numpy(), ids[order])
+        assert int(np.diff(r.ranges.cpu().numpy().reshape(-1, 2), axis=1).max()) == np.bincount(t).max()
