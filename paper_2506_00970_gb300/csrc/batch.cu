@@ -246,7 +246,7 @@ BatchWs carve_batch_ws(void* base, const gs2d_view* views, int n_views, int n) {
     const size_t cap = views[v].bins.capacity > 0 ? views[v].bins.capacity : 1;
     w.partials[v] = c.take<float>(cap * bwd_regions(views[v].cfg) * 16);
     const int m = views[v].active ? views[v].n_active : n;
-    w.pose_part[v] = c.take<float>((size_t)max(1, grad_blocks(m)) * 6);
+    w.pose_part[v] = c.take<float>((size_t)max(1, grad_blocks_room(m)) * 6);
   }
   w.bytes = align_up(c.off, 256);
   return w;

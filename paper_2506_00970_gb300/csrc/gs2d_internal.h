@@ -154,11 +154,15 @@ struct GradTable {
 // Surfels per warp: eight, whose partials a warp sums in one pass, while all
 // their warps fit one resident wave (152 SMs x 24); else 32, in up to four
 // passes.  4,096 surfels with eight regions a tile: 19.8 -> 11.6 us.
-inline int grad_surfels_per_warp(int m) { return m <= 152 * 24 * 8 ? 8 : 32; }
+constexpr int kGradSmallMap = 152 * 24 * 8;
+inline int grad_surfels_per_warp(int m) { return m <= kGradSmallMap ? 8 : 32; }
 inline int grad_blocks(int m) {
   const int per = 8 * grad_surfels_per_warp(m);
   return (m + per - 1) / per;
 }
+// The most blocks that any map of at most m surfels takes: what workspaces
+// have room for, so that one sized for a map also serves every smaller one.
+inline int grad_blocks_room(int m) { return max(grad_blocks(m), grad_blocks(min(m, kGradSmallMap))); }
 int surfel_grad_launch(const gs2d_surfels* s, const int32_t* active, int m, int mode, int Q,
                        const GradTable& t, float* d_mu, float* d_quat, float* d_scale,
                        float* d_opac, float* d_rgb, cudaStream_t st);

@@ -869,7 +869,7 @@ BwdWs carve_bwd_ws(void* base, int n, size_t cap, int n_tiles, bool full, int Q)
   Carver c(base);
   BwdWs w;
   w.partials = c.take<float>(full ? (cap > 0 ? cap : 1) * Q * kRedVals : 1);
-  const int nb = max(n_tiles, grad_blocks(n));
+  const int nb = max(n_tiles, grad_blocks_room(n));
   w.pose_part = c.take<float>((size_t)max(nb, 1) * 6);
   w.bytes = align_up(c.off, 256);
   return w;

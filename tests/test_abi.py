@@ -202,3 +202,30 @@ def test_tile_configs_are_validated_on_the_host(built_lib):
         assert rc == 1, (tile, px, rc)
         assert ok == (tile[0] * tile[1] == 256 * px and tile[0] % 8 == 0 and
                       tile[1] % (4 * px) == 0 and px in (1, 2, 3, 4))
+
+
+def test_backward_workspaces_grow_with_the_map(built_lib):
+    """A workspace sized for a map serves every smaller map, and one sized for
+    a view's largest active set every smaller one: the sizes never fall as the
+    map grows, on both sides of 29,184 surfels, where the reduction's blocks
+    change from 64 to 256 surfels."""
+    from paper_2506_00970_gb300 import gs2d
+    L, cfg = gs2d.lib(), gs2d.default_config()
+    sizes = [0, 1, 63, 64, 65, 4096, 20_000, 29_120, 29_183, 29_184, 29_185, 29_441, 40_000, 60_000,
+             116_735, 116_736, 116_737, 200_000, 2_000_000]
+    cams = [gs2d.Camera(100.0, 100.0, w / 2, h / 2, w, h, 0.05) for w, h in ((16, 16), (160, 120), (640, 480))]
+
+    def batch(cam, n, m):
+        views = (gs2d.View * 2)()
+        for k, active in enumerate((None, 8)):
+            bins = gs2d.Bins(None, 8, 8, 8, 8, 8, 8, 5000)
+            views[k] = gs2d.View(cam, cfg, 8, active, m, 16, 8, bins)
+        return L.gs2d_render_batch_workspace(views, 2, n)
+
+    for cam in cams:
+        tiles = L.gs2d_tiles_x(ctypes.byref(cam), ctypes.byref(cfg)) * \
+            L.gs2d_tiles_y(ctypes.byref(cam), ctypes.byref(cfg))
+        for need in (lambda n: gs2d.gs2d_render_bwd_workspace(n, 5000, tiles),
+                     lambda n: batch(cam, n, 100), lambda n: batch(cam, 2_000_000, n)):
+            got = [need(n) for n in sizes]
+            assert got == sorted(got) and got[0] > 0, got
