@@ -180,7 +180,7 @@ __device__ __forceinline__ void bwd_region(
         const F3 gC = f3(u0.x, u0.y, u0.z), gN = f3(u1.x, u1.y, u1.z);
         const float gD = u0.w;
         const float om = 1.f - e.a;
-        const float iom = __fdividef(1.f, om);
+        const float iom = rcp_ftz(om);
         const float Tb = T[k] * iom;
         const float w = e.a * Tb;
         const float vj = dot3(col, gC) + e.z * gD + dot3(tn, gN);

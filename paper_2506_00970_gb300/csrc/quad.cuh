@@ -213,7 +213,7 @@ __device__ __forceinline__ void quad_replay(const QuadStage<kBwdVec4>& s, int nh
     if (!hits) continue;
     // the lane's own pair, as far as it needs no running state
     const float4 r3 = s.rec[j][3], r4 = s.rec[j][4], r5 = s.rec[j][5], r6 = s.rec[j][6];
-    const float iom = __fdividef(1.f, 1.f - ev.a);
+    const float iom = rcp_ftz(1.f - ev.a);
     const float vj = fmaf(r2.w, pg.gC.x, fmaf(r3.x, pg.gC.y, fmaf(r3.y, pg.gC.z, ev.z * pg.gD)));
     // the pixel's state over the four pairs; the lane keeps its own w and ga
     float w = 0.f, ga = 0.f;

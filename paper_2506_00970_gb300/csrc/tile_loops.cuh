@@ -127,6 +127,26 @@ __device__ __forceinline__ int warp_hit_list(const uint32_t* s_mask, uint8_t* my
   return n;
 }
 
+// Approximate reciprocal and power of two of the pair loops.  They flush
+// denormals: without that each carries a scaling sequence for denormal
+// operands and results, which none of these quantities reaches: 1 - a is at
+// least 1 - alpha_max, exponents lie within the cutoff, and p2, of the order of
+// the product of the surfel's two scales, is that small for scales below 1e-19
+// or a disc seen edge-on.  Everything else keeps denormals: sums,
+// transmittances (t_min may be 0), the chain rule to the parameters, the pose
+// update.  10 tracking iterations at 640x480 1103 -> 1026 us, the 8-view
+// mapping step 6.37 -> 6.08 ms.
+__device__ __forceinline__ float rcp_ftz(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float exp2_ftz(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // Evaluation of one (pixel, surfel) pair shared by every pass, so all take
 // bit-identical skip decisions.  Returns false if skipped.
 struct Eval {
@@ -139,14 +159,14 @@ __device__ __forceinline__ bool eval_pair(const float4 r0, const float4 r1, cons
   const float p0 = fmaf(ly, r1.z, fmaf(lx, r0.w, r0.x));
   const float p1 = fmaf(ly, r1.w, fmaf(lx, r1.x, r0.y));
   const float p2 = fmaf(ly, r2.x, fmaf(lx, r1.y, r0.z));
-  e.rinv = __fdividef(1.0f, p2);
+  e.rinv = rcp_ftz(p2);
   e.u = __fmul_rn(p0, e.rinv);
   e.v = __fmul_rn(p1, e.rinv);
   const float rr = fmaf(e.u, e.u, __fmul_rn(e.v, e.v));
   if (!(rr <= cutoff_r2)) return false;
   e.z = __fmul_rn(r2.y, e.rinv);
   if (!(e.z > near_z)) return false;
-  e.G = __expf(-0.5f * rr);
+  e.G = exp2_ftz(__fmul_rn(rr, -0.72134752f));   // exp(-rr / 2): log2(e) / 2
   e.araw = __fmul_rn(r2.z, e.G);
   e.a = fminf(e.araw, alpha_max);
   return e.a >= alpha_min;
@@ -366,7 +386,7 @@ __device__ __forceinline__ void pose_pair(const Eval& e, const float4 r2, const 
   const F3 gC = pgk.gC, gN = pgk.gN;
   const float gD = pgk.gD;
   const float4 r3 = rec[3], r4 = rec[4], r5 = rec[5], r6 = rec[6];
-  const float iom = __fdividef(1.f, 1.f - e.a);
+  const float iom = rcp_ftz(1.f - e.a);
   const float Tb = T * iom;
   const float w = e.a * Tb;
   float vj = fmaf(r2.w, gC.x, fmaf(r3.x, gC.y, fmaf(r3.y, gC.z, e.z * gD)));

@@ -135,3 +135,18 @@ def test_covisibility_counts_and_keyframe_rule(torch_cuda, orc):
             assert float(sc.item()) == float(np.float32(score))
             assert bool(kf.item()) == orc.keyframe_rule(float(np.float32(score)), pa[9:], pb[9:],
                                                         c_k, 0.15)
+
+
+def test_covisibility_counts_denormal_contributions(torch_cuda):
+    """A contribution below the normal range is above a threshold of zero."""
+    torch = torch_cuda
+    from paper_2506_00970_gb300 import gs2d
+    ca = torch.tensor([1e-40, 0.0, 1e-40, 2e-40, 1.0], device="cuda")
+    cb = torch.tensor([1e-41, 1e-45, 0.0, 1e-40, 0.0], device="cuda")
+    pose = gs2d.pose_tensor(scenes.identity_pose())
+    counts = torch.zeros(2, dtype=torch.int32, device="cuda")
+    score, kf = torch.zeros(1, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    for thr, inter, union in ((0.0, 2, 5), (5e-41, 1, 4)):
+        gs2d.gs2d_covisibility(ca, cb, 5, thr, pose, pose, 0.9, 0.15, counts, score, kf)
+        torch.cuda.synchronize()
+        assert counts.tolist() == [inter, union]

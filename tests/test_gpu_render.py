@@ -445,3 +445,63 @@ def test_bins_of_rectangles_that_reach_past_the_grid(torch_cuda, n, grid, onto):
         assert int(r.status.item()) == 0 and int(r.n_isect.item()) == len(t)
         np.testing.assert_array_equal(r.vals[: len(t)].cpu().numpy(), ids[order])
         assert int(np.diff(r.ranges.cpu().numpy().reshape(-1, 2), axis=1).max()) == np.bincount(t).max()
+
+
+def _facing_slab(n, length):
+    """A slab whose discs face the camera: quaternions (length, 0, 0, 0), whose
+    rotation is exactly the identity whatever the length."""
+    s = scenes.slab_scene(5, n)
+    s.quat[:] = [length, 0.0, 0.0, 0.0]
+    return s
+
+
+@pytest.mark.parametrize("batched", [False, True])
+def test_gradients_of_tiny_quaternions(torch_cuda, batched):
+    """Quaternions need not be normalised: at length 2^-65, whose square is a
+    denormal, the gradients are the unit ones', the quaternion's times 2^65.
+    Only the approximate 1 / |q| differs, by 2 units in the last place, three
+    times in the quaternion's gradient: 1e-6."""
+    torch = torch_cuda
+    from paper_2506_00970_gb300 import gs2d
+    cam, pose = scenes.Camera(150.0, 150.0, 80.0, 60.0, 160, 120), scenes.identity_pose()
+    up = [torch.tensor(u, dtype=torch.float32, device="cuda")
+          for u in scenes.random_upstream(3, 120, 160)[:2]]
+    out = []
+    for length in (1.0, 2.0 ** -65):
+        s = _facing_slab(2000, length)
+        ds = gs2d.DeviceSurfels(s)
+        if batched:
+            br = gs2d.BatchRasterizer([cam], s.n, capacities=[400_000])
+            br.set_poses([pose])
+            br.forward(ds)
+            br.keep[0]["d_rgb"].copy_(up[0])
+            br.keep[0]["d_depth"].copy_(up[1])
+            g = br.backward(ds)
+        else:
+            r = gs2d.Rasterizer(cam, s.n, capacity=400_000)
+            r.forward(ds, gs2d.pose_tensor(pose))
+            g = r.backward(ds, gs2d.pose_tensor(pose), *up)
+        out.append({k: g[k].double().cpu().reshape(s.n, -1) for k in ("mu", "quat", "scale", "opacity", "rgb")})
+    out[1]["quat"] *= 2.0 ** -65
+    for k in out[0]:
+        lim = 1e-6 * float(out[0][k].abs().max())
+        assert lim > 0 and float((out[0][k] - out[1][k]).abs().max()) <= lim, k
+
+
+def test_gradients_below_the_normal_range(torch_cuda):
+    """Upstream gradients of 2^-135 give the colour gradients of 1 times 2^-135,
+    denormals most of them: each of at most 19,200 pixels adds one rounding to a
+    multiple of 2^-149 in its product and one in the sum."""
+    torch = torch_cuda
+    from paper_2506_00970_gb300 import gs2d
+    cam, pose = scenes.Camera(150.0, 150.0, 80.0, 60.0, 160, 120), gs2d.pose_tensor(scenes.identity_pose())
+    s = _facing_slab(2000, 1.0)
+    ds, r, out = gs2d.DeviceSurfels(s), gs2d.Rasterizer(cam, s.n, capacity=400_000), []
+    r.forward(ds, pose)
+    for scale in (1.0, 2.0 ** -135):
+        g = r.backward(ds, pose, torch.full((120, 160, 3), scale, device="cuda"),
+                       torch.zeros(120, 160, device="cuda"))
+        out.append(g["rgb"].double().cpu())
+    want = out[0] * 2.0 ** -135
+    assert float(want.max()) > 19_200 * 2.0 ** -149
+    assert float((out[1] - want).abs().max()) <= 19_200 * 2.0 ** -149
