@@ -91,3 +91,21 @@ def test_mapping_loss_with_ssim(torch_cuda, orc):
     torch.cuda.synchronize()
     assert float(loss.item()) == pytest.approx(L, rel=1e-5)
     _grad_close(to_np(out[0]), g["rgb"])
+
+
+@pytest.mark.parametrize("value", [1.2e19, 1e20, 3e19])
+def test_ssim_of_equal_images_with_a_huge_pixel(torch_cuda, value):
+    """Where the images agree the loss and its gradient are exactly zero, also
+    where the variances overflow to infinity or their reciprocals are below the
+    normal range."""
+    torch = torch_cuda
+    from paper_2506_00970_gb300 import gs2d
+    h, w = 48, 56
+    x = torch.rand(h, w, 3, generator=torch.Generator().manual_seed(1))
+    x[20, 30] = value
+    x = x.cuda()
+    g_x, loss = torch.zeros(h, w, 3, device="cuda"), torch.zeros(1, device="cuda")
+    ws = torch.empty(gs2d.gs2d_ssim_workspace(h, w), dtype=torch.uint8, device="cuda")
+    gs2d.gs2d_ssim_loss(x, x, h, w, 0.125, g_x, loss, ws)
+    torch.cuda.synchronize()
+    assert float(loss.item()) == 0.0 and not g_x.any()
