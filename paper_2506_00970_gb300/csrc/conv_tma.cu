@@ -37,6 +37,7 @@
 
 #include "conv_tma.h"
 #include "gs2d_common.cuh"
+#include "per_device.h"
 
 namespace gs2d {
 namespace net {
@@ -695,6 +696,28 @@ __global__ void __launch_bounds__(kConvThreads) dgrad_tma_kernel(
                  "r"(C::TMEM_COLS));
 }
 
+// Raises a kernel's dynamic shared-memory limit on the current device, once
+// per device and kernel (limits: the kernel's own table), before any stream
+// capture that runs it.  With threads, *resident = the CTAs that the device
+// holds at once.
+int prepare_kernel(const void* kern, int smem, PerDevice& limits, int threads = 0,
+                   int* resident = nullptr) {
+  int dev = 0, value = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return (int)e;
+  const int r = limits.get(dev, &value, [&](int* v) {
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess || !threads) return (int)e;
+    int per_sm = 0, sms = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    *v = max(per_sm, 1) * max(sms, 1);
+    return (int)e;
+  });
+  if (resident) *resident = value;
+  return r;
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
                                   const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -748,19 +771,12 @@ int run(const bf16* x, int B, const bf16* w, const float* bias, bf16* out, int* 
           CU_TENSOR_MAP_INTERLEAVE_NONE, C::SW == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return GS2D_ERR_CUDA;
-  // the dynamic shared memory exceeds the 48 KB default: raise the limit once
-  // (before any stream capture that runs the network)
-  static std::once_flag smem_once;
-  static cudaError_t smem_err = cudaSuccess;
-  std::call_once(smem_once, [] {
-    smem_err = cudaFuncSetAttribute(conv_tma_kernel<CIN, COUT, HI, WI, TW, TH, S, NI, NB>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-  });
-  if (smem_err != cudaSuccess) return GS2D_ERR_CUDA;
+  static PerDevice limits;
+  const auto kern = conv_tma_kernel<CIN, COUT, HI, WI, TW, TH, S, NI, NB>;
+  if (prepare_kernel(reinterpret_cast<const void*>(kern), C::SMEM, limits)) return GS2D_ERR_CUDA;
   const int grid = NI == 1 ? B * C::TX * C::TY : (B + NI - 1) / NI;
   if (grid <= 0) return GS2D_OK;
-  conv_tma_kernel<CIN, COUT, HI, WI, TW, TH, S, NI, NB>
-      <<<dim3(grid, C::NSPLIT), kConvThreads, C::SMEM, st>>>(mx, mw, bias, out, B, err);
+  kern<<<dim3(grid, C::NSPLIT), kConvThreads, C::SMEM, st>>>(mx, mw, bias, out, B, err);
   GS2D_LAUNCH_CHECK();
   return GS2D_OK;
 }
@@ -796,27 +812,14 @@ int run_pers(const bf16* x, int B, const bf16* w, const float* bias, bf16* out, 
           CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return GS2D_ERR_CUDA;
-  // the dynamic shared memory exceeds the 48 KB default: raise the limit
-  // and size the resident grid once (before any stream capture)
-  static std::once_flag once;
-  static cudaError_t once_err = cudaSuccess;
-  static int resident = 0;
-  std::call_once(once, [] {
-    auto kern = conv_tma_pers_kernel<CIN, COUT, HI, WI, TW, TH, S>;
-    once_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    int per_sm = 0, dev = 0, sms = 0;
-    if (once_err == cudaSuccess)
-      once_err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPersThreads, C::SMEM);
-    if (once_err == cudaSuccess) once_err = cudaGetDevice(&dev);
-    if (once_err == cudaSuccess)
-      once_err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    resident = max(per_sm, 1) * max(sms, 1);
-  });
-  if (once_err != cudaSuccess) return GS2D_ERR_CUDA;
+  static PerDevice limits;
+  int resident = 0;
+  const auto kern = conv_tma_pers_kernel<CIN, COUT, HI, WI, TW, TH, S>;
+  if (prepare_kernel(reinterpret_cast<const void*>(kern), C::SMEM, limits, kPersThreads, &resident))
+    return GS2D_ERR_CUDA;
   const int n_tiles = B * C::TX * C::TY;
   if (n_tiles <= 0) return GS2D_OK;
-  conv_tma_pers_kernel<CIN, COUT, HI, WI, TW, TH, S>
-      <<<min(n_tiles, resident), kPersThreads, C::SMEM, st>>>(mx, mw, bias, out, n_tiles, err);
+  kern<<<min(n_tiles, resident), kPersThreads, C::SMEM, st>>>(mx, mw, bias, out, n_tiles, err);
   GS2D_LAUNCH_CHECK();
   return GS2D_OK;
 }
@@ -850,16 +853,11 @@ int run_dgrad(const bf16* dz, int B, const bf16* w, const bf16* act, bf16* out,
           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return GS2D_ERR_CUDA;
-  static std::once_flag smem_once;
-  static cudaError_t smem_err = cudaSuccess;
-  std::call_once(smem_once, [] {
-    smem_err = cudaFuncSetAttribute(dgrad_tma_kernel<CIN, COUT, HI, WI, TW, TH, S, NI, NB, Z>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-  });
-  if (smem_err != cudaSuccess) return GS2D_ERR_CUDA;
+  static PerDevice limits;
+  const auto kern = dgrad_tma_kernel<CIN, COUT, HI, WI, TW, TH, S, NI, NB, Z>;
+  if (prepare_kernel(reinterpret_cast<const void*>(kern), C::SMEM, limits)) return GS2D_ERR_CUDA;
   const int tiles = NI == 1 ? B * C::TX * C::TY : (B + NI - 1) / NI;
-  dgrad_tma_kernel<CIN, COUT, HI, WI, TW, TH, S, NI, NB, Z>
-      <<<dim3(4 * tiles, C::NSPLIT), kConvThreads, C::SMEM, st>>>(mz, mw, act, out, B, tiles, splits, err);
+  kern<<<dim3(4 * tiles, C::NSPLIT), kConvThreads, C::SMEM, st>>>(mz, mw, act, out, B, tiles, splits, err);
   GS2D_LAUNCH_CHECK();
   return GS2D_OK;
 }

@@ -47,6 +47,7 @@
 #include "f32x2.cuh"
 #include "gs2d_common.cuh"
 #include "gs2d_internal.h"
+#include "per_device.h"
 
 namespace gs2d {
 
@@ -329,13 +330,14 @@ int ssim_launch(const float* x, const float* y, int height, int width, float wei
   const size_t need = ssim_ws_bytes(height, width);
   if (ws_needed) *ws_needed = need;
   if (!workspace || ws_bytes < need) return GS2D_ERR_WORKSPACE;
-  static bool attr_set = false;
-  if (!attr_set) {
-    if (cudaFuncSetAttribute(ssim_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kSsimSmemBytes) != cudaSuccess)
-      return GS2D_ERR_CUDA;
-    attr_set = true;
-  }
+  static PerDevice limits;
+  int dev = 0, unused = 0;
+  GS2D_CUDA_TRY(cudaGetDevice(&dev));
+  if (limits.get(dev, &unused, [](int*) {
+        return (int)cudaFuncSetAttribute(ssim_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kSsimSmemBytes);
+      }))
+    return GS2D_ERR_CUDA;
   const dim3 grid((width + kSsimT - 1) / kSsimT, (height + kSsimT - 1) / kSsimT, 3);
   float* part = static_cast<float*>(workspace);
   ssim_kernel<<<grid, kSsimThreads, kSsimSmemBytes, st>>>(x, y, height, width, weight,
