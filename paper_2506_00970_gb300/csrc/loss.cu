@@ -396,7 +396,8 @@ int gs2d_mapping_loss_batch(const gs2d_loss_view* views, int n_views, float w_d,
     const long long mine = (long long)d.strips_x * strips_along(x.cam.height, rows);
     d.n_items = (int)mine;
     items += mine;
-    if (items > 0x7FFFFFFF / kLossWarps) return GS2D_ERR_INVALID_ARG;
+    // an int counts strips, past the last one by at most a grid's stride
+    if (items > 0x7FFFFFFF - (1 << 20)) return GS2D_ERR_INVALID_ARG;
   }
   tab.n_items = (int)items;
   const size_t need = gs2d_mapping_loss_batch_workspace(views, n_views);

@@ -229,3 +229,15 @@ def test_backward_workspaces_grow_with_the_map(built_lib):
                      lambda n: batch(cam, n, 100), lambda n: batch(cam, 2_000_000, n)):
             got = [need(n) for n in sizes]
             assert got == sorted(got) and got[0] > 0, got
+
+
+def test_mapping_loss_batch_takes_images_of_a_thousand_million_pixels(built_lib):
+    """Views of one-pixel columns: 500 million strips of 28 x 4 pixels are
+    counted in an int (a missing workspace is what is reported); 2,147 million
+    are not."""
+    from paper_2506_00970_gb300 import gs2d
+    L = gs2d.lib()
+    cam = gs2d.Camera(100.0, 100.0, 0.5, 30.0, 1, 1_000_000_000, 0.05)
+    for n, rc in ((1, 2), (2, 2), (8, 2), (9, 1), (32, 1)):
+        views = (gs2d.LossView * n)(*([gs2d.LossView(cam, *([8] * 10))] * n))
+        assert L.gs2d_mapping_loss_batch(views, n, 0.5, 0.02, 8, None, 0, None, None) == rc, n
