@@ -237,7 +237,7 @@ int gs2d_render_count(const float* proj, const gs2d_bins* bins, const gs2d_camer
  * rest, where each pixel's serial walk over its tile's list is the bound.
  * -1 (the default): gs2d_render_fwd takes that form for at most twice the
  * device's SM count of tiles, gs2d_track_step decides tile by tile from the
- * list lengths; 0 = never.  Process-wide; read at each launch (so a captured
+ * list lengths for maps of more than 8,000 surfels and 30 a tile; 0 = never.  Process-wide; read at each launch (so a captured
  * graph keeps the form it was captured with).  Not thread-safe against
  * concurrent launches from other host threads. */
 void gs2d_set_grouped_tiles(int max_tiles);

@@ -284,6 +284,29 @@ __device__ __forceinline__ void key_ids(const unsigned long long* keys, int n, u
   __syncthreads();
 }
 
+// The same for n <= kRankKeys unsorted, distinct keys: a key's place is its
+// rank, counted by its own thread -- one pass and one barrier, where the runs
+// and merges of the sort have four to six at these lengths.  The keys are
+// visible to the block and 16-byte aligned.  40 iterations of whole tiles at
+// 640x480, 26,400 surfels: 1895 -> 1770 us with the launch rule below; lists
+// cut off at 64, 128 or 256 keys measure alike.
+constexpr int kRankKeys = 256;
+__device__ __forceinline__ void rank_ids(const unsigned long long* keys, int n, uint32_t* ids,
+                                         int n_ids) {
+  static_assert(kRankKeys <= kTileThreads, "a key per thread");
+  if ((int)threadIdx.x < n) {
+    const unsigned long long k = keys[threadIdx.x];
+    int rank = 0, j = 0;
+    for (; j + 1 < n; j += 2) {
+      const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(keys + j);
+      rank += (int)(kk.x < k) + (int)(kk.y < k);
+    }
+    if (j < n) rank += (int)(keys[j] < k);
+    ids[rank] = min((uint32_t)(k & 0xFFFFFFFFull), (uint32_t)(n_ids - 1));
+  }
+  __syncthreads();
+}
+
 // Fused tracking iteration on one tile: the depth sort of the tile's
 // segment, forward compositing, the tracking loss and its image gradient per
 // pixel (in registers), and the pose-only backward replay -- the images never
@@ -323,11 +346,15 @@ __device__ __forceinline__ void track_tile(
     if (len <= kSegSmem) {
       for (int i = threadIdx.x; i < len; i += kTileThreads) keys[i] = ts.seg_keys[start + i];
       __syncthreads();
-      if (len <= kTwice)   // room for two copies
-        keys = merge_sort(keys, keys + kTwice, len);
-      else
-        bitonic_sort(keys, len);
-      key_ids(keys, len, s_ids, ts.n);
+      if (len <= kRankKeys) {
+        rank_ids(keys, len, s_ids, ts.n);
+      } else {
+        if (len <= kTwice)   // room for two copies
+          keys = merge_sort(keys, keys + kTwice, len);
+        else
+          bitonic_sort(keys, len);
+        key_ids(keys, len, s_ids, ts.n);
+      }
       ids = s_ids;
     } else {
       sort_long_segment<kSegSmem>(tile, proj, ts.n, tiles_x, ranges, ts.seg_keys, ts.seg_tmp,
@@ -443,7 +470,7 @@ __global__ void __launch_bounds__(kTileThreads, tile_blocks_per_sm<P>()) track_t
 // the loss and replays.  The first `split` tiles of the launch order have four
 // blocks each (three of them leave at once when their tile runs whole), the
 // others one; SplitRule says where the line lies.  Segments of more than
-// kQuadKeys keys run whole.
+// kQuadKeys keys run whole, and maps of few surfels do not come here at all.
 // A quadrant writes one partial per 8 x 4 pixel block and the last of the
 // tile's four blocks adds the eight up in the whole-tile form's order, so the
 // results do not depend on the choice.
@@ -475,6 +502,17 @@ constexpr int kTileParts = kTileThreads / 32;   // 8 x 4 blocks (partials) per t
 // each follow the tiles (their early exits then cost nothing where no tile
 // splits); in larger grids only the half of the SM count longest tiles may,
 // and their blocks lead the launch, so that they overlap the whole of it.
+//
+// Maps of few surfels for the grid have no lists worth splitting, and
+// track_quad_kernel then costs more than track_tile_kernel<1>: its blocks that
+// only leave, and more code to fetch.  Up to the line, 8,000 surfels and 30 more
+// a tile, whole tiles were no slower at any grid; 40 iterations, us, whole
+// tiles -> quadrants (median of three maps) at 0.6 / 1 / 1.5 / 2.2 times its
+// surfels:
+//   160x120   1234 -> 1249  1315 -> 1328  1413 -> 1412  1707 -> 1586
+//   320x240   1328 -> 1400  1455 -> 1487  1592 -> 1644  1853 -> 1789
+//   480x360   1498 -> 1538  1740 -> 1805  1985 -> 2033  2298 -> 2246
+//   640x480   1770 -> 1847  2159 -> 2277  2470 -> 2574  2961 -> 3074
 struct SplitRule {
   int split;         // tiles (in launch order) that may run on quadrants
   int extras_first;  // their four blocks each lead the grid
@@ -547,12 +585,16 @@ __global__ void __launch_bounds__(kTileThreads, 4) track_quad_kernel(
     }
     __syncthreads();
     const int n = s.cnt;
-    unsigned long long* sorted = s.keys;
-    if (n <= kQuadKeys / 2)   // room for two copies
-      sorted = merge_sort(s.keys, s.keys + kQuadKeys / 2, n);
-    else
-      bitonic_sort(s.keys, n);
-    key_ids(sorted, n, s.ids, ts.n);
+    if (n <= kRankKeys) {
+      rank_ids(s.keys, n, s.ids, ts.n);
+    } else {
+      unsigned long long* sorted = s.keys;
+      if (n <= kQuadKeys / 2)   // room for two copies
+        sorted = merge_sort(s.keys, s.keys + kQuadKeys / 2, n);
+      else
+        bitonic_sort(s.keys, n);
+      key_ids(sorted, n, s.ids, ts.n);
+    }
     auto stage = [&](int b, int cnt) {   // entries b .. b + cnt - 1; returns the warp's hits
       if ((int)threadIdx.x < cnt) {
         stage_record_to<kBwdVec4>(proj, s.ids[b + threadIdx.x], xt, yt, s.st.rec[threadIdx.x]);
@@ -904,9 +946,15 @@ static bool use_grouped(int px_per_thread, int n_tiles) {
   return n_tiles <= (g_grouped_max_tiles < 0 ? 2 * sm_count() : g_grouped_max_tiles);
 }
 
+// Whether a tracking iteration over n surfels runs the kernel whose tiles may
+// split (see SplitRule).
+static bool track_splits(int n, int n_tiles) {
+  if (g_grouped_max_tiles >= 0) return n_tiles <= g_grouped_max_tiles;
+  return n > 8000 + 30 * n_tiles;
+}
+
 static SplitRule split_rule(int n_tiles) {
-  if (g_grouped_max_tiles >= 0)
-    return SplitRule{n_tiles <= g_grouped_max_tiles ? n_tiles : 0, 0, 0, 0.f};
+  if (g_grouped_max_tiles >= 0) return SplitRule{n_tiles, 0, 0, 0.f};
   const int sms = max(sm_count(), 1), slots = 4 * sms;
   if (n_tiles <= 2 * sms) return SplitRule{n_tiles, 0, 80, 1.25f / slots};
   return SplitRule{min(sms / 2, n_tiles), 1, 80, 1.75f / slots};
@@ -950,7 +998,7 @@ int track_tile_launch(const float* proj, const gs2d_bins* bins, const gs2d_camer
       !loss_part || !pose_part || !ts.pose || !ts.adam || !ts.counter || !status)
     return GS2D_ERR_INVALID_ARG;
   const int tx = gs2d_tiles_x(cam, cfg), ty = gs2d_tiles_y(cam, cfg);
-  if (cfg->px_per_thread == 1) {
+  if (cfg->px_per_thread == 1 && track_splits(ts.n, tx * ty)) {
     if (!bins->n_isect || !ts.order || !ts.quad_part || !ts.quad_done) return GS2D_ERR_INVALID_ARG;
     const SplitRule rule = split_rule(tx * ty);
     track_quad_kernel<<<tx * ty + (kQuads - 1) * rule.split, kTileThreads, 0, st>>>(
@@ -958,6 +1006,7 @@ int track_tile_launch(const float* proj, const gs2d_bins* bins, const gs2d_camer
         *cfg, tx, tx * ty, obs_rgb, obs_depth, *prm, loss_part, pose_part, rule, ts, status);
   } else {
     switch (cfg->px_per_thread) {
+      case 1: GS2D_TRACK_TILE(1); break;
       case 2: GS2D_TRACK_TILE(2); break;
       case 3: GS2D_TRACK_TILE(3); break;
       default: GS2D_TRACK_TILE(4); break;

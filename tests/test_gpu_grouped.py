@@ -156,3 +156,36 @@ def test_tiles_four_pixels_high_have_quadrants_of_their_own(torch_cuda, w, h, f)
     assert out[0]["opacity"].max() > 0.9
     assert_images_close(out[1], {k: out[0][k].astype(np.float64)
                                  for k in ("rgb", "depth", "normal", "opacity")})
+
+
+@pytest.mark.parametrize("w,h,f", [(160, 120, 150.0), (333, 251, 275.0)])
+@pytest.mark.parametrize("past", [0, 1])
+def test_tracking_forms_agree_at_the_line_between_their_launches(torch_cuda, w, h, f, past):
+    """The last map size that runs whole tiles only, and the first whose tiles
+    may split (8,000 surfels and 30 a tile); lists of up to 256 keys, which are
+    ordered by rank, and longer ones: bit-identical histories in every form."""
+    torch = torch_cuda
+    from paper_2506_00970_gb300 import gs2d
+    cam = scenes.Camera(f, f, w / 2, h / 2, w, h)
+    n_tiles = -(-w // 16) * -(-h // 16)
+    s = scenes.room_scene(4, 8000 + 30 * n_tiles + past)
+    ds, gt = gs2d.DeviceSurfels(s), scenes.room_pose(11)
+    img = gs2d.Rasterizer(cam, s.n).forward(ds, gs2d.pose_tensor(gt))
+    obs = img["rgb"].clone(), img["depth"] / img["opacity"].clamp_min(1e-6)
+    ccam, cfg, cap = gs2d.camera(cam), gs2d.default_config(), 8 * s.n
+    res = []
+    for limit in (0, 1 << 30, -1):
+        gs2d.gs2d_set_grouped_tiles(limit)
+        ws = torch.empty(gs2d.gs2d_track_workspace(s.n, cap, ccam, cfg), dtype=torch.uint8, device="cuda")
+        pose = gs2d.pose_tensor(scenes.perturb_pose(gt, 0.02, 1.0, seed=7))
+        lh, gh = torch.zeros(4, device="cuda"), torch.zeros(4, 6, device="cuda")
+        gs2d.gs2d_track_step(ds, ccam, cfg, gs2d.default_track_params(stop_tol=0.0), pose, *obs, 4, cap,
+                             lh, None, ws, grad_hist=gh)
+        torch.cuda.synchronize()
+        assert int(gs2d.gs2d_track_status(ws).item()) == 0
+        res.append((lh, gh, pose))
+    gs2d.gs2d_set_grouped_tiles(-1)
+    assert float(res[0][0][0]) > 0
+    for other in res[1:]:
+        for a, b in zip(res[0], other):
+            assert torch.equal(a, b)
