@@ -77,16 +77,33 @@ __global__ void __launch_bounds__(256) sum_parts_kernel(const float* __restrict_
 // instructions a pixel (31 us at 1200x680, 197 us for eight such views, 7.9
 // us at 160x120).  R = 4: 24, 140 and 11.8 us; taller strips repeat fewer
 // halo rows but chain more latencies (R = 6: 21, 147, 14.5 us; R = 16: 45 us
-// at 1200x680); R = 2 where R = 4 would leave fewer than eight warps per SM
-// (160x120: 8.8 us).
+// at 1200x680).
+//
+// Up to 200,000 pixels the strips are too few to hide those latencies among
+// warps: R = 2, every input of the strip loaded before the first is used (with
+// registers for 16 warps per SM, which is all there are), and in a batch
+// blocks of two warps, so that they spread over the SMs.  Device time of a
+// call in a graph, us, views of one size -- the tiles / R = 2 without that up to
+// 136,000 pixels and R = 4 beyond / now:
+//   1, 8 x 64x48     5.7  6.7  5.4     6.1  7.2  5.9
+//   1, 8 x 160x120   6.6  7.1  5.8     8.7 10.5  8.0
+//   1, 2 x 320x240   6.9  8.4  7.3     8.6 10.8  9.3
+//   1, 2 x 480x360  10.6 11.4 10.1    15.5 12.9 13.0
+//   one view's own call: 160x120  5.8 6.1 5.3, 320x240  7.3 7.0 6.4
 constexpr int kStripW = 28;        // output columns of a strip
 constexpr int kStripRows = 4;      // and rows
 constexpr int kStripRowsSmall = 2;
+constexpr int kSmallImages = 200000;   // pixels of a call
 constexpr int kLossWarps = kLossThreads / 32;
 
 __host__ __device__ inline int strips_along(int n, int step) { return (n + step - 1) / step; }
-inline int strip_rows(long long px) {
-  return px >= 8ll * 152 * kStripW * kStripRows ? kStripRows : kStripRowsSmall;
+inline int strip_rows(long long px) { return px >= kSmallImages ? kStripRows : kStripRowsSmall; }
+// Threads of a batch kernel's block, and blocks per SM of either kernel.
+__host__ __device__ constexpr int batch_threads(int rows) {
+  return rows == kStripRows ? kLossThreads : 64;
+}
+constexpr int loss_blocks_per_sm(int rows, int threads) {
+  return (rows == kStripRows ? 32 : 16) / (threads / 32);
 }
 
 __device__ __forceinline__ F3 cross_rn(F3 a, F3 b) {
@@ -123,6 +140,7 @@ __device__ __forceinline__ float mapping_loss_strip(int x0, int y0,
   // D / max(O, 1e-6), O and D of rows y0 - 2 .. y0 + R + 1 (0 outside
   // the image)
   constexpr int kR = R + 4;
+  constexpr bool kAhead = R == kStripRowsSmall;
   float dv[kR], ov[kR], Dv[kR];
 #pragma unroll
   for (int k = 0; k < kR; ++k) {
@@ -132,6 +150,30 @@ __device__ __forceinline__ float mapping_loss_strip(int x0, int y0,
       const int i = y * W + px;
       ov[k] = __ldg(im.opac + i);
       Dv[k] = __ldg(im.depth + i);
+    }
+  }
+  // kAhead: the other inputs too, N_r of rows y0 - 1 .. y0 + R and the colours
+  // and observed depths of the strip's own
+  F3 nr_in[kAhead ? R + 2 : 1], rgb_in[kAhead ? R : 1], obs_in[kAhead ? R : 1];
+  float od_in[kAhead ? R : 1];
+  auto rgb_at = [](const float* p, int i) {
+    return f3(__ldg(p + 3 * i), __ldg(p + 3 * i + 1), __ldg(p + 3 * i + 2));
+  };
+  if (kAhead) {
+#pragma unroll
+    for (int k = 0; k < R + 2; ++k) {
+      const int y = y0 - 1 + k;
+      nr_in[k] = f3(0.f, 0.f, 0.f);
+      if (in_x && y >= 0 && y < H) nr_in[k] = rgb_at(im.normal, y * W + px);
+    }
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      const int i = (y0 + k) * W + px;
+      if (out_x && y0 + k < H) {
+        rgb_in[k] = rgb_at(im.rgb, i);
+        obs_in[k] = rgb_at(im.obs_rgb, i);
+        od_in[k] = __ldg(im.obs_depth + i);
+      }
     }
   }
 #pragma unroll
@@ -170,8 +212,7 @@ __device__ __forceinline__ float mapping_loss_strip(int x0, int y0,
         ok = true;
         const float inn = rsqrtf(n2);  // 1 / |n|
         const F3 ND = inn * n;
-        const F3 Nr = f3(__ldg(im.normal + 3 * i), __ldg(im.normal + 3 * i + 1),
-                         __ldg(im.normal + 3 * i + 2));
+        const F3 Nr = kAhead ? nr_in[kAhead ? k - 1 : 0] : rgb_at(im.normal, i);
         const float dp = dot3(ND, Nr);
         Ln = 1.f - dp;
         gNr = (-1.f) * ND;
@@ -200,10 +241,11 @@ __device__ __forceinline__ float mapping_loss_strip(int x0, int y0,
       const float O = ou, Dh = du;
       const float Oc = fmaxf(O, 1e-6f);
       const float D = Dv[k - 1];
-      const float d0 = __ldg(im.rgb + 3 * i) - __ldg(im.obs_rgb + 3 * i);
-      const float d1 = __ldg(im.rgb + 3 * i + 1) - __ldg(im.obs_rgb + 3 * i + 1);
-      const float d2 = __ldg(im.rgb + 3 * i + 2) - __ldg(im.obs_rgb + 3 * i + 2);
-      const float ddp = Dh - __ldg(im.obs_depth + i);
+      const int own = kAhead ? k - 3 : 0;   // the strip's row
+      const F3 cr = kAhead ? rgb_in[own] : rgb_at(im.rgb, i);
+      const F3 co = kAhead ? obs_in[own] : rgb_at(im.obs_rgb, i);
+      const float d0 = cr.x - co.x, d1 = cr.y - co.y, d2 = cr.z - co.z;
+      const float ddp = Dh - (kAhead ? od_in[own] : __ldg(im.obs_depth + i));
       acc += fmaf(w_l1, fabsf(d0) + fabsf(d1) + fabsf(d2), __fmul_rn(w_d, fabsf(ddp)));
       const float sl = w_l1 * inv;
       im.g_rgb[3 * i] = sgnf(d0) * sl;
@@ -237,7 +279,7 @@ __device__ __forceinline__ float mapping_loss_strip(int x0, int y0,
 }
 
 template <int R>
-__global__ void __launch_bounds__(kLossThreads, 4) mapping_loss_kernel(
+__global__ void __launch_bounds__(kLossThreads, loss_blocks_per_sm(R, kLossThreads)) mapping_loss_kernel(
     MapLossImages im, gs2d_camera cam, float w_l1, float w_d, float w_n,
     float* __restrict__ part) {
   __shared__ float s[kLossWarps];
@@ -268,10 +310,11 @@ struct LossTable {
 };
 
 template <int R>
-__global__ void __launch_bounds__(kLossThreads, 4) mapping_loss_batch_kernel(
-    const LossTable tab, float w_d, float w_n, float* __restrict__ part) {
-  for (int item = blockIdx.x * kLossWarps + (threadIdx.x >> 5); item < tab.n_items;
-       item += gridDim.x * kLossWarps) {
+__global__ void __launch_bounds__(batch_threads(R), loss_blocks_per_sm(R, batch_threads(R)))
+    mapping_loss_batch_kernel(const LossTable tab, float w_d, float w_n, float* __restrict__ part) {
+  constexpr int kWarps = batch_threads(R) / 32;
+  for (int item = blockIdx.x * kWarps + (threadIdx.x >> 5); item < tab.n_items;
+       item += gridDim.x * kWarps) {
     int v = 0;
     while (v + 1 < tab.n_views && item >= tab.v[v + 1].item0) ++v;
     const LossViewDev& V = tab.v[v];
@@ -405,8 +448,8 @@ int gs2d_mapping_loss_batch(const gs2d_loss_view* views, int n_views, float w_d,
   if (!workspace || ws_bytes < need) return GS2D_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   float* part = static_cast<float*>(workspace);
-  // a resident grid (the partials are per item, so the result does not
-  // depend on it)
+  // a resident grid, or every strip's block (the partials are per item, so
+  // the result does not depend on it)
   static int slots[64] = {};
   int dev = 0;
   GS2D_CUDA_TRY(cudaGetDevice(&dev));
@@ -414,13 +457,16 @@ int gs2d_mapping_loss_batch(const gs2d_loss_view* views, int n_views, float w_d,
   if (!slots[dev]) {
     int sms = 0;
     GS2D_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    slots[dev] = 4 * max(1, sms);   // the launch bounds' blocks per SM
+    slots[dev] = loss_blocks_per_sm(kStripRows, kLossThreads) * max(1, sms);
   }
-  const int blocks = min(slots[dev], strips_along(tab.n_items, kLossWarps));
-  if (rows == kStripRows)
+  if (rows == kStripRows) {
+    const int blocks = min(slots[dev], strips_along(tab.n_items, kLossWarps));
     mapping_loss_batch_kernel<kStripRows><<<blocks, kLossThreads, 0, st>>>(tab, w_d, w_n, part);
-  else
-    mapping_loss_batch_kernel<kStripRowsSmall><<<blocks, kLossThreads, 0, st>>>(tab, w_d, w_n, part);
+  } else {
+    constexpr int kThreads = batch_threads(kStripRowsSmall);
+    mapping_loss_batch_kernel<kStripRowsSmall>
+        <<<strips_along(tab.n_items, kThreads / 32), kThreads, 0, st>>>(tab, w_d, w_n, part);
+  }
   GS2D_LAUNCH_CHECK();
   mapping_loss_batch_sum_kernel<<<n_views, 256, 0, st>>>(tab, part, loss_out);
   GS2D_LAUNCH_CHECK();

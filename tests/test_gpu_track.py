@@ -360,3 +360,53 @@ def test_track_step_beyond_the_fused_scatter_tile_count(torch_cuda, orc):
         assert int(gs2d.gs2d_track_status(ws).item()) in (0, gs2d.CONVERGED), cam.width
         assert float(lh[0].item()) == pytest.approx(float(loss.item()), rel=1e-4), cam.width
         assert float(lh[-1].item()) < float(lh[0].item()), cam.width
+
+
+def test_mapping_loss_of_few_and_of_many_pixels_agree(torch_cuda):
+    """Calls of up to 199,999 pixels take strips of two rows with their inputs
+    loaded ahead, larger ones strips of four: a view's gradients are the same
+    bits alone, in a small batch and in a batch past the line, down to images
+    of one pixel, one strip and a ragged strip; losses up to the FP32 order of
+    their sums."""
+    torch = torch_cuda
+    from paper_2506_00970_gb300 import gs2d
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    u = lambda *s: torch.rand(*s, generator=g, device="cuda")
+    small = [(1, 1), (3, 3), (28, 2), (29, 3), (57, 5), (5, 61), (333, 251)]
+    views = []
+    for w, h in small + [(401, 498), (400, 500)]:   # the last two: either side of the line
+        op = torch.where(u(h, w) < 0.9, 0.6 + 0.4 * u(h, w), 0.4 * u(h, w))
+        x = torch.arange(w, device="cuda") / 9.0
+        y = torch.arange(h, device="cuda")[:, None] / 7.0
+        depth = (2.0 + 0.3 * torch.sin(x) + 0.2 * torch.cos(y) + 0.01 * u(h, w)) * op
+        nrm = torch.nn.functional.normalize(torch.randn(h, w, 3, generator=g, device="cuda"), dim=-1)
+        views.append((gs2d.Camera(0.8 * w, 0.8 * w, w / 2, h / 2, w, h, 0.05),
+                      [u(h, w, 3), depth, nrm, op, u(h, w, 3), 1.0 + 2.0 * u(h, w)]))
+
+    def outs(ins):
+        return [torch.full_like(a, 7.0) for a in ins[:4]]
+
+    def alone(cam, ins):
+        o, loss, ws = outs(ins), torch.empty(1, device="cuda"), torch.empty(1 << 16, dtype=torch.uint8, device="cuda")
+        gs2d.gs2d_mapping_loss(*ins, cam, 0.5, 0.02, *o, loss, ws)
+        return o, loss
+
+    def batch(vs):
+        os = [outs(ins) for _, ins in vs]
+        arr = gs2d.loss_views([(cam, *ins, *o) for (cam, ins), o in zip(vs, os)])
+        loss = torch.full((len(vs),), -1.0, device="cuda")
+        ws = torch.empty(gs2d.gs2d_mapping_loss_batch_workspace(arr), dtype=torch.uint8, device="cuda")
+        gs2d.gs2d_mapping_loss_batch(arr, 0.5, 0.02, loss, ws)
+        return list(zip(os, loss))
+
+    few = batch(views[:len(small)]) + [batch([v])[0] for v in views[len(small):]]
+    many = batch(views)
+    torch.cuda.synchronize()
+    for v, a, b in zip(views, few, many):
+        ref, loss = alone(*v)
+        for got in (a, b):
+            for x, y in zip(got[0], ref):
+                assert torch.equal(x, y), (v[0].width, v[0].height)
+            assert float(got[1]) == pytest.approx(float(loss), rel=1e-5) and float(loss) > 0.0
+    assert float(few[6][0][2].abs().max()) > 0
