@@ -42,13 +42,17 @@ __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
 // a - b (as a - 1 b: exact product, one rounding)
 __device__ __forceinline__ F2 sub2(F2 a, F2 b) { return fma2(b, dup2(-1.f), a); }
 
-// 1 / a, correctly rounded and for every a (no pair instruction divides).  An
-// approximation with a Newton step on pairs (68 us for the SSIM kernel at
-// 1200x680, against 70) is wrong where a or 1 / a is not normal, and a test for
-// that costs what the divisions do.
+// 1 / a.  kTame: a is positive and normal and so is its reciprocal; then the
+// hardware approximation and one Newton step y + y (1 - a y) on the pair,
+// within 1 ulp.  Otherwise two divisions: the step would make NaN of an infinite
+// a, and zero of a reciprocal below the normal range.
+template <bool kTame>
 __device__ __forceinline__ F2 recip2(F2 a) {
   const float2 s = split2(a);
-  return make2(1.f / s.x, 1.f / s.y);
+  if (!kTame) return make2(1.f / s.x, 1.f / s.y);
+  const F2 y = make2(__fdividef(1.f, s.x), __fdividef(1.f, s.y));
+  const F2 e = fma2(mul2(a, dup2(-1.f)), y, dup2(1.f));
+  return fma2(y, e, y);
 }
 
 }  // namespace gs2d

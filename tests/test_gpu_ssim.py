@@ -109,3 +109,29 @@ def test_ssim_of_equal_images_with_a_huge_pixel(torch_cuda, value):
     gs2d.gs2d_ssim_loss(x, x, h, w, 0.125, g_x, loss, ws)
     torch.cuda.synchronize()
     assert float(loss.item()) == 0.0 and not g_x.any()
+
+
+def test_ssim_divides_where_a_value_exceeds_four(torch_cuda):
+    """A tile with a value past 4 divides where the others take approximate
+    reciprocals within 1 unit in the last place: out of that pixel's reach (10
+    pixels) its gradients are the same up to six such units a term, whose sum
+    cancels a hundredfold at most: 1e-4 of the largest."""
+    torch = torch_cuda
+    from paper_2506_00970_gb300 import gs2d
+    h = w = 32
+    x, y = _images(5, h, w)
+    out = []
+    for corner in (x[0, 0], [5.0, 5.0, 5.0]):
+        x = x.copy()
+        x[0, 0] = corner
+        g_x, loss = torch.zeros(h, w, 3, device="cuda"), torch.zeros(1, device="cuda")
+        ws = torch.empty(gs2d.gs2d_ssim_workspace(h, w), dtype=torch.uint8, device="cuda")
+        gs2d.gs2d_ssim_loss(torch.tensor(x, device="cuda"), torch.tensor(y, device="cuda"), h, w, 0.125, g_x,
+                            loss, ws)
+        torch.cuda.synchronize()
+        out.append(to_np(g_x).astype(np.float64))
+    far = np.ones((h, w), bool)
+    far[:11, :11] = False
+    scale = np.abs(out[0][far]).max()
+    assert 0 < scale and np.abs(out[0] - out[1])[far].max() <= 1e-4 * scale
+    assert np.abs(out[0] - out[1])[~far].max() > 1e-4 * scale
