@@ -43,7 +43,6 @@
 // with one value per instruction, 72 us with pairs in 192 threads, 68 us
 // so.
 #include <cmath>
-#include <type_traits>
 
 #include "f32x2.cuh"
 #include "gs2d_common.cuh"
@@ -195,49 +194,61 @@ __global__ void __launch_bounds__(kSsimThreads, 3) ssim_kernel(const float* __re
       for (int k = 0; k < 5; ++k) v[k] = load2(sb + (k * kSsimA + q0 + i) * kSsimBP + 2 * p);
       filter_tap(w, v, i, acc);
     }
-    // (one branch for the four outputs: a division, or a branch around it, in
-    // each keeps them from overlapping; the full loss at 1200x680 101.8 us with
-    // approximations alone, 103.6 so and 102.4 with the one branch)
-    auto eval = [&](auto is_tame) {
-      constexpr bool kTame = decltype(is_tame)::value;
+    // the reciprocals of the four outputs' denominators, with one branch for all:
+    // a division, or a branch around it, in each output keeps the outputs from
+    // overlapping (whole SSIM pass at 1200x680: 66.5 us with approximations
+    // only, 2 us more so, 67.6 with the one branch)
+    F2 ib[kSsimM][2];
+#pragma unroll
+    for (int o = 0; o < kSsimM; ++o) {
+      const F2 mx = acc[0][o], my = sub2(mx, acc[1][o]);
+      ib[o][0] = fma2(mx, mx, fma2(my, my, dup2(kSsimC1)));
+      ib[o][1] = add2(add2(sub2(acc[2][o], mul2(mx, mx)), sub2(acc[3][o], mul2(my, my))),
+                      dup2(kSsimC2));
+    }
+    if (tame) {
 #pragma unroll
       for (int o = 0; o < kSsimM; ++o) {
-        const int q = q0 + o, px = tx0 - kSsimR + q, py = ty0 - kSsimR + 2 * p;
-        if (q >= kSsimB) break;
-        const F2 mx = acc[0][o], md = acc[1][o], my = sub2(mx, md);
-        const F2 one = dup2(1.f);
-        const F2 b1 = fma2(mx, mx, fma2(my, my, dup2(kSsimC1)));
-        const F2 b2 = add2(add2(sub2(acc[2][o], mul2(mx, mx)), sub2(acc[3][o], mul2(my, my))),
-                           dup2(kSsimC2));
-        const F2 vd = sub2(acc[4][o], mul2(md, md));
-        const F2 ib1 = recip2<kTame>(b1), ib2 = recip2<kTame>(b2);
-        const F2 p1 = mul2(mul2(md, md), ib1), q1 = mul2(vd, ib2);   // 1 - P, 1 - Q
-        const F2 P = sub2(one, p1), Q = sub2(one, q1);
-        const F2 dmx = mul2(mul2(dup2(2.f), add2(mx, my)),
-                            sub2(mul2(mul2(Q, p1), ib1), mul2(mul2(P, q1), ib2)));
-        const F2 dmd = fma2(mul2(mul2(Q, dup2(-2.f)), ib1), fma2(my, p1, md),
-                            mul2(mul2(mul2(P, dup2(2.f)), ib2), fma2(my, q1, md)));
-        const F2 u2 = dup2(up), Pi = mul2(mul2(u2, P), ib2);
-        const float2 g0 = split2(mul2(u2, add2(dmx, dmd))), g1 = split2(mul2(Pi, q1));
-        const float2 g2 = split2(Pi), l = split2(sub2(add2(p1, q1), mul2(p1, q1)));   // 1 - S
-        const bool in_x = px >= 0 && px < W;
-        const bool i0 = in_x && py >= 0 && py < H, i1 = in_x && py + 1 >= 0 && py + 1 < H;
-        if (q >= kSsimR && q < kSsimR + kSsimT) {
-          if (i0 && 2 * p >= kSsimR && 2 * p < kSsimR + kSsimT) loss += l.x;
-          if (i1 && 2 * p + 1 >= kSsimR && 2 * p + 1 < kSsimR + kSsimT) loss += l.y;
-        }
-        float* g = sa + q * kSsimBP + 2 * p;
-        *reinterpret_cast<float2*>(g) = make_float2(i0 ? g0.x : 0.f, i1 ? g0.y : 0.f);
-        *reinterpret_cast<float2*>(g + kSsimB * kSsimBP) =
-            make_float2(i0 ? g1.x : 0.f, i1 ? g1.y : 0.f);
-        *reinterpret_cast<float2*>(g + 2 * kSsimB * kSsimBP) =
-            make_float2(i0 ? -g2.x : 0.f, i1 ? -g2.y : 0.f);
+        ib[o][0] = recip2<true>(ib[o][0]);
+        ib[o][1] = recip2<true>(ib[o][1]);
       }
-    };
-    if (tame)
-      eval(std::true_type());
-    else
-      eval(std::false_type());
+    } else {
+#pragma unroll
+      for (int o = 0; o < kSsimM; ++o) {
+        ib[o][0] = recip2<false>(ib[o][0]);
+        ib[o][1] = recip2<false>(ib[o][1]);
+      }
+    }
+#pragma unroll
+    for (int o = 0; o < kSsimM; ++o) {
+      const int q = q0 + o, px = tx0 - kSsimR + q, py = ty0 - kSsimR + 2 * p;
+      if (q >= kSsimB) break;
+      const F2 mx = acc[0][o], md = acc[1][o], my = sub2(mx, md);
+      const F2 one = dup2(1.f);
+      const F2 vd = sub2(acc[4][o], mul2(md, md));
+      const F2 ib1 = ib[o][0], ib2 = ib[o][1];
+      const F2 p1 = mul2(mul2(md, md), ib1), q1 = mul2(vd, ib2);   // 1 - P, 1 - Q
+      const F2 P = sub2(one, p1), Q = sub2(one, q1);
+      const F2 dmx = mul2(mul2(dup2(2.f), add2(mx, my)),
+                          sub2(mul2(mul2(Q, p1), ib1), mul2(mul2(P, q1), ib2)));
+      const F2 dmd = fma2(mul2(mul2(Q, dup2(-2.f)), ib1), fma2(my, p1, md),
+                          mul2(mul2(mul2(P, dup2(2.f)), ib2), fma2(my, q1, md)));
+      const F2 u2 = dup2(up), Pi = mul2(mul2(u2, P), ib2);
+      const float2 g0 = split2(mul2(u2, add2(dmx, dmd))), g1 = split2(mul2(Pi, q1));
+      const float2 g2 = split2(Pi), l = split2(sub2(add2(p1, q1), mul2(p1, q1)));   // 1 - S
+      const bool in_x = px >= 0 && px < W;
+      const bool i0 = in_x && py >= 0 && py < H, i1 = in_x && py + 1 >= 0 && py + 1 < H;
+      if (q >= kSsimR && q < kSsimR + kSsimT) {
+        if (i0 && 2 * p >= kSsimR && 2 * p < kSsimR + kSsimT) loss += l.x;
+        if (i1 && 2 * p + 1 >= kSsimR && 2 * p + 1 < kSsimR + kSsimT) loss += l.y;
+      }
+      float* g = sa + q * kSsimBP + 2 * p;
+      *reinterpret_cast<float2*>(g) = make_float2(i0 ? g0.x : 0.f, i1 ? g0.y : 0.f);
+      *reinterpret_cast<float2*>(g + kSsimB * kSsimBP) =
+          make_float2(i0 ? g1.x : 0.f, i1 ? g1.y : 0.f);
+      *reinterpret_cast<float2*>(g + 2 * kSsimB * kSsimBP) =
+          make_float2(i0 ? -g2.x : 0.f, i1 ? -g2.y : 0.f);
+    }
   }
   if (g_x) {
     __syncthreads();
