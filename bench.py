@@ -752,11 +752,11 @@ def slab_render(K, W_, flush):
         "ms_per_step_direct": float(np.median(direct)),
         "mpix_per_s_direct": P / (np.median(direct) / 1e3) / 1e6,
         "phases_ms": {k: float(np.median(v)) for k, v in per.items()},
-        "launch": "one CUDA graph per step (project, bin_sort 5 kernels, render_fwd, loss, "
-                  "render_bwd 2 kernels); L2 flushed before each",
+        "launch": "one CUDA graph per step (project, bin_sort 5 kernels, render_fwd, loss 2 kernels, "
+                  "render_bwd 3 kernels); L2 flushed before each",
         "pairs": {"evaluated": int(E[0]), "inside_cutoff": int(E[1]), "blended": int(E[2]),
                   "replayed_evaluated": int(E[3]), "replayed_inside_cutoff": int(E[4])},
-        "roofline": {"kernel": "render_fwd_kernel + render_bwd_kernel<full> + surfel_grad_kernel",
+        "roofline": {"kernel": "render_fwd_quad_kernel + render_bwd_warp_kernel<1> + surfel_grad_kernel<8>",
                      "bound": "alu", "unit": "TFLOP/s", "peak": peak,
                      "fwd_achieved": w_f / tf / 1e12, "fwd_frac": w_f / tf / 1e12 / peak,
                      "bwd_achieved": w_b / tb / 1e12, "bwd_frac": w_b / tb / 1e12 / peak,

@@ -47,7 +47,8 @@ __host__ __device__ inline int bwd_regions(const gs2d_config& c, int R = kBwdReg
 //   480x360   690 tiles   119  107 [111] 190   ( 85   60  [55]  72)
 //   640x480  1200 tiles   169  127 [119] 170   (123   82  [65]  75)
 //   800x600  1900 tiles   232  168  149 [165]  (169  109   84  [78])
-// (before: 4 blocks below 304 tiles, else 8).  Taken with a warp per 32
+// (before: 4 blocks below 304 tiles, else 8).  At 800x600 the room prefers 4
+// blocks and the slab 8; the line is the slab's.  Taken with a warp per 32
 // surfels in the reduction that follows; with eight it is ~8 us less in the
 // 4,000-surfel figures at 1 block.
 inline int bwd_region_for(const gs2d_config& c, int n_tiles) {
